@@ -172,7 +172,10 @@ enum {
  * acc_out (nullable): int32 NCHW [B][O][Ho][Wo], the exact accumulator.
  * y_out (nullable): fp32 NCHW, y = fmaf((float)acc, scale[o], shift[o]);
  *   scale/shift (length O) are required when y_out is given.
- * variant: MINW_VARIANT_*.  At least one output must be non-null.
+ * variant: MINW_VARIANT_AUTO (the tensor cores, the planes expanded to level
+ * codes inside the kernel, for kh kw C < 2^20; else the popcount path) or
+ * MINW_VARIANT_POPC; both give the same bits.  At least one output must be
+ * non-null.
  * Errors: MINW_EINVAL (sizes, pointers, bits), MINW_EUNSUPPORTED (C % 32,
  * a variant that does not cover the shape). */
 MINW_API minw_status minw_conv2d(const uint32_t *act, int32_t B, int32_t C, int32_t H,

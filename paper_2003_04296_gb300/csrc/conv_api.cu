@@ -44,10 +44,13 @@ int choose_variant(const ConvArgs &a, int requested) {
     return conv_tc_supported(a) ? MINW_VARIANT_TC : MINW_VARIANT_POPC;
 }
 
-// Packed-plane operands run on the popcount path; the tensor-core path takes
-// its operands in the codes layout (minw_conv2d_codes / minw_conv_block_codes).
+// Packed-plane operands: the popcount path on request, else the tensor cores
+// with the planes expanded on the way (conv_planes_tc.cu) wherever that kernel
+// covers the shape.  The kernels on level codes (MINW_VARIANT_TC) take their
+// operands in the codes layout (minw_conv2d_codes / minw_conv_block_codes).
 minw_status run_conv(const ConvArgs &a, int variant, cudaStream_t s) {
     if (variant == MINW_VARIANT_TC) return MINW_EUNSUPPORTED;
+    if (variant != MINW_VARIANT_POPC && planes_tc_supported(a)) return launch_planes_tc(a, s);
     return launch_conv_popc(a, s);
 }
 

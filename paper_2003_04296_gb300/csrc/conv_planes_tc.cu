@@ -1,0 +1,515 @@
+// conv_planes_tc.cu -- the bit-plane convolution on the tensor cores: the
+// same operands and results as conv_popc.cu (exact int32 accumulators), with
+// the planes expanded to E2M1 level codes on the way into shared memory.
+//
+// The levels {0, +-1, +-2, +-4} are exact in E2M1 and their products and sums
+// exact in the fp32 accumulators (|acc| <= 16 K < 2^24, checked by the host),
+// so tcgen05.mma kind::mxf4 with unit block scales computes the integer
+// product of Table I.  A nibble is sign * 8 + magnitude code * 2, and the
+// planes hold exactly those bits: nibble j of register r takes channel bit
+// 4 j + r of its word, i.e. one shift and one masked OR per plane and eight
+// channels.  The channel order inside a word is permuted that way for both
+// operands alike, which leaves the contraction unchanged.
+//
+// Implicit GEMM: CTA tile = 128 consecutive output pixels (MMA M) x BN output
+// channels (MMA N), K = kh kw taps x C/32 words, flattened and taken in chunks
+// of four words (128 channels, 64-byte operand rows with the 64-byte swizzle).
+// Warp roles (288 threads): warps 0-3 expand activation rows, one pixel per
+// thread, warps 4-7 weight rows, one channel per thread; each thread keeps two
+// chunks of loads in flight in registers.  Warp 8 issues the MMAs.  After the
+// last chunk warps 0-7 run the epilogue from tensor memory: raw accumulators,
+// BN, HardTanh + quantize + pack, 2x2 max pool (through shared memory).
+// One tile per CTA, two or more CTAs per SM: one CTA's epilogue and set-up
+// overlap the other's main loop.
+//
+// Bound: the expansion's integer instructions (about 6 P per 8 channels and
+// operand row) and, for raw outputs, the int32 / fp32 stores.  The popcount
+// kernel spends 2 P_a P_w popcounts per 32 products at 16 a clock and SM; on a
+// 256 x 512 x 14 x 14, 3x3, 3-bit x 3-bit layer (quantize + convolve, raw and
+// fp32 outputs) it took 8.24 ms, this kernel 0.38 ms; a 4 x 128 x 32 x 32,
+// 1-bit x 1-bit layer 32.8 -> 20.5 us.
+//
+// Every mbarrier wait is bounded; one that runs out sets this file's error
+// flag (read by minw_get_last_device_error) and the CTA winds down.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "kernels.cuh"
+
+namespace minw {
+
+__device__ int g_planes_tc_error = 0;
+
+namespace ptc {
+
+constexpr int BM = 128;
+constexpr int NPROD = 256;               // producer / epilogue threads
+constexpr int NT = NPROD + 32;
+constexpr int ROWB = 64;                 // bytes of one operand row of a chunk: 128 E2M1 channels
+constexpr int CW = 4;                    // 32-channel words per chunk
+constexpr int SMAX = 6;
+constexpr int POOL_LD = BM + 1;          // padded channel row of the pooling stage
+
+struct Params {
+    ConvArgs a;
+    int BN;                // output channels per tile: 32, 64 or 128
+    int ntn;               // channel tiles
+    int nchunks;           // K chunks
+    int S;                 // ring slots
+    uint32_t stage_bytes;  // BM rows then BN rows of ROWB bytes
+    uint32_t idesc, tmem_cols;
+    long long wait_cycles;
+    int stall;             // timeout-path test: the MMA issuer first waits on a barrier nothing completes
+};
+
+__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void bar_init(uint64_t *b, uint32_t n) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(su32(b)), "r"(n));
+}
+__device__ __forceinline__ void bar_arrive(uint64_t *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(b)) : "memory");
+}
+__device__ __forceinline__ bool bar_try(uint64_t *b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 100000;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(su32(b)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait: false (and the error flag set) after limit SM clocks.
+__device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, long long limit) {
+    if (bar_try(b, parity)) return true;
+    const long long t0 = clock64();
+    while (!bar_try(b, parity)) {
+        if (clock64() - t0 > limit) {
+            atomicExch(&g_planes_tc_error, 1);
+            return false;
+        }
+    }
+    return true;
+}
+
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+
+// K-major operand rows of 64 bytes with the 64-byte swizzle (8-row groups 512 bytes apart).
+__device__ __forceinline__ uint64_t desc64(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)((8 * ROWB) >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
+// Executed by the whole (converged) issuing warp; one elected lane issues.
+__device__ __forceinline__ void mma_f4(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                       uint32_t accumulate, uint32_t sfa, uint32_t sfb) {
+    asm volatile("{\n .reg .pred p, e;\n .reg .b32 r;\n setp.ne.b32 p, %4, 0;\n elect.sync r|e, 0xffffffff;\n"
+                 " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%6], p;\n}\n"
+                 ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb));
+}
+__device__ __forceinline__ void mma_commit(uint64_t *bar) {
+    asm volatile("{\n .reg .pred e;\n .reg .b32 r;\n elect.sync r|e, 0xffffffff;\n"
+                 " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(su32(bar))
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+// E2M1 codes of the 32 channels of one word (P planes at pl[0], pl[CW], ...):
+// nibble j of word r is channel 4 j + r.  valid = 0 (1-bit only: a padded tap
+// or a word past the last) gives zeros; multi-level planes are then zero.
+template <int P>
+__device__ __forceinline__ uint4 expand(const uint32_t *pl, bool valid) {
+    const uint32_t s = pl[0];
+    uint32_t r0 = (s << 3) & 0x88888888u, r1 = (s << 2) & 0x88888888u, r2 = (s << 1) & 0x88888888u,
+             r3 = s & 0x88888888u;
+    if constexpr (P == 1) {
+        const uint32_t one = valid ? 0x22222222u : 0u;   // a zero magnitude with the sign set is -0
+        r0 |= one; r1 |= one; r2 |= one; r3 |= one;
+    } else {
+        const uint32_t m = pl[CW];                       // non-zero mask, or bit 0 of the magnitude code
+        r0 |= (m << 1) & 0x22222222u;
+        r1 |= m & 0x22222222u;
+        r2 |= (m >> 1) & 0x22222222u;
+        r3 |= (m >> 2) & 0x22222222u;
+        if constexpr (P == 3) {
+            const uint32_t c = pl[2 * CW];
+            r0 |= (c << 2) & 0x44444444u;
+            r1 |= (c << 1) & 0x44444444u;
+            r2 |= c & 0x44444444u;
+            r3 |= (c >> 1) & 0x44444444u;
+        }
+    }
+    return make_uint4(r0, r1, r2, r3);
+}
+
+// One chunk of an operand row in registers: word j of plane p at w[p * CW + j].
+template <int P>
+struct Chunk {
+    uint32_t w[P * CW];
+    uint32_t valid;        // bit j: word j lies in the image and before the last word of K
+};
+
+// Position of a row's next load in K: tap (ky, kx) and word w of its NW.
+struct Cursor {
+    int ky, kx, w;
+};
+
+// Loads the next chunk of a row.  ACT: an activation row (tap (ky, kx) reads
+// pixel (y0 + ky, x0 + kx) of image pix0 where it lies inside), else a weight
+// row (consecutive taps).  VEC: NW is a multiple of four, so a chunk lies in
+// one tap and each plane's four words are one 16-byte load; otherwise every
+// word is placed by itself.
+template <int P, bool ACT, bool VEC>
+__device__ __forceinline__ void load_chunk(Chunk<P> &ch, Cursor &k, const ConvArgs &a, bool live, int64_t row, int y0,
+                                           int x0) {
+    ch.valid = 0u;
+#pragma unroll
+    for (int i = 0; i < P * CW; ++i) ch.w[i] = 0u;
+    constexpr int STEP = VEC ? CW : 1;
+#pragma unroll
+    for (int j = 0; j < CW; j += STEP) {
+        const uint32_t *src;
+        bool in = live && k.ky < a.kh;
+        if constexpr (ACT) {
+            const int y = y0 + k.ky, x = x0 + k.kx;
+            in = in && y >= 0 && y < a.H && x >= 0 && x < a.W;
+            src = a.act + (row + (int64_t)y * a.W + x) * P * a.NW + k.w;
+        } else {
+            src = a.wgt + (row + k.ky * a.kw + k.kx) * P * a.NW + k.w;
+        }
+        if (in) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                if constexpr (VEC) {
+                    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + p * a.NW));
+                    ch.w[p * CW] = v.x; ch.w[p * CW + 1] = v.y; ch.w[p * CW + 2] = v.z; ch.w[p * CW + 3] = v.w;
+                } else {
+                    ch.w[p * CW + j] = __ldg(src + p * a.NW);
+                }
+            }
+            ch.valid |= (VEC ? 0xFu : 1u) << j;
+        }
+        k.w += STEP;
+        if (k.w >= a.NW) {
+            k.w = 0;
+            if (++k.kx == a.kw) { k.kx = 0; ++k.ky; }
+        }
+    }
+}
+
+// The producer loop of one thread: every chunk of its row, expanded into the
+// ring slot's 64-byte row (chunk j of four at j ^ ((row >> 1) & 3): the 64-byte
+// swizzle, and no bank conflict between eight neighbouring rows).
+template <int P, bool ACT, bool VEC>
+__device__ __forceinline__ bool produce(const Params &p, uint8_t *dst, int r, bool write, bool live, int64_t row,
+                                        int y0, int x0, uint64_t *full, uint64_t *empty) {
+    const ConvArgs &a = p.a;
+    Cursor k{0, 0, 0};
+    Chunk<P> c[2];
+    load_chunk<P, ACT, VEC>(c[0], k, a, live, row, y0, x0);
+    load_chunk<P, ACT, VEC>(c[1], k, a, live, row, y0, x0);
+    const uint32_t sw = (uint32_t)((r >> 1) & 3);
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    int s = 0, lap = 0;
+    for (int i = 0; i < p.nchunks; i += 2) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (i + h >= p.nchunks) break;
+            uint4 v[CW];
+#pragma unroll
+            for (int j = 0; j < CW; ++j) v[j] = expand<P>(c[h].w + j, (c[h].valid >> j) & 1u);
+            load_chunk<P, ACT, VEC>(c[h], k, a, live, row, y0, x0);
+            if (lap > 0 && !__all_sync(0xffffffffu, bar_wait(&empty[s], (lap - 1) & 1, p.wait_cycles))) return false;
+            if (write) {
+                uint4 *d = reinterpret_cast<uint4 *>(dst + (size_t)s * p.stage_bytes + r * ROWB);
+#pragma unroll
+                for (int j = 0; j < CW; ++j) d[j ^ sw] = v[j];
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane0) bar_arrive(&full[s]);
+            if (++s == p.S) { s = 0; ++lap; }
+        }
+    }
+    return true;
+}
+
+// Level planes of BN output y of one channel (bits 0 .. OUTB - 1), the fp32
+// chain of the block: HardTanh, prescale, thresholds.
+template <int OUTB>
+__device__ __forceinline__ uint32_t planes_of_y(float y, const QParams &q) {
+    QParams qb = q;
+    qb.bits = OUTB;
+    y = fminf(fmaxf(y, -1.0f), 1.0f);
+    return level_plane_bits(level_units(y * qb.scale, qb), OUTB);
+}
+
+// Epilogue of one 32-channel group without pooling: lane = output pixel m.
+template <int OUTB>
+__device__ __forceinline__ void store_group(const ConvArgs &a, const uint32_t (&v)[32], int o0, long long m) {
+    if (m >= a.M) return;
+    const int HoWo = a.Ho * a.Wo;
+    const long long b = m / HoWo;
+    const long long at = (b * a.O + o0) * HoWo + (m - b * HoWo);
+    const int nv = min(32, a.O - o0);
+    if (a.acc_out != nullptr) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+            if (c < nv) __stcs(a.acc_out + at + (long long)c * HoWo, __float2int_rn(__uint_as_float(v[c])));
+    }
+    if (a.y_out == nullptr && OUTB == 0) return;
+    uint32_t w[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        if (c >= nv) break;
+        const float y = fmaf(__uint_as_float(v[c]), __ldg(a.scale + o0 + c), __ldg(a.shift + o0 + c));
+        if constexpr (OUTB > 0) {
+            const uint32_t pb = planes_of_y<OUTB>(y, a.qo);
+#pragma unroll
+            for (int u = 0; u < OUTB; ++u) w[u] |= ((pb >> u) & 1u) << c;
+        }
+        if (a.y_out != nullptr)
+            __stcs(a.y_out + at + (long long)c * HoWo, OUTB > 0 ? fminf(fmaxf(y, -1.0f), 1.0f) : y);
+    }
+    if constexpr (OUTB > 0) {
+        const int NWo = (a.O + 31) >> 5;
+        uint32_t *dst = a.planes_out + m * OUTB * NWo + (o0 >> 5);
+#pragma unroll
+        for (int u = 0; u < OUTB; ++u) dst[u * NWo] = w[u];
+    }
+}
+
+// Epilogue of one 32-channel group with the 2x2 max pool: the group's
+// accumulators in shared memory [channel][pixel], lane = channel, warp q of
+// four takes pooled pixels q, q + 4, ... of the tile's 32.
+template <int OUTB>
+__device__ __forceinline__ void store_pooled(const ConvArgs &a, const float *acc, int o0, long long m0, int q,
+                                             int lane) {
+    const int o = o0 + lane, HoWo = a.Ho * a.Wo, half = a.Wo / 2, Wp = half, HpWp = (a.Ho / 2) * Wp;
+    const bool live = o < a.O;
+    const float sc = live ? __ldg(a.scale + o) : 0.0f, sh = live ? __ldg(a.shift + o) : 0.0f;
+    const int NWo = (a.O + 31) >> 5;
+    for (int t = q; t < BM / 4; t += 4) {
+        const int pr = t / half, r00 = 2 * pr * a.Wo + 2 * (t - pr * half);
+        const long long m = m0 + r00;
+        if (m >= a.M) break;
+        const long long b = m / HoWo;
+        const int pix = (int)(m - b * HoWo), yo = pix / a.Wo, xo = pix - yo * a.Wo;
+        const long long op = (long long)(yo / 2) * Wp + xo / 2;
+        const float *p = acc + lane * POOL_LD + r00;
+        const float v = fmaxf(fmaxf(p[0], p[1]), fmaxf(p[a.Wo], p[a.Wo + 1]));
+        const float y = fmaf(v, sc, sh);
+        if (a.y_out != nullptr && live)
+            a.y_out[(b * a.O + o) * HpWp + op] = OUTB > 0 ? fminf(fmaxf(y, -1.0f), 1.0f) : y;
+        if constexpr (OUTB > 0) {
+            const uint32_t pb = live ? planes_of_y<OUTB>(y, a.qo) : 0u;
+            uint32_t *dst = a.planes_out + ((b * HpWp + op) * OUTB) * NWo + (o0 >> 5);
+#pragma unroll
+            for (int u = 0; u < OUTB; ++u) {
+                const uint32_t w = __ballot_sync(0xffffffffu, (pb >> u) & 1u);
+                if (lane == u) dst[u * NWo] = w;
+            }
+        }
+    }
+}
+
+template <bool VEC, int OUTB>
+__global__ void __launch_bounds__(NT, 2) conv_planes_tc_kernel(const __grid_constant__ Params p) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (su32(smem_raw) & 1023u)) & 1023u);
+    __shared__ uint64_t full[SMAX], empty[SMAX], tfull, tstall;
+    __shared__ uint32_t tmem_slot;
+    const ConvArgs &a = p.a;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tn = (int)(blockIdx.x % (unsigned)p.ntn);
+    const long long m0 = (long long)(blockIdx.x / (unsigned)p.ntn) * BM;
+    const int o0 = tn * p.BN;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.S; ++s) {
+            bar_init(&full[s], NPROD / 32);
+            bar_init(&empty[s], 1);
+        }
+        bar_init(&tfull, 1);
+        bar_init(&tstall, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == NPROD / 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(su32(&tmem_slot)),
+                     "r"(p.tmem_cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = tmem_slot;
+    const uint32_t sf = tmem + (uint32_t)p.BN;            // unit scale factors: 32 columns of A's, 32 of B's
+    if (warp < 4) {
+        // UE8M0 0x7F = 2^0 in every lane of 64 columns, one warp per lane quarter
+#pragma unroll
+        for (int c = 0; c < 64; c += 8)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};\n" ::"r"(
+                             sf + ((uint32_t)(warp * 32) << 16) + (uint32_t)c),
+                         "r"(0x7F7F7F7Fu));
+        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    pdl_trigger();
+    pdl_wait();                                           // operands and outputs are shared with earlier kernels
+
+    if (warp == NPROD / 32) {
+        bool alive = true;
+        if (p.stall && !__all_sync(0xffffffffu, bar_wait(&tstall, 0u, p.wait_cycles))) alive = false;
+        const uint64_t ad0 = desc64(su32(smem)), bd0 = desc64(su32(smem) + BM * ROWB);
+        const uint32_t step = p.stage_bytes >> 4;
+        int s = 0;
+        uint32_t phase = 0u, acc = 0u;
+        for (int i = 0; alive && i < p.nchunks; ++i) {
+            if (!__all_sync(0xffffffffu, bar_wait(&full[s], phase, p.wait_cycles))) { alive = false; break; }
+            fence_after();
+            const uint64_t off = (uint64_t)((uint32_t)s * step);
+            mma_f4(tmem, ad0 + off, bd0 + off, p.idesc, acc, sf, sf + 32u);
+            mma_f4(tmem, ad0 + off + 2, bd0 + off + 2, p.idesc, 1u, sf, sf + 32u);
+            acc = 1u;
+            mma_commit(&empty[s]);
+            if (++s == p.S) { s = 0; phase ^= 1u; }
+        }
+        if (alive) mma_commit(&tfull);
+    } else {
+        const int r = threadIdx.x & (BM - 1);
+        if (warp < 4) {
+            const long long m = m0 + r;
+            const bool live = m < a.M;
+            const int HoWo = a.Ho * a.Wo;
+            const int b = live ? (int)(m / HoWo) : 0;
+            const int pix = live ? (int)(m - (long long)b * HoWo) : 0;
+            const int yo = pix / a.Wo, xo = pix - yo * a.Wo;
+            const int64_t row = (int64_t)b * a.H * a.W;
+            const int y0 = yo * a.stride - a.pad, x0 = xo * a.stride - a.pad;
+            if (a.bits_a == 1) produce<1, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
+            else if (a.bits_a == 2) produce<2, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
+            else produce<3, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
+        } else {
+            const int o = o0 + r;
+            const bool write = r < p.BN, live = write && o < a.O;
+            const int64_t row = (int64_t)o * a.kh * a.kw;
+            uint8_t *dst = smem + BM * ROWB;
+            if (a.bits_w == 1) produce<1, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
+            else if (a.bits_w == 2) produce<2, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
+            else produce<3, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
+        }
+        __syncwarp();
+        // a wait that ran out (here or in the MMA warp) leaves tfull open: no output is written
+        const bool ok = __all_sync(0xffffffffu, bar_wait(&tfull, 0u, p.wait_cycles));
+        fence_after();
+        const int q = warp & 3, h = warp >> 2;
+        if (!a.pool) {
+            for (int g = h; g < p.BN / 32 && ok; g += 2) {
+                if (o0 + g * 32 >= a.O) break;
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 32), v);
+                store_group<OUTB>(a, v, o0 + g * 32, m0 + q * 32 + lane);
+            }
+        } else {
+            // the ring is free: every MMA has completed.  Each half of the warps stages its groups in turn.
+            float *stage = reinterpret_cast<float *>(smem) + h * (32 * POOL_LD);
+            for (int g = h; g < p.BN / 32; g += 2) {
+                if (o0 + g * 32 >= a.O) break;
+                if (ok) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * 32), v);
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) stage[c * POOL_LD + q * 32 + lane] = __uint_as_float(v[c]);
+                }
+                asm volatile("bar.sync %0, 128;\n" ::"r"(1 + h) : "memory");
+                if (ok) store_pooled<OUTB>(a, stage, o0 + g * 32, m0, q, lane);
+                asm volatile("bar.sync %0, 128;\n" ::"r"(1 + h) : "memory");
+            }
+        }
+        fence_before();
+    }
+    __syncthreads();
+    if (warp == NPROD / 32) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(p.tmem_cols));
+    }
+}
+
+}  // namespace ptc
+
+// Accumulators of magnitude <= 16 kh kw C must stay below 2^24 (exact in fp32);
+// outputs are those of the bit-plane entry points (planes, fp32, raw).
+bool planes_tc_supported(const ConvArgs &a) {
+    if ((long long)a.kh * a.kw * a.C >= (1ll << 20) || a.codes_out != nullptr) return false;
+    if (a.pool && ptc::BM % (2 * a.Wo) != 0) return false;
+    return (a.M + ptc::BM - 1) / ptc::BM * ((a.O + 31) / 32) < (1ll << 31);
+}
+
+minw_status launch_planes_tc(const ConvArgs &a, cudaStream_t s) {
+    ptc::Params p{};
+    p.a = a;
+    const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 152;
+    const long long tiles_m = (a.M + ptc::BM - 1) / ptc::BM;
+    // channels per tile: as wide as O needs (activation rows are expanded once per
+    // channel tile), narrower while that leaves SMs without a tile
+    int BN = a.O > 64 ? 128 : a.O > 32 ? 64 : 32;
+    while (BN > 32 && tiles_m * ((a.O + BN - 1) / BN) < sms) BN /= 2;
+    p.BN = BN;
+    p.ntn = (a.O + BN - 1) / BN;
+    p.nchunks = (a.kh * a.kw * a.NW + ptc::CW - 1) / ptc::CW;
+    p.S = p.nchunks < ptc::SMAX ? p.nchunks : ptc::SMAX;
+    p.stage_bytes = (uint32_t)((ptc::BM + BN) * ptc::ROWB);
+    // D fp32, A and B E2M1 with UE8M0 scales (kind::mxf4)
+    p.idesc = (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | (1u << 23) | ((uint32_t)(ptc::BM >> 4) << 24);
+    p.tmem_cols = BN == 128 ? 256u : 128u;                // BN accumulator columns, 64 of scale factors
+    p.wait_cycles = (long long)minw_host::plan_options().wait_cycles;
+    p.stall = minw_host::take_stall(MINW_STALL_CONV_TC);
+    size_t smem = (size_t)p.S * p.stage_bytes;
+    const size_t pool = a.pool ? sizeof(float) * 2 * 32 * ptc::POOL_LD : 0;
+    if (smem < pool) smem = pool;
+    smem += 1024;
+    typedef void (*Kernel)(const ptc::Params);
+    static const Kernel kernels[2][4] = {
+        {ptc::conv_planes_tc_kernel<false, 0>, ptc::conv_planes_tc_kernel<false, 1>,
+         ptc::conv_planes_tc_kernel<false, 2>, ptc::conv_planes_tc_kernel<false, 3>},
+        {ptc::conv_planes_tc_kernel<true, 0>, ptc::conv_planes_tc_kernel<true, 1>,
+         ptc::conv_planes_tc_kernel<true, 2>, ptc::conv_planes_tc_kernel<true, 3>}};
+    const Kernel kern = kernels[a.NW % ptc::CW == 0][a.quant_out ? a.qo.bits : 0];
+    constexpr int SMEM_MAX = ptc::SMAX * (ptc::BM + 128) * ptc::ROWB + 1024;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess)
+        return MINW_ECUDA;
+    if (minw_host::launch_pdl(kern, dim3((unsigned)(tiles_m * p.ntn)), dim3(ptc::NT), smem, s, p) != cudaSuccess)
+        return MINW_ECUDA;
+    return cudaGetLastError() == cudaSuccess ? MINW_OK : MINW_ECUDA;
+}
+
+int take_planes_tc_error() {
+    int flag = 0;
+    if (cudaMemcpyFromSymbol(&flag, g_planes_tc_error, sizeof(int)) != cudaSuccess) return -1;
+    if (flag) {
+        const int zero = 0;
+        if (cudaMemcpyToSymbol(g_planes_tc_error, &zero, sizeof(int)) != cudaSuccess) return -1;
+    }
+    return flag ? 1 : 0;
+}
+
+}  // namespace minw

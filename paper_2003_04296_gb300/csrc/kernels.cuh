@@ -96,6 +96,11 @@ minw_status launch_first_weights(const float *w, int O, int K, int quant_w, cons
 minw_status launch_thresholds_f32(const float *scale, const float *shift, int O, const QParams &q, float *out,
                                   cudaStream_t s);
 minw_status launch_conv_popc(const ConvArgs &a, cudaStream_t s);
+// The bit-plane convolution on the tensor cores (conv_planes_tc.cu): whether it
+// covers the shape, its launch, and its timeout flag (as take_first_error).
+bool planes_tc_supported(const ConvArgs &a);
+minw_status launch_planes_tc(const ConvArgs &a, cudaStream_t s);
+int take_planes_tc_error();
 minw_status make_conv_args(ConvArgs &a, const uint32_t *act, int B, int C, int H, int W,
                            int bits_a, const uint32_t *wgt, int O, int kh, int kw, int bits_w,
                            int stride, int pad);
