@@ -1340,7 +1340,7 @@ def run_sweep(args, rank, world, local_rank):
     roofline["candidate_ms"] = {"order": ["e4m3", "e2m1", "e2m1 CTA pairs of 128-channel tiles"], **cand_ms}
     # the A2 step: fp32 NCHW in, level codes out (4 + 1/2 bytes per element for E2M1, 4 + 1 for E4M3)
     q_bytes = (4.5 if q_first[1] == "e2m1" else 5.0) * x.numel()
-    quant_roof = {"bound": "hbm", "kernel": f"quantize_codes_kernel<{q_first[1].upper()}> (1-bit)", "ms": round(q_ms, 5),
+    quant_roof = {"bound": "hbm", "kernel": f"quantize_kernel ({q_first[1].upper()} codes, 1-bit)", "ms": round(q_ms, 5),
                   "achieved": q_bytes / (q_ms * 1e-3) / 1e9, "peak": HBM_GBS, "unit": "GB/s",
                   "frac": q_bytes / (q_ms * 1e-3) / 1e9 / HBM_GBS, "algorithmic_bytes": q_bytes,
                   "peak_basis": "measured copy bandwidth, of measured"}

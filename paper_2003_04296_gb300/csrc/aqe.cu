@@ -166,128 +166,269 @@ __global__ void __launch_bounds__(256) aqe_backward_masked_kernel(const uint32_t
 }
 
 // ---------------------------------------------------------------------------
-// Quantize + pack of NCHW activations into [B][H][W][P][NW] planes, with the
-// AQE forward output and the |x| <= 1 mask of the backward produced from the
-// same load of x.
+// Quantize NCHW activations into a channel-contiguous layout: bit-planes
+// [B][H][W][P][NW] (with the AQE forward output and the |x| <= 1 mask of the
+// backward from the same load of x), E4M3 codes [B][H][W][C], or E2M1 codes
+// [B][H][W][C/2].
 //
-// One warp owns 32 channels x 128 pixels of one image: lane l holds pixels
-// p0 + 4l .. p0 + 4l + 3 and reads them with one 128-bit load per channel, so
-// every load instruction of the warp covers 512 contiguous bytes.  A lane
-// owns whole output words (32 channels of one pixel), so no transpose is
-// needed.  Requires HW % 4 == 0 (16-byte aligned channel rows).
+// HBM bound: 4 B read per element.  A block takes PX pixels x 4 G channels
+// of one image, one item of 4 channels x V pixels per thread: all of a
+// thread's loads are independent and issue first (four 16-byte loads with
+// V = 4, HW % 4 == 0; four 4-byte loads with V = 1), and a warp's loads cover
+// whole 128-byte runs of a channel row.  The four channels of a pixel leave
+// each thread as one 32-bit word (four E4M3 bytes, four E2M1 nibbles, or one
+// nibble per plane in bytes 0 .. P - 1), exchanged through shared memory so
+// that one thread assembles the 32 channels of a pixel.  Shared word of
+// channel group g of pixel V j + i: [i][j][g], rows of G + 4 words (16-byte
+// aligned, no conflict at G = 32, two-way below).  PX is 32 for 128 channels
+// and more, and grows to 128 as the channels shrink to 32 (V = 4), so that
+// the 256 threads stay busy.
+// A warp per 32 channels with its channels in a serial loop, as before, had
+// one load in flight and few warps on small tensors: 256 x 512 x 14 x 14,
+// 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (MEASURED_NOW).
 // ---------------------------------------------------------------------------
 
-template <int P>
-__global__ void __launch_bounds__(256) quantize_pack_vec_kernel(
-    const float *__restrict__ x, int B, int C, int HW, QParams q, uint32_t *__restrict__ planes,
-    float alpha, float oma, float *__restrict__ y, uint32_t *__restrict__ mask, int mask_atomic) {
+enum QuantOut { OUT_PLANES, OUT_E4M3, OUT_E2M1 };
+
+// A level's representation by selects alone (the thresholds descend, so each test that holds
+// overrides the ones before): nested conditionals compile to divergent branches here.
+template <int BITS, typename T>
+__device__ __forceinline__ T pick(float m, const QParams &q, T zero, T l1, T l2, T l4) {
+    if constexpr (BITS == 1) return l1;
+    T r = zero;
+    if constexpr (BITS == 2) {
+        r = (m <= q.thr0) ? r : l1;
+    } else {
+        r = (m <= q.thr2) ? r : l1;
+        r = (m <= q.thr1) ? r : l2;
+        r = (m <= q.thr0) ? r : l4;
+    }
+    return r;
+}
+
+// Plane bits of one value's level, bit of plane k at bit 8 k.
+template <int BITS>
+__device__ __forceinline__ uint32_t plane_bytes(float u, const QParams &q) {
+    const uint32_t neg = (u > 0.0f) ? 0u : 1u;
+    if constexpr (BITS == 1) return neg;
+    return pick<BITS, uint32_t>(fabsf(u), q, 0u, 0x100u | neg, 0x10000u | neg, 0x10100u | neg);
+}
+
+// The level's value (level_value with the bit width known: no integer conversion).
+template <int BITS>
+__device__ __forceinline__ float level_of(float u, const QParams &q) {
+    constexpr float one = BITS == 3 ? 0.25f : 1.0f;
+    const float s = (u > 0.0f) ? 1.0f : -1.0f;
+    return s * pick<BITS, float>(fabsf(u), q, 0.0f, one, 0.5f, 1.0f);
+}
+
+// E2M1 nibble or E4M3 byte of the level.
+template <int BITS, bool FP4>
+__device__ __forceinline__ uint32_t code_of(float u, const QParams &q) {
+    const uint32_t neg = (u > 0.0f) ? 0u : (FP4 ? 0x8u : 0x80u);
+    constexpr uint32_t c1 = FP4 ? 2u : 0x38u, c2 = FP4 ? 4u : 0x40u, c4 = FP4 ? 6u : 0x48u;
+    return pick<BITS, uint32_t>(fabsf(u), q, 0u, c1 | neg, c2 | neg, c4 | neg);
+}
+
+template <int BITS, int OUT, int V>
+__global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restrict__ x, int B, int C, int HW, QParams q,
+                                                          int lgl, int chunks, int cgs, int64_t total,
+                                                          uint32_t *__restrict__ planes, uint8_t *__restrict__ codes,
+                                                          float alpha, float oma, float *__restrict__ y,
+                                                          uint32_t *__restrict__ mask, int mask_atomic) {
+    __shared__ __align__(16) uint32_t sw[V * (256 + 4 * 32)];
+    pdl_trigger();
+    pdl_wait();
+    const int LN = 1 << lgl, G = 256 >> lgl, PX = V << lgl;      // lanes per pixel run, channel groups, pixels
+    const int RS = G + 4, IS = LN * RS;                           // shared strides of j and i
     const int NW = (C + 31) >> 5;
-    const int chunks = (HW + 127) >> 7;               // 128-pixel chunks per image
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t total = (int64_t)B * NW * chunks;
-    for (int64_t t = warp; t < total; t += nwarps) {
-        const int chunk = (int)(t % chunks);
-        const int cw = (int)((t / chunks) % NW);
-        const int b = (int)(t / ((int64_t)chunks * NW));
-        const int p = chunk * 128 + lane * 4;          // first pixel of this lane
-        const bool live = p < HW;                      // HW % 4 == 0: all 4 or none
-        uint32_t w[4][P];
+    const int j = threadIdx.x & (LN - 1), g = threadIdx.x >> lgl;
+
+    struct Item {
+        int64_t b;
+        int cg, p0;
+    };
+    auto item = [&](int64_t t) {
+        Item it;
+        if (total < (1ll << 31)) {                                // 32-bit divisions
+            const uint32_t u = (uint32_t)t, r = u / (uint32_t)cgs;
+            it.cg = (int)(u - r * (uint32_t)cgs);
+            const uint32_t bb = r / (uint32_t)chunks;
+            it.p0 = (int)(r - bb * (uint32_t)chunks) * PX;
+            it.b = bb;
+        } else {
+            const int64_t r = t / cgs;
+            it.cg = (int)(t - r * cgs);
+            it.b = r / chunks;
+            it.p0 = (int)(r - it.b * chunks) * PX;
+        }
+        return it;
+    };
+    float nx[4][V];                                               // the next item's values, in flight
+    auto load = [&](const Item &it) {
+        const int p = it.p0 + V * j, c = it.cg * 4 * G + 4 * g;
+        const float *src = x + (it.b * C + c) * HW + p;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int k = 0; k < P; ++k) w[i][k] = 0u;
-        const int cmax = min(32, C - cw * 32);
-        for (int c = 0; c < cmax; ++c) {
-            const int ch = cw * 32 + c;
-            const int64_t off = ((int64_t)b * C + ch) * HW + p;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (live) v = __ldcs(reinterpret_cast<const float4 *>(x + off));
-            const float vv[4] = {v.x, v.y, v.z, v.w};
-            uint32_t mbits = 0u;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int lv = level_units(vv[i] * q.scale, q);
-                const uint32_t pb = level_plane_bits(lv, P);
-#pragma unroll
-                for (int k = 0; k < P; ++k) w[i][k] |= ((pb >> k) & 1u) << c;
-                mbits |= (fabsf(vv[i]) <= 1.0f ? 1u : 0u) << i;
+        for (int k = 0; k < 4; ++k) {
+            const bool in = p < HW && c + k < C;                  // V = 4: all four pixels or none
+            if constexpr (V == 4) {
+                float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (in) f = __ldcs(reinterpret_cast<const float4 *>(src));
+                nx[k][0] = f.x; nx[k][1] = f.y; nx[k][2] = f.z; nx[k][3] = f.w;
+            } else {
+                nx[k][0] = in ? __ldcs(src) : 0.0f;
             }
-            if (y != nullptr && live) {
-                const float hs = (P == 3) ? 0.25f : 1.0f;
-                float4 r;
-                r.x = fmaf(alpha, hs * (float)level_units(v.x * q.scale, q), oma * v.x);
-                r.y = fmaf(alpha, hs * (float)level_units(v.y * q.scale, q), oma * v.y);
-                r.z = fmaf(alpha, hs * (float)level_units(v.z * q.scale, q), oma * v.z);
-                r.w = fmaf(alpha, hs * (float)level_units(v.w * q.scale, q), oma * v.w);
-                __stcs(reinterpret_cast<float4 *>(y + off), r);
+            src += HW;
+        }
+    };
+    int64_t t = blockIdx.x;
+    Item it = item(t);
+    load(it);
+    while (true) {
+        const int cg = it.cg, p0 = it.p0, p = p0 + V * j, c = cg * 4 * G + 4 * g;
+        const int64_t b = it.b;
+        const bool pin = p < HW;
+        const int64_t off = (b * C + c) * HW + p;
+        float v[4][V];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < V; ++i) v[k][i] = nx[k][i];
+        t += gridDim.x;
+        const bool more = t < total;
+        if (more) {
+            it = item(t);
+            load(it);
+        }
+        uint32_t w[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) w[i] = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const float u = v[k][i] * q.scale;
+                if constexpr (OUT == OUT_PLANES) w[i] |= plane_bytes<BITS>(u, q) << k;
+                else if constexpr (OUT == OUT_E2M1) w[i] |= code_of<BITS, true>(u, q) << (4 * k);
+                else w[i] |= code_of<BITS, false>(u, q) << (8 * k);
+            }
+        }
+        // this thread's channels of the tensor (planes: bits of channels past C stay zero)
+        const int nc = max(0, min(4, C - c)), nst = pin ? nc : 0;
+        if constexpr (OUT == OUT_PLANES) {
+            const uint32_t cm = ((1u << nc) - 1u) * 0x010101u;
+#pragma unroll
+            for (int i = 0; i < V; ++i) w[i] &= cm;
+        }
+#pragma unroll
+        for (int i = 0; i < V; ++i) sw[i * IS + j * RS + g] = w[i];
+        if constexpr (OUT == OUT_PLANES) {
+            if (y != nullptr) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float yv[V];
+#pragma unroll
+                    for (int i = 0; i < V; ++i)
+                        yv[i] = fmaf(alpha, level_of<BITS>(v[k][i] * q.scale, q), oma * v[k][i]);
+                    if (k < nst) {
+                        float *dst = y + off + (int64_t)k * HW;
+                        if constexpr (V == 4) __stcs(reinterpret_cast<float4 *>(dst), make_float4(yv[0], yv[1], yv[2], yv[3]));
+                        else __stcs(dst, yv[0]);
+                    }
+                }
             }
             if (mask != nullptr) {
-                if (!mask_atomic) {
-                    // HW % 32 == 0: 8 lanes cover one 32-bit mask word
-                    uint32_t mw = mbits << ((lane & 7) * 4);
-                    mw |= __shfl_xor_sync(0xffffffffu, mw, 1);
-                    mw |= __shfl_xor_sync(0xffffffffu, mw, 2);
-                    mw |= __shfl_xor_sync(0xffffffffu, mw, 4);
-                    if (live && (lane & 7) == 0) mask[off >> 5] = mw;
-                } else if (live && mbits) {
-                    atomicOr(mask + (off >> 5), mbits << (off & 31));
+                // 32 consecutive pixels of a channel row sit in 32 / V neighbouring lanes of one warp
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    uint32_t m = 0u;
+                    const bool in = k < nst;
+#pragma unroll
+                    for (int i = 0; i < V; ++i) m |= (fabsf(v[k][i]) <= 1.0f ? 1u : 0u) << i;
+                    m = in ? m : 0u;
+                    bool first;                                   // run's first lane
+                    if constexpr (V == 4) {
+                        m <<= (threadIdx.x & 7) * 4;
+                        m |= __shfl_xor_sync(0xffffffffu, m, 1);
+                        m |= __shfl_xor_sync(0xffffffffu, m, 2);
+                        m |= __shfl_xor_sync(0xffffffffu, m, 4);
+                        first = (threadIdx.x & 7) == 0;
+                    } else {
+                        m = __ballot_sync(0xffffffffu, m);
+                        first = (threadIdx.x & 31) == 0;
+                    }
+                    if (first && in) {                            // flat bit offset of the run's first pixel
+                        const int64_t at = off + (int64_t)k * HW;
+                        uint32_t *mw = mask + (at >> 5);
+                        const uint32_t sh = (uint32_t)at & 31u;
+                        const uint32_t hi = __funnelshift_l(m, 0u, sh);     // bits past the first word
+                        if (!mask_atomic) {
+                            *mw = m;
+                        } else {
+                            atomicOr(mw, m << sh);
+                            if (hi) atomicOr(mw + 1, hi);
+                        }
+                    }
                 }
             }
         }
-        if (live) {
+        __syncthreads();
+        // word wi (32 channels: shared words 8 wi .. + 7) of pixel px; neighbouring threads on neighbouring words
+        const int lgn = 5 - lgl, nwi = 1 << lgn;                  // 32-channel words per pixel
+        for (int e = threadIdx.x; e < PX * nwi; e += 256) {
+            const int wi = e & (nwi - 1), px = e >> lgn;
+            const int cw = (cg * G >> 3) + wi;
+            if (p0 + px >= HW || cw >= NW) continue;
+            const uint32_t *src = sw + (px & (V - 1)) * IS + (px / V) * RS + 8 * wi;
+            const uint4 a = *reinterpret_cast<const uint4 *>(src), d = *reinterpret_cast<const uint4 *>(src + 4);
+            const uint32_t s[8] = {a.x, a.y, a.z, a.w, d.x, d.y, d.z, d.w};
+            const int64_t pix = b * HW + p0 + px;
+            if constexpr (OUT == OUT_PLANES) {
+                // byte k of each word is plane k's nibble: fold pairs, then fours, then the eight
+                const uint32_t e0 = s[0] | (s[1] << 4), e1 = s[2] | (s[3] << 4), e2 = s[4] | (s[5] << 4),
+                               e3 = s[6] | (s[7] << 4);           // byte k: 8 channels of plane k
+                uint32_t *dst = planes + pix * (BITS * NW) + cw;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                uint32_t *dst = planes + ((int64_t)b * HW + p + i) * (P * NW) + cw;
-#pragma unroll
-                for (int k = 0; k < P; ++k) dst[k * NW] = w[i][k];
+                for (int k = 0; k < BITS; ++k) {
+                    const uint32_t lo = __byte_perm(e0, e1, k | ((4 + k) << 4)), hi = __byte_perm(e2, e3, k | ((4 + k) << 4));
+                    dst[k * NW] = __byte_perm(lo, hi, 0x5410);
+                }
+            } else if constexpr (OUT == OUT_E4M3) {
+                uint4 *dst = reinterpret_cast<uint4 *>(codes + pix * C + cw * 32);
+                dst[0] = a;
+                if (C - cw * 32 > 16) dst[1] = d;
+            } else {
+                uint4 *dst = reinterpret_cast<uint4 *>(codes + ((pix * C + cw * 32) >> 1));
+                *dst = make_uint4(s[0] | (s[1] << 16), s[2] | (s[3] << 16), s[4] | (s[5] << 16), s[6] | (s[7] << 16));
             }
         }
+        if (!more) break;
+        __syncthreads();
     }
 }
 
-// Scalar variant for HW % 4 != 0: lane l owns pixel p0 + l.
-template <int P>
-__global__ void __launch_bounds__(256) quantize_pack_scalar_kernel(
-    const float *__restrict__ x, int B, int C, int HW, QParams q, uint32_t *__restrict__ planes,
-    float alpha, float oma, float *__restrict__ y, uint32_t *__restrict__ mask) {
-    const int NW = (C + 31) >> 5;
-    const int chunks = (HW + 31) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t total = (int64_t)B * NW * chunks;
-    for (int64_t t = warp; t < total; t += nwarps) {
-        const int chunk = (int)(t % chunks);
-        const int cw = (int)((t / chunks) % NW);
-        const int b = (int)(t / ((int64_t)chunks * NW));
-        const int p = chunk * 32 + lane;
-        const bool live = p < HW;
-        uint32_t w[P];
-#pragma unroll
-        for (int k = 0; k < P; ++k) w[k] = 0u;
-        const int cmax = min(32, C - cw * 32);
-        for (int c = 0; c < cmax; ++c) {
-            const int64_t off = ((int64_t)b * C + cw * 32 + c) * HW + p;
-            if (!live) continue;
-            const float v = __ldcs(x + off);
-            const int lv = level_units(v * q.scale, q);
-            const uint32_t pb = level_plane_bits(lv, P);
-#pragma unroll
-            for (int k = 0; k < P; ++k) w[k] |= ((pb >> k) & 1u) << c;
-            if (y != nullptr) {
-                const float hs = (P == 3) ? 0.25f : 1.0f;
-                y[off] = fmaf(alpha, hs * (float)lv, oma * v);
-            }
-            if (mask != nullptr && fabsf(v) <= 1.0f) atomicOr(mask + (off >> 5), 1u << (off & 31));
-        }
-        if (live) {
-            uint32_t *dst = planes + ((int64_t)b * HW + p) * (P * NW) + cw;
-#pragma unroll
-            for (int k = 0; k < P; ++k) dst[k * NW] = w[k];
-        }
-    }
+template <int OUT>
+static minw_status launch_quantize(const float *x, int B, int C, int64_t HW, const QParams &q, uint32_t *planes,
+                                   uint8_t *codes, float alpha, float *y, uint32_t *mask, int mask_atomic,
+                                   cudaStream_t s) {
+    const bool vec = HW % 4 == 0 && minw_host::aligned16(x) && (!y || minw_host::aligned16(y));
+    // pixels per block: 32 (lanes 8 x 4 pixels) for more than 64 channels, 64 and 128 below; scalar: 32
+    const int lgl = !vec ? 5 : C > 64 ? 3 : C > 32 ? 4 : 5;
+    const int PX = (vec ? 4 : 1) << lgl, CG = 4 * (256 >> lgl);
+    const int chunks = (int)((HW + PX - 1) / PX), cgs = (C - 1) / CG + 1;
+    const int64_t total = (int64_t)B * chunks * cgs;
+    // persistent: four blocks per SM, each with its next item's loads in flight behind the current one
+    const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 152;
+    const dim3 grid((unsigned)(total < 4 * sms ? total : 4 * sms));
+    typedef void (*Kernel)(const float *, int, int, int, QParams, int, int, int, int64_t, uint32_t *, uint8_t *, float,
+                           float, float *, uint32_t *, int);
+    static const Kernel kernels[2][3] = {
+        {quantize_kernel<1, OUT, 1>, quantize_kernel<2, OUT, 1>, quantize_kernel<3, OUT, 1>},
+        {quantize_kernel<1, OUT, 4>, quantize_kernel<2, OUT, 4>, quantize_kernel<3, OUT, 4>}};
+    if (minw_host::launch_pdl(kernels[vec][q.bits - 1], grid, dim3(256), 0, s, x, B, C, (int)HW, q, lgl, chunks, cgs,
+                              total, planes, codes, alpha, 1.0f - alpha, y, mask, mask_atomic) != cudaSuccess)
+        return MINW_ECUDA;
+    return minw_host::launch_status();
 }
 
 // ---------------------------------------------------------------------------
@@ -320,55 +461,6 @@ __global__ void pack_weights_kernel(const float *__restrict__ w, int O, int C, i
         uint32_t *dst = planes + ((int64_t)o * kh * kw + tap) * (P * NW) + cw;
 #pragma unroll
         for (int k = 0; k < P; ++k) dst[k * NW] = wd[k];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Level codes: NCHW fp32 -> NHWC bytes (E4M3 levels), the tensor-core operand.
-// One warp owns 32 pixels x 32 channels of an image: lane l reads pixel p0+l of
-// each channel (coalesced along the row) and writes its 32 channel bytes with
-// two 16-byte stores.  C % 16 == 0.  With FP4 the codes are E2M1 nibbles, two
-// channels per byte (16 bytes per lane; C % 32 == 0).
-// ---------------------------------------------------------------------------
-
-template <bool FP4>
-__global__ void __launch_bounds__(256) quantize_codes_kernel(const float *__restrict__ x, int B, int C,
-                                                             int HW, QParams q, uint8_t *__restrict__ codes) {
-    const int groups = (C + 31) >> 5;
-    const int chunks = (HW + 31) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t total = (int64_t)B * groups * chunks;
-    for (int64_t t = warp; t < total; t += nwarps) {
-        const int chunk = (int)(t % chunks);
-        const int g = (int)((t / chunks) % groups);
-        const int b = (int)(t / ((int64_t)chunks * groups));
-        const int p = chunk * 32 + lane;
-        if (p >= HW) continue;
-        const int c0 = g * 32;
-        const int cmax = min(32, C - c0);
-        uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-#pragma unroll 8
-        for (int c = 0; c < cmax; ++c) {
-            const float v = __ldcs(x + ((int64_t)b * C + c0 + c) * HW + p);
-            const int u = level_units(v * q.scale, q);
-            if (FP4)
-                w[c >> 3] |= level_code_e2m1(u) << ((c & 7) * 4);
-            else
-                w[c >> 2] |= (uint32_t)level_code_e4m3(u) << ((c & 3) * 8);
-        }
-        if (FP4) {
-            uint8_t *dst = codes + ((((int64_t)b * HW + p) * C + c0) >> 1);
-            if (cmax > 16)
-                *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-            else
-                *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
-        } else {
-            uint4 *dst = reinterpret_cast<uint4 *>(codes + ((int64_t)b * HW + p) * C + c0);
-            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            if (cmax > 16) dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        }
     }
 }
 
@@ -576,31 +668,14 @@ minw_status aqe_quantize_pack(const float *x, int32_t B, int32_t C, int32_t H, i
     const QParams qp = to_qparams(q);
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t n = (int64_t)B * C * HW;
-    const bool vec = (HW % 4 == 0) && aligned16(x) && (!y || aligned16(y));
-    const bool mask_atomic = mask && !(vec && HW % 32 == 0);
+    // a 32-pixel run of a channel row fills whole mask words when HW % 32 == 0; else its bits are merged into
+    // the two words it may straddle
+    const bool mask_atomic = mask && HW % 32 != 0;
     if (mask_atomic) {
         if (cudaMemsetAsync(mask, 0, sizeof(uint32_t) * ((n + 31) / 32), s) != cudaSuccess)
             return MINW_ECUDA;
     }
-    const int NW = (C + 31) / 32;
-    if (vec) {
-        const int64_t warps = (int64_t)B * NW * ((HW + 127) / 128);
-        const int64_t g = grid_for(warps * 32, 256);
-        switch (q->bits) {
-            case 1: quantize_pack_vec_kernel<1><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask, mask_atomic); break;
-            case 2: quantize_pack_vec_kernel<2><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask, mask_atomic); break;
-            default: quantize_pack_vec_kernel<3><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask, mask_atomic); break;
-        }
-    } else {
-        const int64_t warps = (int64_t)B * NW * ((HW + 31) / 32);
-        const int64_t g = grid_for(warps * 32, 256);
-        switch (q->bits) {
-            case 1: quantize_pack_scalar_kernel<1><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask); break;
-            case 2: quantize_pack_scalar_kernel<2><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask); break;
-            default: quantize_pack_scalar_kernel<3><<<(unsigned)g, 256, 0, s>>>(x, B, C, (int)HW, qp, planes, alpha, 1.0f - alpha, y, mask); break;
-        }
-    }
-    return launch_status();
+    return launch_quantize<OUT_PLANES>(x, B, C, HW, qp, planes, nullptr, alpha, y, mask, mask_atomic, s);
 }
 
 minw_status minw_pack_weights(const float *w, int32_t O, int32_t C, int32_t kh, int32_t kw,
@@ -626,10 +701,8 @@ minw_status aqe_quantize_codes(const float *x, int32_t B, int32_t C, int32_t H, 
     if (C % 16 != 0 || !aligned16(codes)) return MINW_EUNSUPPORTED;
     const int64_t HW = (int64_t)H * W;
     if (HW > (1ll << 30)) return MINW_EUNSUPPORTED;
-    const int64_t warps = (int64_t)B * ((C + 31) / 32) * ((HW + 31) / 32);
-    const int64_t g = grid_for(warps * 32, 256);
-    quantize_codes_kernel<false><<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, B, C, (int)HW, to_qparams(q), codes);
-    return launch_status();
+    return launch_quantize<OUT_E4M3>(x, B, C, HW, to_qparams(q), nullptr, codes, 0.0f, nullptr, nullptr, 0,
+                                     (cudaStream_t)stream);
 }
 
 minw_status aqe_quantize_codes_e2m1(const float *x, int32_t B, int32_t C, int32_t H, int32_t W,
@@ -638,10 +711,8 @@ minw_status aqe_quantize_codes_e2m1(const float *x, int32_t B, int32_t C, int32_
     if (C % 32 != 0 || !aligned16(codes)) return MINW_EUNSUPPORTED;
     const int64_t HW = (int64_t)H * W;
     if (HW > (1ll << 30)) return MINW_EUNSUPPORTED;
-    const int64_t warps = (int64_t)B * ((C + 31) / 32) * ((HW + 31) / 32);
-    const int64_t g = grid_for(warps * 32, 256);
-    quantize_codes_kernel<true><<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, B, C, (int)HW, to_qparams(q), codes);
-    return launch_status();
+    return launch_quantize<OUT_E2M1>(x, B, C, HW, to_qparams(q), nullptr, codes, 0.0f, nullptr, nullptr, 0,
+                                     (cudaStream_t)stream);
 }
 
 minw_status minw_pack_weight_codes(const float *w, int32_t O, int32_t C, int32_t kh, int32_t kw,
