@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "net.cuh"
+#include "wres_fused.cuh"
 
 using namespace minw;
 using namespace minw_host;
@@ -207,6 +208,8 @@ struct WResPlan {
     std::vector<float *> keep;             // with keep_activations: the stem's and every block's fp32 output
     std::vector<size_t> keep_elems;        // ... their sizes at max_batch
     int keep_B = 0;                        // batch of the most recent forward
+    uint8_t *blob = nullptr;               // one-kernel forward: every convolution's item (null: not used)
+    float **keep_dev = nullptr;            // ... and the kept activations' pointers on the device
 };
 
 template <typename T>
@@ -290,12 +293,28 @@ void wresnet_variants(const minw_net *net, int32_t *v) {
     while (k < n) v[k++] = 0;
 }
 
+// Images of up to 32 x 32 take the one-kernel forward (wres_fused.cu): 1.855
+// -> 0.260 ms for ResNet-110 at batch 128.  Larger images, whose activations do not fit a CTA's
+// shared memory, and forwards with per-op timing run layer by layer.
+static bool wresnet_fused(const minw_net *net) { return net->wres->blob != nullptr && !net->timing; }
+
 int32_t wresnet_kernels(const minw_net *net) {
-    return wresnet_ops(net) + 1;                       // the head is two kernels
+    return wresnet_fused(net) ? 1 : wresnet_ops(net) + 1;                 // the head is two kernels
 }
 
 minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits, cudaStream_t s) {
     WResPlan *R = net->wres;
+    if (wresnet_fused(net)) {
+        wfu::Args a{};
+        a.x = x; a.hw = R->hw; a.n = R->n; a.classes = R->classes;
+        a.stem_wt = R->stem_wt; a.stem_scale = R->stem_scale; a.stem_shift = R->stem_shift;
+        a.blob = R->blob;
+        a.fc_wt = R->fc_wt; a.fc_scale = R->fc_scale; a.fc_shift = R->fc_shift;
+        a.logits = logits;
+        a.keep = R->keep_dev;
+        R->keep_B = B;
+        return launch_wres_fused(a, B, s);
+    }
     int ev = 0;
     auto mark = [&]() -> minw_status {
         ++ev;
@@ -465,6 +484,33 @@ extern "C" minw_status minw_wresnet_create(const minw_wresnet_desc *d, int32_t m
             float *q = nullptr;
             if ((st = walloc(n, &q, k)) != MINW_OK) return fail(st);
             R->keep.push_back(q);
+        }
+    }
+    if (wres_fused_supported(d->image_hw)) {
+        size_t bytes = 0;
+        auto each = [&](auto &&f) -> minw_status {
+            for (const WBlock &bk : R->blocks) {
+                minw_status e = f(bk.c1);
+                if (e == MINW_OK && bk.down) e = f(bk.d);
+                if (e == MINW_OK) e = f(bk.c2);
+                if (e != MINW_OK) return e;
+            }
+            return MINW_OK;
+        };
+        each([&](const WConv &c) { bytes += wres_item_bytes(c.C, c.O, c.k * c.k); return MINW_OK; });
+        if ((st = walloc(n, &R->blob, bytes)) != MINW_OK) return fail(st);
+        size_t off = 0;
+        st = each([&](const WConv &c) {
+            uint8_t *dst = R->blob + off;
+            off += wres_item_bytes(c.C, c.O, c.k * c.k);
+            return wres_write_item(c.wb, c.scale, c.shift, c.C, c.Cp, c.O, c.k * c.k, dst, s);
+        });
+        if (st != MINW_OK) return fail(st);
+        if (!R->keep.empty()) {
+            if ((st = walloc(n, &R->keep_dev, R->keep.size())) != MINW_OK) return fail(st);
+            if (cudaMemcpyAsync(R->keep_dev, R->keep.data(), R->keep.size() * sizeof(float *), cudaMemcpyHostToDevice,
+                                s) != cudaSuccess)
+                return fail(MINW_ECUDA);
         }
     }
     n->x_elems = px * 3;
