@@ -38,6 +38,7 @@
 #include <mutex>
 
 #include "kernels.cuh"
+#include "wdense_fused.cuh"
 #include "wres_fused.cuh"
 
 namespace minw {
@@ -2232,8 +2233,9 @@ extern "C" minw_status minw_get_last_device_error(void *stream) {
     const int first_tc = minw::take_first_tc_error();
     const int planes_tc = minw::take_planes_tc_error();
     const int wres = minw::take_wres_error();
-    if (first < 0 || first_tc < 0 || planes_tc < 0 || wres < 0) return MINW_ECUDA;
-    return (flag || first || first_tc || planes_tc || wres) ? MINW_ETIMEOUT : MINW_OK;
+    const int wdense = minw::take_wdense_error();
+    if (first < 0 || first_tc < 0 || planes_tc < 0 || wres < 0 || wdense < 0) return MINW_ECUDA;
+    return (flag || first || first_tc || planes_tc || wres || wdense) ? MINW_ETIMEOUT : MINW_OK;
 }
 
 minw_host::EncodeTiledFn minw_host::tensor_map_encoder() {

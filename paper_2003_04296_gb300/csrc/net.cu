@@ -507,6 +507,8 @@ minw_status minw_forward(minw_net *net, const float *x, int32_t B, float *logits
         net->glogits = logits;
         net->gB = B;
     }
+    if (net->kind == 2) wresnet_note(net, B);
+    if (net->kind == 3) wdense_note(net, B);
     return cudaGraphLaunch(net->gexec, s) == cudaSuccess ? MINW_OK : MINW_ECUDA;
 }
 

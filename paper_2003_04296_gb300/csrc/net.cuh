@@ -74,6 +74,8 @@ void resnet_free(minw_net *net);
 
 // The weight-only residual network (wonly_nets.cu).
 minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits, cudaStream_t s);
+// What the introspection entry points need to know of the most recent forward (a graph replay too).
+void wresnet_note(minw_net *net, int B);
 int32_t wresnet_ops(const minw_net *net);
 void wresnet_variants(const minw_net *net, int32_t *variants);
 int32_t wresnet_kernels(const minw_net *net);
@@ -81,6 +83,7 @@ void wresnet_free(minw_net *net);
 
 // The weight-only DenseNet-BC (wonly_nets.cu).
 minw_status wdense_forward(minw_net *net, const float *x, int B, float *logits, cudaStream_t s);
+void wdense_note(minw_net *net, int B);
 int32_t wdense_ops(const minw_net *net);
 void wdense_variants(const minw_net *net, int32_t *variants);
 int32_t wdense_kernels(const minw_net *net);

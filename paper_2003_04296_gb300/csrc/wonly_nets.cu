@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "net.cuh"
+#include "wdense_fused.cuh"
 #include "wres_fused.cuh"
 
 using namespace minw;
@@ -302,6 +303,8 @@ int32_t wresnet_kernels(const minw_net *net) {
     return wresnet_fused(net) ? 1 : wresnet_ops(net) + 1;                 // the head is two kernels
 }
 
+void wresnet_note(minw_net *net, int B) { net->wres->keep_B = B; }
+
 minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits, cudaStream_t s) {
     WResPlan *R = net->wres;
     if (wresnet_fused(net)) {
@@ -312,7 +315,7 @@ minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits,
         a.fc_wt = R->fc_wt; a.fc_scale = R->fc_scale; a.fc_shift = R->fc_shift;
         a.logits = logits;
         a.keep = R->keep_dev;
-        R->keep_B = B;
+        wresnet_note(net, B);
         return launch_wres_fused(a, B, s);
     }
     int ev = 0;
@@ -364,7 +367,7 @@ minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits,
         acur = anext;
         xin = xout;
     }
-    R->keep_B = B;
+    wresnet_note(net, B);
     {
         const WConv &last = R->blocks.back().c2;
         const int HW = last.Ho * last.Wo, C = last.O;
@@ -563,6 +566,10 @@ struct WDensePlan {
     float *Y = nullptr;                  // fp32 NCHW convolution outputs
     float *fc_wt = nullptr, *fc_scale = nullptr, *fc_shift = nullptr, *pooled = nullptr;
     int last_B = 0;                      // batch of the most recent forward
+    uint8_t *blob = nullptr;             // one-kernel forward: every convolution's item (null: not used)
+    uint16_t *FP[3] = {nullptr, nullptr, nullptr};   // ... and its block features, planes of eight channels
+    int planes[3] = {0, 0, 0};
+    bool last_fused = false;             // the most recent forward wrote FP, not F
 };
 
 void wdense_free(minw_net *net) {
@@ -597,12 +604,38 @@ void wdense_variants(const minw_net *net, int32_t *v) {
     v[k++] = 0;
 }
 
+// The sizes wdense_fused.cu covers take its one-kernel forward: 1.473 -> MEASURED
+// ms for DenseNet-100 at batch 128.  Other sizes and forwards with per-op
+// timing run layer by layer.
+static bool wdense_fused(const minw_net *net) { return net->wdense->blob != nullptr && !net->timing; }
+
 int32_t wdense_kernels(const minw_net *net) {
-    return wdense_ops(net) + 1;                        // the head is two kernels
+    return wdense_fused(net) ? 1 : wdense_ops(net) + 1;                  // the head is two kernels
+}
+
+void wdense_note(minw_net *net, int B) {
+    net->wdense->last_B = B;
+    net->wdense->last_fused = wdense_fused(net);
 }
 
 minw_status wdense_forward(minw_net *net, const float *x, int B, float *logits, cudaStream_t s) {
     WDensePlan *D = net->wdense;
+    wdense_note(net, B);
+    if (wdense_fused(net)) {
+        dfu::Args a{};
+        a.x = x; a.hw = D->hw; a.layers = D->layers; a.k = D->growth; a.classes = D->classes;
+        a.stem_wt = D->stem_wt; a.stem_scale = D->stem_scale; a.stem_shift = D->stem_shift;
+        a.blob = D->blob;
+        for (int b = 0; b < 3; ++b) {
+            a.F[b] = D->FP[b];
+            a.cstart[b] = D->lay[b][0].cin;
+            a.cfin[b] = D->cfin[b];
+            a.planes[b] = D->planes[b];
+        }
+        a.fc_wt = D->fc_wt; a.fc_scale = D->fc_scale; a.fc_shift = D->fc_shift;
+        a.logits = logits;
+        return launch_wdense_fused(a, B, s);
+    }
     int ev = 0;
     auto mark = [&]() -> minw_status {
         ++ev;
@@ -647,7 +680,6 @@ minw_status wdense_forward(minw_net *net, const float *x, int B, float *logits, 
             if ((st = mark()) != MINW_OK) return st;
         }
     }
-    D->last_B = B;
     {
         const int h = D->hw >> 2, C = D->cfin[2];
         wdense_avgpool_kernel<<<(unsigned)((B * C + 255) / 256), 256, 0, s>>>(D->F[2], B, C, h * h, D->row[2],
@@ -760,6 +792,33 @@ extern "C" minw_status minw_wdense_create(const minw_wdense_desc *d, int32_t max
         if (b < 3) D->F[b] = q; else D->HB = q;
     }
     if ((st = walloc(n, &D->Y, (size_t)max_batch * y_px)) != MINW_OK) return fail(st);
+    if (wdense_fused_supported(hw, d->layers, k)) {
+        for (int b = 0; b < 3; ++b) {
+            D->planes[b] = wdense_planes(cfin[b]);
+            const size_t e = (size_t)max_batch * D->planes[b] * (hw >> b) * (hw >> b) * 8;
+            if ((st = walloc(n, &D->FP[b], e)) != MINW_OK) return fail(st);
+            if (cudaMemsetAsync(D->FP[b], 0, e * sizeof(uint16_t), s) != cudaSuccess) return fail(MINW_ECUDA);
+        }
+        auto each = [&](auto &&f) -> minw_status {
+            minw_status e = MINW_OK;
+            for (int b = 0; b < 3; ++b) {
+                for (const WDenseLayer &L : D->lay[b])
+                    if ((e = f(L.b)) != MINW_OK || (e = f(L.c)) != MINW_OK) return e;
+                if (b < 2 && (e = f(D->trans[b])) != MINW_OK) return e;
+            }
+            return e;
+        };
+        size_t bytes = 0;
+        each([&](const WConv &c) { bytes += wdense_item_bytes(c.C, c.O, c.k * c.k); return MINW_OK; });
+        if ((st = walloc(n, &D->blob, bytes)) != MINW_OK) return fail(st);
+        size_t off = 0;
+        st = each([&](const WConv &c) {
+            uint8_t *dst = D->blob + off;
+            off += wdense_item_bytes(c.C, c.O, c.k * c.k);
+            return wdense_write_item(c.wb, c.scale, c.shift, c.C, c.Cp, c.O, c.k * c.k, dst, s);
+        });
+        if (st != MINW_OK) return fail(st);
+    }
     n->x_elems = (size_t)max_batch * 3 * hw * hw;
     n->logit_elems = (size_t)max_batch * d->num_classes;
     if ((st = walloc(n, &n->x_stage, n->x_elems)) != MINW_OK ||
@@ -780,6 +839,9 @@ extern "C" minw_status minw_wdense_features(const minw_net *net, int32_t block, 
     if (count < elems) return MINW_EINVAL;
     if (channels) *channels = D->cfin[block];
     if (row) *row = D->row[block];
+    if (D->last_fused)
+        return wdense_planes_to_nhwc(D->FP[block], D->last_B, h * h, D->planes[block], D->cfin[block], D->row[block],
+                                     dst, (cudaStream_t)stream);
     return cudaMemcpyAsync(dst, D->F[block], elems * sizeof(uint16_t), cudaMemcpyDeviceToDevice,
                            (cudaStream_t)stream) == cudaSuccess ? MINW_OK : MINW_ECUDA;
 }

@@ -9,14 +9,8 @@
 // a convolution reads its input in place and the next one starts as soon as
 // the last epilogue warp is done.
 //
-// Shared-memory activations: planes of eight channels, [C / 8][(S + 2)(S + 1)
-// + 1 pixels][8] bf16, image pixel (y, x) at (y + 1)(S + 1) + x + 1: one zero
-// column serves as the right border of one row and the left border of the
-// next, and rows -1 and S are zero.  Without swizzle a matrix descriptor may
-// start at any pixel (16 bytes), so the tap (dy, dx) of a 3x3 convolution is
-// the same tile with a shifted start address: no im2col.  An MMA tile is 16
-// image rows x 8 columns (M = 128: 8-pixel groups, one image row apart), K =
-// 16 channels (two planes), N = the output channels.  The convolution entering
+// The activations sit in the padded plane layout of smem_conv.cuh, in which a
+// 3x3 convolution's tap is a shifted start address.  The convolution entering
 // a stage has stride 2: the last block of the stage before it writes its
 // output split by row and column parity, where stride 2 is again contiguous.
 //
@@ -40,110 +34,21 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "smem_conv.cuh"
 #include "wres_fused.cuh"
 
 namespace minw {
 
-__device__ int g_wres_error = 0;
-
 namespace wfu {
 
-constexpr int EPI = 256, NT = EPI + 64;
+using namespace smc;
+
+constexpr int NT = EPI + 64;
 constexpr int R0_BYTES = 40960, R1_BYTES = 36864;            // activation regions (32 x 32 images and smaller)
 constexpr int WBUF_BYTES = 9 * 64 * 64 * 2 + 64 * 8;         // the largest convolution with its BN map
 constexpr int SMEM_BYTES = R0_BYTES + R1_BYTES + 2 * WBUF_BYTES + 128;
 constexpr int MAX_TILES = 8;
 constexpr uint32_t D_COL = 256;                              // TMEM column of the shortcut convolution
-
-__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(uint64_t *b, uint32_t n) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(su32(b)), "r"(n));
-}
-__device__ __forceinline__ void bar_arrive(uint64_t *b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(b)) : "memory");
-}
-__device__ __forceinline__ bool bar_try(uint64_t *b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 100000;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(su32(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait of a whole warp: sets dead (warp-uniform) and the error flag
-// after limit SM clocks; returns at once when dead is set.
-__device__ __forceinline__ void warp_wait(uint64_t *b, uint32_t parity, long long limit, bool &dead) {
-    if (dead) return;
-    bool ok = bar_try(b, parity);
-    if (!ok) {
-        const long long t0 = clock64();
-        while (!(ok = bar_try(b, parity)) && clock64() - t0 <= limit) {
-        }
-    }
-    if (!__all_sync(0xffffffffu, ok)) {
-        atomicExch(&g_wres_error, 1);
-        dead = true;
-    }
-}
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(EPI) : "memory"); }
-
-// K-major operand without swizzle: 8-row groups sbo bytes apart (16 bytes per row), K steps of 16 bytes lbo apart.
-__device__ __forceinline__ uint64_t desc_ns(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
-           ((uint64_t)1 << 46);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n .reg .pred p, e;\n .reg .b32 r;\n setp.ne.b32 p, %4, 0;\n elect.sync r|e, 0xffffffff;\n"
-                 " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                 "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-__device__ __forceinline__ void mma_commit(uint64_t *bar) {
-    asm volatile("{\n .reg .pred e;\n .reg .b32 r;\n elect.sync r|e, 0xffffffff;\n"
-                 " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(su32(bar))
-                 : "memory");
-}
-
-template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t ta, float (&o)[N]) {
-    uint32_t v[N];
-    if constexpr (N == 8)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                     : "r"(ta));
-    else if constexpr (N == 16)
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15}, [%16];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(ta));
-    else
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-              "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(ta));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < N; ++i) o[i] = __uint_as_float(v[i]);
-}
-
-// One image of S x S pixels in the padded plane layout.
-struct Geo {
-    int S, Wp;
-    uint32_t plane;        // bytes of one plane of eight channels
-    __device__ __forceinline__ explicit Geo(int s) : S(s), Wp(s + 1), plane(((s + 2) * (s + 1) + 1) * 16u) {}
-    __device__ __forceinline__ uint32_t at(int y, int x) const { return (uint32_t)((y + 1) * Wp + x + 1) * 16u; }
-    __device__ __forceinline__ int ntx() const { return (S + 7) >> 3; }
-    __device__ __forceinline__ int tiles() const { return ntx() * ((S + 15) >> 4); }
-};
 
 struct Shared {
     uint64_t wfull[2], wempty[2], tile[MAX_TILES], dbar, act;
@@ -155,46 +60,6 @@ struct Shared {
 // sit in buffer i & 1 in the (i >> 1)-th filling of it.
 __device__ __forceinline__ uint32_t item_bytes(int cin, int cout, int taps) {
     return (uint32_t)(taps * cin * cout * 2 + cout * 8);
-}
-
-template <int V>
-struct Int {
-    static constexpr int value = V;
-};
-
-// The MMAs of one convolution, TAPS = 9 or 1 (the shortcut), tile t in TMEM
-// columns t COUT (the shortcut's from D_COL).  Each tile's completion goes to
-// its barrier (the shortcut's to dbar).  PAR: stride 2 on the parity images:
-// input row 2 y + dy has parity dy & 1 and row y (y - 1 for dy = -1).
-// Issued by the whole warp with uniform operands; the descriptors differ from
-// their first ones by start-address steps (16-byte units) that unroll to one
-// addition per MMA, as an N = 16 MMA takes few cycles itself.
-template <int CIN, int COUT, int TAPS, bool PAR>
-__device__ __forceinline__ void issue(uint32_t tmem, uint32_t abase, uint32_t wbase, const Geo &g, Shared &sh) {
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(COUT >> 3) << 17) | (8u << 24);
-    const uint64_t bd0 = desc_ns(wbase, (uint32_t)COUT * 16u, 128u);
-    const uint32_t p16 = g.plane >> 4, img = (uint32_t)(CIN / 8) * p16;      // 16-byte units
-    const int nt = g.tiles();
-    int y0 = 0, x0 = 0;
-    for (int t = 0; t < nt; ++t) {
-        const uint64_t ad0 = desc_ns(abase + g.at(y0, x0), g.plane, (uint32_t)g.Wp * 16u);
-        const uint32_t d = tmem + (TAPS == 1 ? D_COL : 0u) + (uint32_t)(t * COUT);
-#pragma unroll
-        for (int tap = 0; tap < TAPS; ++tap) {
-            const int dy = TAPS == 9 ? tap / 3 - 1 : 0, dx = TAPS == 9 ? tap % 3 - 1 : 0;
-            const int oy = PAR ? (dy < 0 ? -1 : 0) : dy, ox = PAR ? (dx < 0 ? -1 : 0) : dx;
-            const uint64_t ad = ad0 + (uint64_t)(int64_t)((PAR ? ((dy & 1) * 2 + (dx & 1)) * (int)img : 0) +
-                                                          oy * g.Wp + ox);
-            const uint64_t bd = bd0 + (uint64_t)(tap * (CIN / 8) * COUT);
-#pragma unroll
-            for (int k = 0; k < CIN / 16; ++k)
-                mma_bf16(d, ad + (uint64_t)(2u * k * p16), bd + (uint64_t)(2 * k * COUT), idesc, tap + k > 0 ? 1u : 0u);
-        }
-        if (TAPS == 9) mma_commit(&sh.tile[t]);
-        x0 += 8;
-        if (x0 >= g.S) { x0 = 0; y0 += 16; }
-    }
-    if (TAPS == 1) mma_commit(&sh.dbar);
 }
 
 // State of an epilogue thread.
@@ -424,7 +289,9 @@ __global__ void __launch_bounds__(NT, 1) wres_fused_kernel(const __grid_constant
             warp_wait(&sh.wfull[item & 1], (item >> 1) & 1, p.wait_cycles, dead);
             if (!dead) {
                 fence_after();
-                issue<CIN, COUT, TAPS, PAR>(tmem, abase, w0 + (uint32_t)(item & 1) * WBUF_BYTES, g, sh);
+                issue<CIN, COUT, TAPS, PAR>(tmem + (TAPS == 1 ? D_COL : 0u), abase,
+                                            w0 + (uint32_t)(item & 1) * WBUF_BYTES, g, TAPS == 9 ? sh.tile : nullptr,
+                                            TAPS == 1 ? &sh.dbar : nullptr);
                 mma_commit(&sh.wempty[item & 1]);
             }
             ++item;
@@ -598,10 +465,10 @@ minw_status launch_wres_fused(wfu::Args a, int B, cudaStream_t s) {
 
 int take_wres_error() {
     int flag = 0;
-    if (cudaMemcpyFromSymbol(&flag, g_wres_error, sizeof(int)) != cudaSuccess) return -1;
+    if (cudaMemcpyFromSymbol(&flag, smc::g_error, sizeof(int)) != cudaSuccess) return -1;
     if (flag) {
         const int zero = 0;
-        if (cudaMemcpyToSymbol(g_wres_error, &zero, sizeof(int)) != cudaSuccess) return -1;
+        if (cudaMemcpyToSymbol(smc::g_error, &zero, sizeof(int)) != cudaSuccess) return -1;
     }
     return flag ? 1 : 0;
 }
