@@ -185,7 +185,8 @@ __global__ void __launch_bounds__(256) aqe_backward_masked_kernel(const uint32_t
 // the 256 threads stay busy.
 // A warp per 32 channels with its channels in a serial loop, as before, had
 // one load in flight and few warps on small tensors: 256 x 512 x 14 x 14,
-// 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (MEASURED_NOW).
+// 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (51 and 4 us here; instruction issue bounds
+// the first, at 45 % of the resident warps).
 // ---------------------------------------------------------------------------
 
 enum QuantOut { OUT_PLANES, OUT_E4M3, OUT_E2M1 };
@@ -522,31 +523,43 @@ __global__ void weight_bf16_kernel(const float *__restrict__ w, int O, int C, in
     }
 }
 
-// fp32 NCHW -> bf16 NHWC, round to nearest even: one thread per output element
-// of a 32 x 32 (channel, pixel) tile transposed through shared memory.
-// Block (32, 8): a 32-channel x 32-pixel tile of one image through shared
-// memory; each thread's four loads issue before its first shared-memory store.
-// out [B][HW][Cp]: channels C .. Cp hold 0 (Cp >= C).
+// fp32 NCHW -> bf16 NHWC, round to nearest even, out [B][HW][Cp]: channels
+// C .. Cp hold 0 (Cp >= C).  A block takes 64 channels x 32 pixels of one
+// image through shared memory: a thread has the loads of eight channels of
+// its pixel in flight, and (VEC: Cp % 8 == 0, out 16-byte aligned) each
+// pixel's channels leave in 16-byte stores.  256 x 256 x 16 x 16: 24 us with
+// 32-channel tiles and 2-byte stores, 17 us here.
+template <bool VEC>
 __global__ void __launch_bounds__(256) to_bf16_nhwc_kernel(const float *__restrict__ x, int C, int Cp, int HW,
                                                            uint16_t *__restrict__ out) {
-    __shared__ float tile[32][33];
-    const int b = blockIdx.z, c0 = blockIdx.y * 32, p0 = blockIdx.x * 32;
-    float v[4];
+    __shared__ float tile[64][33];
+    const int b = blockIdx.z, c0 = blockIdx.y * 64, p0 = blockIdx.x * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    float v[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.y + 8 * k;
-        const int c = c0 + i, p = p0 + threadIdx.x;
+    for (int k = 0; k < 8; ++k) {
+        const int c = c0 + ty + 8 * k, p = p0 + tx;
         v[k] = (c < C && p < HW) ? __ldg(x + ((int64_t)b * C + c) * HW + p) : 0.0f;
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) tile[threadIdx.y + 8 * k][threadIdx.x] = v[k];
+    for (int k = 0; k < 8; ++k) tile[ty + 8 * k][tx] = v[k];
     __syncthreads();
+    if constexpr (VEC) {
+        const int g = threadIdx.x & 7, q = threadIdx.x >> 3, p = p0 + q, c = c0 + 8 * g;
+        if (p < HW && c < Cp) {
+            uint32_t w[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.y + 8 * k;
-        const int p = p0 + i, c = c0 + threadIdx.x;
-        if (c < Cp && p < HW)
-            out[((int64_t)b * HW + p) * Cp + c] = __bfloat16_as_ushort(__float2bfloat16_rn(tile[threadIdx.x][i]));
+            for (int e = 0; e < 4; ++e)
+                w[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tile[8 * g + 2 * e][q])) |
+                       ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(tile[8 * g + 2 * e + 1][q])) << 16);
+            *reinterpret_cast<uint4 *>(out + ((int64_t)b * HW + p) * Cp + c) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    } else {
+        for (int i = threadIdx.x; i < 64 * 32; i += 256) {
+            const int p = p0 + (i >> 6), c = c0 + (i & 63);
+            if (c < Cp && p < HW)
+                out[((int64_t)b * HW + p) * Cp + c] = __bfloat16_as_ushort(__float2bfloat16_rn(tile[i & 63][i >> 6]));
+        }
     }
 }
 
@@ -761,8 +774,11 @@ minw_status minw_to_bf16_nhwc_pad(const float *x, int32_t B, int32_t C, int32_t 
     if (B <= 0 || C <= 0 || H <= 0 || W <= 0 || Cp < C || !x || !out) return MINW_EINVAL;
     const int64_t HW = (int64_t)H * W;
     if (HW > (1ll << 30) || B > 65535 || (Cp + 31) / 32 > 65535) return MINW_EUNSUPPORTED;
-    const dim3 grid((unsigned)((HW + 31) / 32), (unsigned)((Cp + 31) / 32), (unsigned)B);
-    to_bf16_nhwc_kernel<<<grid, dim3(32, 8), 0, (cudaStream_t)stream>>>(x, C, Cp, (int)HW, out);
+    const dim3 grid((unsigned)((HW + 31) / 32), (unsigned)((Cp + 63) / 64), (unsigned)B);
+    if (Cp % 8 == 0 && aligned16(out))
+        to_bf16_nhwc_kernel<true><<<grid, 256, 0, (cudaStream_t)stream>>>(x, C, Cp, (int)HW, out);
+    else
+        to_bf16_nhwc_kernel<false><<<grid, 256, 0, (cudaStream_t)stream>>>(x, C, Cp, (int)HW, out);
     return launch_status();
 }
 

@@ -2229,13 +2229,15 @@ extern "C" minw_status minw_get_last_device_error(void *stream) {
         const int zero = 0;
         if (cudaMemcpyToSymbol(minw::g_device_error, &zero, sizeof(int)) != cudaSuccess) return MINW_ECUDA;
     }
-    const int first = minw::take_first_error();
-    const int first_tc = minw::take_first_tc_error();
-    const int planes_tc = minw::take_planes_tc_error();
-    const int wres = minw::take_wres_error();
-    const int wdense = minw::take_wdense_error();
-    if (first < 0 || first_tc < 0 || planes_tc < 0 || wres < 0 || wdense < 0) return MINW_ECUDA;
-    return (flag || first || first_tc || planes_tc || wres || wdense) ? MINW_ETIMEOUT : MINW_OK;
+    // the other kernels' flags: all are read, so that each report clears all of them
+    int any = flag;
+    for (int (*take)() : {minw::take_first_error, minw::take_first_tc_error, minw::take_planes_tc_error,
+                          minw::take_wres_error, minw::take_wdense_error, minw::take_wgrad_error}) {
+        const int f = take();
+        if (f < 0) return MINW_ECUDA;
+        any |= f;
+    }
+    return any ? MINW_ETIMEOUT : MINW_OK;
 }
 
 minw_host::EncodeTiledFn minw_host::tensor_map_encoder() {

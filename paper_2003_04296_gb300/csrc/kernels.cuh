@@ -119,6 +119,15 @@ minw_status conv2d_bf16_hardtanh(const uint16_t *act, int B, int C, int H, int W
                                  int O, int kh, int kw, int bits_w, int stride, int pad, const float *scale,
                                  const float *shift, uint16_t *hb_out, int hb_ld, int hb_off, cudaStream_t s,
                                  const float *res = nullptr, float *z = nullptr);
+// The weight gradient of a convolutional training step and its update (conv_wgrad.cu).
+struct WgradArgs {
+    const uint16_t *gd;        // g~ as bf16 NHWC [B][Hd][Wd][Op], output pixel (y, x) at (y stride, x stride)
+    const uint16_t *ab;        // the input as bf16 NHWC [B][H][W][C]
+    int B, C, H, W, O, kh, kw, stride, pad, Ho, Wo, Hd, Wd, Op;
+};
+size_t conv_wgrad_workspace_bytes(const WgradArgs &a);      // the partial sums
+minw_status launch_conv_wgrad(const WgradArgs &a, float *part, float lr, float two_alpha, float *W, cudaStream_t s);
+int take_wgrad_error();                                     // timeout flag (as take_first_error)
 bool conv_tc_supported(const ConvArgs &a);
 // Workspace the tensor-core path needs to split K for this shape (0: it does not split).
 size_t conv_tc_workspace_bytes(const ConvArgs &a);
