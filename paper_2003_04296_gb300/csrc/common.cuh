@@ -273,14 +273,12 @@ __device__ __forceinline__ uint32_t code4_k(int k) {
 
 // Stores the planes (bits of channels >= nvalid cleared) and the E4M3 codes
 // (ncodes = 16 or 32 bytes; the second 16 only when nvalid > 16) of OUTB-bit
-// levels given by their masks M[0 .. levels - 2].
+// levels given by their planes P[0 .. OUTB - 1].
 // With codes4 the codes are E2M1 nibbles instead (codes then points at the
 // byte of the first channel: 16 bytes for 32 channels, 8 for 16).
 template <int OUTB>
-__device__ __forceinline__ void store_level_masks(const uint32_t *M, int nvalid, int ncodes, uint32_t *planes, int NWo,
-                                                  uint8_t *codes, bool codes4 = false) {
-    uint32_t P[3];
-    level_planes<OUTB>(M, P);
+__device__ __forceinline__ void store_level_planes(const uint32_t *P, int nvalid, int ncodes, uint32_t *planes, int NWo,
+                                                   uint8_t *codes, bool codes4 = false) {
     if (planes != nullptr) {
         const uint32_t vm = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
 #pragma unroll
@@ -300,6 +298,15 @@ __device__ __forceinline__ void store_level_masks(const uint32_t *M, int nvalid,
             dst[1] = make_uint4(level_code_word<OUTB>(P, 4), level_code_word<OUTB>(P, 5), level_code_word<OUTB>(P, 6),
                                 level_code_word<OUTB>(P, 7));
     }
+}
+
+// ... given by their masks M[0 .. levels - 2].
+template <int OUTB>
+__device__ __forceinline__ void store_level_masks(const uint32_t *M, int nvalid, int ncodes, uint32_t *planes, int NWo,
+                                                  uint8_t *codes, bool codes4 = false) {
+    uint32_t P[3];
+    level_planes<OUTB>(M, P);
+    store_level_planes<OUTB>(P, nvalid, ncodes, planes, NWo, codes, codes4);
 }
 
 // Programmatic dependent launch: the kernels of a forward are launched so

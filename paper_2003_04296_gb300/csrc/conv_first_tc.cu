@@ -42,13 +42,13 @@
 // patches (one TMA box each, zero outside the image, as in conv_first.cu) and
 // a ring of A blocks (128 rows of [x1 | x2] pieces, 64 bytes each, in
 // 128-byte swizzled rows, built by four warps from the patch).
-// Warp roles (448 threads): warp 0 issues the patch boxes, warp 1 owns TMEM
+// Warp roles (512 threads): warp 0 issues the patch boxes, warp 1 owns TMEM
 // and issues the MMAs (two accumulators: the epilogue of one tile overlaps
 // the MMAs of the next), warps 2-5 build the A blocks (one pixel row per
-// thread) and warps 6-13 run the epilogue (two per TMEM lane quarter, each
-// half of the channels): decisions, the exact recompute of open decisions
-// (one per lane, spread over the warp), and stores of the next layer's codes
-// or bit-planes.  Every wait is bounded; a wait that runs out sets the
+// thread), warps 6-13 run the epilogue (two per TMEM lane quarter, each half
+// of the channels: decisions, a list of the open ones, and stores of the next
+// layer's codes or bit-planes) and warps 14-15 recompute a tile's open
+// decisions, one per lane, and correct the stored levels.  Every wait is bounded; a wait that runs out sets the
 // kernel's error flag and the CTA winds down.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -66,8 +66,9 @@ __device__ int g_first_tc_error = 0;
 
 namespace ftc {
 
-constexpr int NT = 448;
-constexpr int BUILD0 = 2, NBUILD = 4, EPI0 = 6, NEPI = 8;
+constexpr int NT = 512;
+constexpr int BUILD0 = 2, NBUILD = 4, EPI0 = 6, NEPI = 8, REC0 = EPI0 + NEPI, NREC = 2;
+constexpr int CAP = 256;       // open decisions a patch slot's list holds
 
 struct Params {
     int B, C, H, W, O, kh, kw, S, pad, Ho, Wo, npix;
@@ -81,7 +82,8 @@ struct Params {
     int NP, SA;            // patch slots, A block slots
     uint32_t b_block;      // bytes of one weight K block (O rows of 128 bytes)
     uint32_t idesc, tmem_cols;
-    uint32_t off_a, off_patch, off_w32, off_chan, off_koff, off_max, off_scr, off_bar;
+    uint32_t off_a, off_patch, off_w32, off_chan, off_koff, off_max, off_scr, off_list, off_bar;
+    int cap;               // entries of a patch slot's list of open decisions (CAP, or 0: recomputed in place)
     float c1;
     int nl;                // levels of the output quantizer
     const float *x;
@@ -189,6 +191,8 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
 // breakpoints -T_u 2^e, the unscaled -T_u of the exact recompute, and 2^e.
 constexpr int CREC = 16, R_SG = 0, R_A = 1, R_B = 2, R_NTS = 3, R_NT = 9, R_SC = 15;
 
+constexpr uint32_t EMPTY = 0xFFFFFFFFu;   // no open decision in this list entry
+
 // Compile-time first-layer shapes (the taps and their patch offsets unroll):
 // 1 = 3 channels 3 x 3 stride 1 (CIFAR), 2 = 3 channels 7 x 7 stride 2 (ResNet stem), 0 = any.
 template <int SHAPE> struct Shape { static constexpr int C = 0, KH = 0, KW = 0, S = 0, K = 0; };
@@ -208,6 +212,48 @@ __device__ __forceinline__ float tap(const float *pat, const int *sK, int k, int
     }
 }
 
+// The exact fp32 chain of one output, in batches of 16 taps: loads first, then
+// the fmafs in tap order (a padded tap past K adds fmaf(0, 0, acc) = acc: acc
+// is never -0).
+template <int SHAPE>
+__device__ __forceinline__ float chain(const float *pat, const float *wo, const int *sK, int K, int Rmax, int RP) {
+    float acc = 0.0f;
+    if constexpr (SHAPE > 0) {
+        constexpr int KC = Shape<SHAPE>::K;
+#pragma unroll
+        for (int k0 = 0; k0 < KC; k0 += 16) {
+            float xs[16], ws[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                xs[i] = tap<SHAPE>(pat, sK, k0 + i, K, Rmax, RP);
+                ws[i] = k0 + i < KC ? wo[k0 + i] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (k0 + i < KC) acc = fmaf(xs[i], ws[i], acc);
+        }
+    } else {
+        for (int k0 = 0; k0 < K; k0 += 16) {
+            float xs[16], ws[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int k = min(k0 + i, K - 1);
+                xs[i] = k0 + i < K ? pat[sK[k]] : 0.0f;
+                ws[i] = k0 + i < K ? wo[k] : 0.0f;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc = fmaf(xs[i], ws[i], acc);
+        }
+    }
+    return acc;
+}
+
+// ... as a call, for the rare recompute in the epilogue (its code stays out of the way).
+template <int SHAPE>
+__device__ __noinline__ float chain_call(const float *pat, const float *wo, const int *sK, int K, int Rmax, int RP) {
+    return chain<SHAPE>(pat, wo, sK, K, Rmax, RP);
+}
+
 template <int OUTB, int SHAPE>
 __global__ void __launch_bounds__(NT, 1)
     first_tc_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap tmX) {
@@ -223,10 +269,13 @@ __global__ void __launch_bounds__(NT, 1)
     int *sK = reinterpret_cast<int *>(smem + p.off_koff);           // [K] patch offset of each tap
     float *sM = reinterpret_cast<float *>(smem + p.off_max);        // [NP][128] maxabs per pixel row
     uint32_t *sS = reinterpret_cast<uint32_t *>(smem + p.off_scr);  // [NEPI][32] recompute lists
+    uint32_t *sL = reinterpret_cast<uint32_t *>(smem + p.off_list); // [NP][cap] open decisions, then [NP] counts
+    uint32_t *sN = sL + p.NP * p.cap;
     uint64_t *pfull = reinterpret_cast<uint64_t *>(smem + p.off_bar);
     uint64_t *pempty = pfull + p.NP;
     uint64_t *mfull = pempty + p.NP;
-    uint64_t *afull = mfull + p.NP;
+    uint64_t *efull = mfull + p.NP;      // a tile's epilogue is done: its stores and its list of open decisions
+    uint64_t *afull = efull + p.NP;
     uint64_t *aempty = afull + p.SA;
     uint64_t *tfull = aempty + p.SA;     // [2]
     uint64_t *tempty = tfull + 2;        // [2]
@@ -247,8 +296,9 @@ __global__ void __launch_bounds__(NT, 1)
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.NP; ++i) {
             bar_init(&pfull[i], 1);
-            bar_init(&pempty[i], NBUILD + NEPI);
+            bar_init(&pempty[i], NBUILD + 1);
             bar_init(&mfull[i], NBUILD);
+            bar_init(&efull[i], NEPI);
         }
         for (int i = 0; i < p.SA; ++i) {
             bar_init(&afull[i], NBUILD);
@@ -275,6 +325,7 @@ __global__ void __launch_bounds__(NT, 1)
         }
     }
     for (int g = threadIdx.x; g < O / 32; g += NT) sOpen[g] = 0u;
+    for (int i = threadIdx.x; i < p.NP * (p.cap + 1); i += NT) sL[i] = i < p.NP * p.cap ? EMPTY : 0u;
     fence_before();
     __syncthreads();
     fence_after();
@@ -358,31 +409,29 @@ __global__ void __launch_bounds__(NT, 1)
             const int pslot = n % p.NP;
             if (!__all_sync(0xffffffffu, bar_wait(&pfull[pslot], (uint32_t)(n / p.NP) & 1u, p.wait_cycles))) break;
             const int b = t / p.tiles_img, p0 = (t - b * p.tiles_img) * 128;
-            const int px = p0 + r;
-            const bool valid = px < npix;
-            const int pc = valid ? px : p0;
+            // rows past the image repeat its last pixel: their outputs are not stored
+            const int pc = min(p0 + r, npix - 1);
             const int oy = pc / p.Wo, ox = pc - oy * p.Wo;
             const float *pat = sP + (size_t)pslot * p.patch_floats + (oy - p0 / p.Wo) * S * RP + ox * S + p.xsh;
-            uint32_t mb = 0u;          // max |x| as a bit pattern (NaN patterns exceed infinity's)
+            float mx = 0.0f;           // max |x|, NaN once any x is
+            // eight taps at a time, two per conversion: x1 = fp16(x), x2 = fp16(x - x1)
             auto build = [&](int kbi, uint8_t *row) {
 #pragma unroll
                 for (int gi = 0; gi < 4; ++gi) {
-                    float x1[8], x2[8];
+                    uint32_t v1[4], v2[4];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float x = tap<SHAPE>(pat, sK, kbi * 32 + 8 * gi + j, K, Rmax, RP);
-                        x = valid ? x : 0.0f;
-                        mb = max(mb, __float_as_uint(x) & 0x7FFFFFFFu);
-                        const float h1 = __half2float(__float2half_rn(x));
-                        x1[j] = h1;
-                        x2[j] = x - h1;
+                    for (int j = 0; j < 4; ++j) {
+                        const float xa = tap<SHAPE>(pat, sK, kbi * 32 + 8 * gi + 2 * j, K, Rmax, RP);
+                        const float xb = tap<SHAPE>(pat, sK, kbi * 32 + 8 * gi + 2 * j + 1, K, Rmax, RP);
+                        asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(mx) : "f"(fabsf(xa)));
+                        asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(mx) : "f"(fabsf(xb)));
+                        const __half2 h = __floats2half2_rn(xa, xb);
+                        const float2 f = __half22float2(h);
+                        v1[j] = *reinterpret_cast<const uint32_t *>(&h);
+                        v2[j] = pack_h2(xa - f.x, xb - f.y);
                     }
-                    const uint4 v1 = make_uint4(pack_h2(x1[0], x1[1]), pack_h2(x1[2], x1[3]), pack_h2(x1[4], x1[5]),
-                                                pack_h2(x1[6], x1[7]));
-                    const uint4 v2 = make_uint4(pack_h2(x2[0], x2[1]), pack_h2(x2[2], x2[3]), pack_h2(x2[4], x2[5]),
-                                                pack_h2(x2[6], x2[7]));
-                    *reinterpret_cast<uint4 *>(row + ((gi ^ (r & 7)) << 4)) = v1;
-                    *reinterpret_cast<uint4 *>(row + (((4 + gi) ^ (r & 7)) << 4)) = v2;
+                    *reinterpret_cast<uint4 *>(row + ((gi ^ (r & 7)) << 4)) = make_uint4(v1[0], v1[1], v1[2], v1[3]);
+                    *reinterpret_cast<uint4 *>(row + (((4 + gi) ^ (r & 7)) << 4)) = make_uint4(v2[0], v2[1], v2[2], v2[3]);
                 }
             };
             auto block = [&](int kbi) -> bool {
@@ -405,14 +454,14 @@ __global__ void __launch_bounds__(NT, 1)
                     if (!block(kbi)) alive = false;
             }
             // the pixel's bound input for the epilogue: inf where the fp16 pieces do not hold x
-            sM[pslot * 128 + r] = mb >= 0x47000000u ? __int_as_float(0x7F800000) : __uint_as_float(mb);
+            sM[pslot * 128 + r] = mx < 32768.0f ? mx : __int_as_float(0x7F800000);
             __syncwarp();
             if (lane == 0) {
                 bar_arrive(&mfull[pslot]);
                 bar_arrive(&pempty[pslot]);
             }
         }
-    } else {
+    } else if (warp < REC0) {
         // ---------------- epilogue warps: weight preparation, then the epilogue ----------------
         const int et = threadIdx.x - EPI0 * 32;   // 0 .. 255
         // the chain's fp32 weights, [O][Ks]
@@ -540,7 +589,9 @@ __global__ void __launch_bounds__(NT, 1)
                 fl |= sOpen[ch0 >> 5];
                 if (!(mx < __int_as_float(0x7F800000))) fl = 0xFFFFFFFFu;
                 if (!valid) fl = 0u;
-                // open decisions: the exact fmaf chain, one output per lane, spread over the warp
+                // open decisions go to the tile's list (row, channel, the mask bits decided here), from which
+                // the recompute warps correct the stored levels; where the list is full they are recomputed here:
+                // the exact fmaf chain, one output per lane, spread over the warp
                 if (__any_sync(0xffffffffu, fl != 0u)) {
                     const uint32_t cnt = __popc(fl);
                     uint32_t excl = cnt;
@@ -551,7 +602,22 @@ __global__ void __launch_bounds__(NT, 1)
                     }
                     const uint32_t total = __shfl_sync(0xffffffffu, excl, 31);
                     excl -= cnt;
-                    for (uint32_t base = 0; base < total; base += 32) {
+                    uint32_t at = 0u;
+                    if (lane == 0) at = atomicAdd(sN + pslot, total);
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    const bool listed = at + total <= (uint32_t)p.cap;
+                    if (listed) {
+                        uint32_t f = fl, *dst = sL + pslot * p.cap + at + excl;
+                        while (f) {
+                            const int j = __ffs(f) - 1;
+                            f &= f - 1u;
+                            uint32_t bits = 0u;
+#pragma unroll
+                            for (int u = 0; u < NL - 1; ++u) bits |= ((M[u] >> j) & 1u) << u;
+                            *dst++ = (uint32_t)r | ((uint32_t)(ch0 + j) << 7) | (bits << 15);
+                        }
+                    }
+                    for (uint32_t base = 0; base < total && !listed; base += 32) {
                         uint32_t f = fl, idx = excl;
                         while (f) {
                             const int j = __ffs(f) - 1;
@@ -568,35 +634,7 @@ __global__ void __launch_bounds__(NT, 1)
                             const int oy = ps / p.Wo, ox = ps - oy * p.Wo;
                             const float *pat = pat0 + (oy - oyf) * S * RP + ox * S + p.xsh;
                             const float *wo = sW + o * Ks;
-                            // the chain in batches of 16 taps: loads first, then the fmafs in tap order
-                            // (a padded tap past K adds fmaf(0, 0, acc) = acc: acc is never -0)
-                            float acc = 0.0f;
-                            if constexpr (SHAPE > 0) {
-#pragma unroll
-                                for (int k0 = 0; k0 < KC; k0 += 16) {
-                                    float xs[16], ws[16];
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i) {
-                                        xs[i] = tap<SHAPE>(pat, sK, k0 + i, K, Rmax, RP);
-                                        ws[i] = k0 + i < KC ? wo[k0 + i] : 0.0f;
-                                    }
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i)
-                                        if (k0 + i < KC) acc = fmaf(xs[i], ws[i], acc);
-                                }
-                            } else {
-                                for (int k0 = 0; k0 < K; k0 += 16) {
-                                    float xs[16], ws[16];
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i) {
-                                        const int k = min(k0 + i, K - 1);
-                                        xs[i] = k0 + i < K ? pat[sK[k]] : 0.0f;
-                                        ws[i] = k0 + i < K ? wo[k] : 0.0f;
-                                    }
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i) acc = fmaf(xs[i], ws[i], acc);
-                                }
-                            }
+                            const float acc = chain_call<SHAPE>(pat, wo, sK, K, Rmax, RP);
                             const float *rec = sC + (size_t)o * CREC;
                             uint32_t bits = 0u;
 #pragma unroll
@@ -632,6 +670,57 @@ __global__ void __launch_bounds__(NT, 1)
             __syncwarp();
             if (lane == 0 && !dead) {
                 bar_arrive(&tempty[ab]);
+                bar_arrive(&efull[pslot]);
+            }
+        }
+    } else {
+        // ---------------- recompute warps: the open decisions of a tile, 32 at a time ----------------
+        // About 0.3 % of the stem's decisions are open, a few per 32-channel chunk: chunk by chunk their
+        // 147-tap chains kept a warp busy for three lanes' work.
+        const int NWo = (O + 31) >> 5;
+        int n = 0;
+        bool dead = false;
+        for (int t = blockIdx.x; t < p.tiles && !dead; t += gridDim.x, ++n) {
+            if (n % NREC != warp - REC0) continue;
+            const int pslot = n % p.NP;
+            if (!__all_sync(0xffffffffu, bar_wait(&efull[pslot], (uint32_t)(n / p.NP) & 1u, p.wait_cycles))) { dead = true; break; }
+            const int b = t / p.tiles_img, p0 = (t - b * p.tiles_img) * 128, oyf = p0 / p.Wo;
+            const float *pat0 = sP + (size_t)pslot * p.patch_floats;
+            uint32_t *list = sL + pslot * p.cap;
+            const int cnt = (int)min(sN[pslot], (uint32_t)p.cap);
+            for (int i = lane; i < cnt; i += 32) {
+                const uint32_t e = list[i];
+                list[i] = EMPTY;
+                if (e == EMPTY) continue;
+                const int ps = p0 + (int)(e & 127u), o = (int)((e >> 7) & 255u);
+                const int oy = ps / p.Wo, ox = ps - oy * p.Wo;
+                const float *pat = pat0 + (oy - oyf) * S * RP + ox * S + p.xsh;
+                const float acc = chain<SHAPE>(pat, sW + o * Ks, sK, K, Rmax, RP);
+                const float *rec = sC + (size_t)o * CREC;
+                uint32_t bits = 0u;
+#pragma unroll
+                for (int u = 0; u < NL - 1; ++u) bits |= (__float_as_uint(fmaf(acc, rec[R_SG], rec[R_NT + u])) >> 31) << u;
+                const int k0 = NL - 1 - __popc(e >> 15), k1 = NL - 1 - __popc(bits);     // nested masks: the level index
+                if (k0 == k1) continue;
+                const long long m = (long long)b * npix + ps;
+                // neighbouring channels of the word may be corrected at the same time: exclusive or of the change
+                if (p.planes_out != nullptr) {
+                    const uint32_t d = planes_of_index(k0, OUTB) ^ planes_of_index(k1, OUTB);
+                    for (int u = 0; u < OUTB; ++u)
+                        if ((d >> u) & 1u) atomicXor(p.planes_out + (m * OUTB + u) * NWo + (o >> 5), 1u << (o & 31));
+                }
+                if (p.codes_out != nullptr) {
+                    const long long c = m * O + o;
+                    uint32_t *w = reinterpret_cast<uint32_t *>(p.codes_out);
+                    if (p.codes4)
+                        atomicXor(w + (c >> 3), (code4_k<OUTB>(k0) ^ code4_k<OUTB>(k1)) << (4 * (int)(c & 7)));
+                    else
+                        atomicXor(w + (c >> 2), (code_of_index(k0, OUTB) ^ code_of_index(k1, OUTB)) << (8 * (int)(c & 3)));
+                }
+            }
+            __syncwarp();
+            if (lane == 0) {
+                sN[pslot] = 0u;
                 bar_arrive(&pempty[pslot]);
             }
         }
@@ -698,9 +787,10 @@ static bool first_tc_plan(const FirstArgs &a, ftc::Params &p) {
     // recompute lists, barriers (three patches and three A blocks in flight where they fit)
     const size_t limit = 227 * 1024 - 1024;
     static const int np_[6] = {4, 3, 3, 2, 2, 1}, sa_[6] = {4, 4, 3, 3, 2, 2};
-    for (int cfg = 0; cfg < 6; ++cfg) {
-        p.NP = np_[cfg];
-        p.SA = sa_[cfg];
+    for (int cfg = 0; cfg < 12; ++cfg) {
+        p.NP = np_[cfg % 6];
+        p.SA = sa_[cfg % 6];
+        p.cap = cfg < 6 ? ftc::CAP : 0;         // lists of open decisions where they fit, else recomputed in place
         size_t off = (size_t)p.nkb * p.b_block;
         p.off_a = (uint32_t)off;
         off += (size_t)p.SA * 16384u;
@@ -716,9 +806,11 @@ static bool first_tc_plan(const FirstArgs &a, ftc::Params &p) {
         off += (size_t)p.NP * 128 * sizeof(float);
         p.off_scr = (uint32_t)off;
         off += (size_t)ftc::NEPI * 32 * sizeof(uint32_t);
+        p.off_list = (uint32_t)off;
+        off += (size_t)p.NP * (p.cap + 1) * sizeof(uint32_t);
         off = align_up(off, 8);
         p.off_bar = (uint32_t)off;
-        off += (size_t)(3 * p.NP + 2 * p.SA + 6) * sizeof(uint64_t) + 16;
+        off += (size_t)(4 * p.NP + 2 * p.SA + 6) * sizeof(uint64_t) + 16;
         if (off <= limit) {
             p.tmem_cols = 32;
             while (p.tmem_cols < (p.split ? 4u : 2u) * (uint32_t)a.O) p.tmem_cols <<= 1;
@@ -731,7 +823,7 @@ static bool first_tc_plan(const FirstArgs &a, ftc::Params &p) {
 }
 
 static size_t first_tc_smem(const ftc::Params &p) {
-    return (size_t)p.off_bar + (size_t)(3 * p.NP + 2 * p.SA + 6) * sizeof(uint64_t) + 16 + 1024;
+    return (size_t)p.off_bar + (size_t)(4 * p.NP + 2 * p.SA + 6) * sizeof(uint64_t) + 16 + 1024;
 }
 
 bool first_tc_supported(const FirstArgs &a) {

@@ -31,6 +31,7 @@
 // CTA stops issuing work, drains its own TMA loads and frees its TMEM.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -85,6 +86,7 @@ struct Params {
     const float *res_f32;      // shortcut as fp32 NHWC [B][Hp][Wp][O] (nullable)
     float *y_nhwc;             // BN output (before the shortcut) as fp32 NHWC (nullable)
     const float *ythr;         // breakpoints of the output quantizer on y (nullable: computed here)
+    int resal;                 // the shortcut and y_nhwc start on 16 bytes (wide accesses)
     uint16_t *hb_out;          // bf16 operands: HardTanh(BN(acc) [+ hb_res]) as bf16 NHWC rows of hb_ld, at hb_off
     int hb_ld, hb_off;
     const float *hb_res;       // fp32 NCHW shortcut (nullable)
@@ -495,15 +497,56 @@ __device__ __forceinline__ void mask_chunk(uint32_t taddr, bool full32, const fl
     mask_chunk_regs<OUTB>(v, full32, th, tstride, sig, pool, bw, writer, nvalid, planes, NWo, codes, codes4);
 }
 
+// The shortcut's level codes of 32 channels of one pixel (16 bytes of E2M1
+// nibbles, or 32 of E4M3; the second half only where those channels exist).
+struct ResCodes {
+    uint4 lo, hi;
+};
+__device__ __forceinline__ ResCodes load_res_codes(const Params &p, int ob, long long opix, bool writer, bool full32) {
+    ResCodes r;
+    r.lo = r.hi = make_uint4(0u, 0u, 0u, 0u);
+    if (!writer || ob >= p.O) return r;
+    const long long base = opix * p.O + ob;
+    const bool two = full32 && p.O - ob > 16;
+    if (p.res4) {
+        const uint2 *src = reinterpret_cast<const uint2 *>(p.res_codes + base / 2);    // 8-byte aligned at O % 16
+        const uint2 a = __ldg(src);
+        const uint2 b = two ? __ldg(src + 1) : make_uint2(0u, 0u);
+        r.lo = make_uint4(a.x, a.y, b.x, b.y);
+    } else {
+        const uint4 *src = reinterpret_cast<const uint4 *>(p.res_codes + base);
+        r.lo = __ldg(src);
+        if (two) r.hi = __ldg(src + 1);
+    }
+    return r;
+}
+
+// Two level codes (the low byte's E2M1 nibbles, or two E4M3 bytes) as fp32 integer units; exact conversions.
+__device__ __forceinline__ float2 res_pair_e2m1(uint32_t v) {
+    uint32_t h;
+    asm("{\n .reg .b8 b;\n cvt.u8.u32 b, %1;\n cvt.rn.f16x2.e2m1x2 %0, b;\n}\n" : "=r"(h) : "r"(v));
+    return __half22float2(*reinterpret_cast<__half2 *>(&h));
+}
+__device__ __forceinline__ float2 res_pair_e4m3(uint32_t v) {
+    uint32_t h;
+    asm("cvt.rn.f16x2.e4m3x2 %0, %1;\n" : "=r"(h) : "h"((uint16_t)v));
+    return __half22float2(*reinterpret_cast<__half2 *>(&h));
+}
+
 // Epilogue of one 32-column chunk (16 when full32 is false) of a residual
-// block, one output pixel per lane: y = fmaf(acc, scale, shift), stored as
-// fp32 NHWC when asked (the BN output before the shortcut), then y + shortcut
-// (one fp32 add) and the next layer's levels from the sign bits of
-// y + (-T_u) against the quantizer's own breakpoints on y (HardTanh included),
-// through the same level masks as the plain epilogue.
+// block, one output pixel per lane: y = fmaf(acc, scale, shift) from the
+// shared-memory maps ssc and ssh, stored as fp32 NHWC when asked (the BN
+// output before the shortcut), then y + shortcut (one fp32 add: a code's value
+// times its unit is exact, so the fused multiply-add rounds once, as the add
+// does) and the next layer's levels from the sign bits of y + (-T_u) against
+// the quantizer's own breakpoints on y (HardTanh included).  A 3-bit
+// quantizer whose breakpoints mirror (sym: a level and its negative at
+// opposite y) needs four masks instead of six: |y| against the three positive
+// breakpoints and the sign of y give its planes.
 template <int OUTB>
 __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const Params &p, int ob, long long opix,
-                                            bool writer, const float *syt, int NWo) {
+                                            bool writer, const float *ssc, const float *ssh, const float *syt, bool sym,
+                                            const ResCodes &rc, int NWo) {
     uint32_t v[32];
     if (full32) {
         tmem_ld32(taddr, v);
@@ -521,9 +564,13 @@ __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const P
     const int ncol = full32 ? 32 : 16;
     float y[32];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const int o = min(ob + j, p.O - 1);
-        y[j] = fmaf(__uint_as_float(v[j]), __ldg(p.scale + o), __ldg(p.shift + o));
+    for (int q4 = 0; q4 < 8; ++q4) {
+        const float4 c = *reinterpret_cast<const float4 *>(ssc + ob + 4 * q4);
+        const float4 h = *reinterpret_cast<const float4 *>(ssh + ob + 4 * q4);
+        y[4 * q4] = fmaf(__uint_as_float(v[4 * q4]), c.x, h.x);
+        y[4 * q4 + 1] = fmaf(__uint_as_float(v[4 * q4 + 1]), c.y, h.y);
+        y[4 * q4 + 2] = fmaf(__uint_as_float(v[4 * q4 + 2]), c.z, h.z);
+        y[4 * q4 + 3] = fmaf(__uint_as_float(v[4 * q4 + 3]), c.w, h.w);
     }
     const long long base = opix * p.O + ob;
     if (p.y_nhwc != nullptr) {
@@ -534,26 +581,20 @@ __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const P
     }
     if constexpr (OUTB > 0) {
         if (p.res_codes != nullptr && p.res4) {
-            const uint2 *src = reinterpret_cast<const uint2 *>(p.res_codes + base / 2);
+            const uint32_t cw[4] = {rc.lo.x, rc.lo.y, rc.lo.z, rc.lo.w};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h * 16 >= nvalid || h * 16 >= ncol) break;
-                const uint2 cv = __ldg(src + h);
-                const uint32_t cw[2] = {cv.x, cv.y};
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    y[h * 16 + j] += code_units_e2m1(cw[j >> 3] >> (4 * (j & 7))) * p.res_unit;
+            for (int j = 0; j < 32; j += 2) {
+                const float2 r = res_pair_e2m1(cw[j >> 3] >> (4 * (j & 7)));
+                y[j] = fmaf(r.x, p.res_unit, y[j]);
+                y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
             }
         } else if (p.res_codes != nullptr) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(p.res_codes + base);
+            const uint32_t cw[8] = {rc.lo.x, rc.lo.y, rc.lo.z, rc.lo.w, rc.hi.x, rc.hi.y, rc.hi.z, rc.hi.w};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h * 16 >= nvalid || h * 16 >= ncol) break;
-                const uint4 cv = __ldg(src + h);
-                const uint32_t cw[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    y[h * 16 + j] += code_units((cw[j >> 2] >> (8 * (j & 3))) & 0xFFu) * p.res_unit;
+            for (int j = 0; j < 32; j += 2) {
+                const float2 r = res_pair_e4m3(cw[j >> 2] >> (8 * (j & 3)));
+                y[j] = fmaf(r.x, p.res_unit, y[j]);
+                y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
             }
         } else if (p.res_f32 != nullptr) {
             const float4 *src = reinterpret_cast<const float4 *>(p.res_f32 + base);
@@ -568,6 +609,22 @@ __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const P
             }
         }
         constexpr int NL = OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7);
+        uint32_t *planes = p.planes_out ? p.planes_out + (opix * OUTB) * NWo + (ob >> 5) : nullptr;
+        uint8_t *codes = p.codes_out ? p.codes_out + (p.out4 ? base / 2 : base) : nullptr;
+        if (OUTB == 3 && sym) {
+            const float t1 = syt[3], t2 = syt[4], t3 = syt[5];       // -T of levels 1, 2 and 4 (units)
+            uint32_t n1 = 0u, n2 = 0u, n3 = 0u, ng = 0u;             // |y| below each; y below zero
+#pragma unroll
+            for (int j = 31; j >= 0; --j) {
+                n1 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t1), n1, 1);
+                n2 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t2), n2, 1);
+                n3 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t3), n3, 1);
+                ng = __funnelshift_l(__float_as_uint(y[j]), ng, 1);
+            }
+            const uint32_t P[3] = {ng & ~n1, ~n1 & (n2 | ~n3), ~n2};
+            store_level_planes<3>(P, nvalid, ncol, planes, NWo, codes, p.out4 != 0);
+            return;
+        }
         float nt[NL - 1];
 #pragma unroll
         for (int u = 0; u < NL - 1; ++u) nt[u] = syt[u];
@@ -578,8 +635,7 @@ __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const P
         for (int j = 31; j >= 0; --j)
 #pragma unroll
             for (int u = 0; u < NL - 1; ++u) M[u] = __funnelshift_l(__float_as_uint(y[j] + nt[u]), M[u], 1);
-        store_level_masks<OUTB>(M, nvalid, ncol, p.planes_out ? p.planes_out + (opix * OUTB) * NWo + (ob >> 5) : nullptr,
-                                NWo, p.codes_out ? p.codes_out + (p.out4 ? base / 2 : base) : nullptr, p.out4 != 0);
+        store_level_masks<OUTB>(M, nvalid, ncol, planes, NWo, codes, p.out4 != 0);
     }
 }
 
@@ -703,10 +759,13 @@ __global__ void __launch_bounds__(NT, 1)
     const int O32 = (p.O + 31) & ~31;
     float *sthr = reinterpret_cast<float *>(smem + (size_t)p.S * p.stage_bytes +
                                             (p.wres ? (size_t)p.nk * p.b_bytes : 0));   // after the resident weights
-    const int thr_floats = OUTB ? O32 * NL : 0;
+    // (residual epilogues: the BN scale, then the shift, of O32 channels in their place)
+    const bool resid = p.res_codes != nullptr || p.res_f32 != nullptr || p.y_nhwc != nullptr;
+    const int thr_floats = OUTB ? O32 * NL : resid ? 2 * O32 : 0;
     uint32_t *ssig = reinterpret_cast<uint32_t *>(sthr + thr_floats);              // [O32 / 32]
     const int sig_words = OUTB ? O32 / 32 : 0;
     // breakpoints of the output quantizer on y itself (residual blocks), held as -T
+    // (its word 7: 1 when a 3-bit quantizer's breakpoints mirror, see resid_chunk)
     float *syt = reinterpret_cast<float *>(ssig + ((sig_words + 1) & ~1));
     // staging tiles of the row-contiguous stores, one 32 x 16-word tile per epilogue warp
     uint32_t *sy = reinterpret_cast<uint32_t *>(syt + (OUTB ? 8 : 0));
@@ -984,31 +1043,40 @@ __global__ void __launch_bounds__(NT, 1)
             // held as (-T_1 .. -T_{n-1}, sigma) with -0 stored as +0, so that
             // fmaf(acc, sigma, -T) is never -0 and its sign bit is [sigma * acc < T]
             // rows u = 0 .. NL - 1 of O32 channels each (channel fastest: four channels per 128-bit load)
-            if (p.thr != nullptr) {
+            if (resid) {
+                // a residual block quantizes y + shortcut: no per-channel breakpoints on acc
+            } else if (p.thr != nullptr) {
                 for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {
                     const float x = __ldg(p.thr + i);
                     const int o = i / NL, u = i - o * NL;
                     sthr[u * O32 + o] = (u == NL - 1) ? x : mask_breakpoint(x);
                 }
-            } else if (p.res_codes == nullptr && p.res_f32 == nullptr) {
-                // (a residual block quantizes y + shortcut: no per-channel breakpoints on acc)
+            } else {
                 for (int o = et; o < p.O; o += EPI_WARPS * 32) {
                     float t[8];
                     channel_thresholds(__ldg(p.scale + o), __ldg(p.shift + o), p.qo, t);
                     for (int u = 0; u < NL; ++u) sthr[u * O32 + o] = (u == NL - 1) ? t[u] : mask_breakpoint(t[u]);
                 }
             }
-            for (int i = p.O * NL + et; i < thr_floats; i += EPI_WARPS * 32) {      // padding channels
+            for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
                 const int k = i - p.O * NL, o = p.O + k / NL, u = k % NL;
                 sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
             }
-            if (p.res_codes != nullptr || p.res_f32 != nullptr) {       // level of y = #{u : y >= T_u}
-                if (p.ythr != nullptr) {
-                    if (et < NL - 1) syt[et] = mask_breakpoint(__ldg(p.ythr + et));
-                } else if (et == 0) {
+            if (resid) {                                        // level of y = #{u : y >= T_u}
+                if (et == 0) {
                     float t[8];
-                    channel_thresholds_f32(1.0f, 0.0f, p.qo, t);         // a long serial search: callers cache it
+                    if (p.ythr != nullptr)
+                        for (int u = 0; u < NL - 1; ++u) t[u] = __ldg(p.ythr + u);
+                    else
+                        channel_thresholds_f32(1.0f, 0.0f, p.qo, t);     // a long serial search: callers cache it
                     for (int u = 0; u < NL - 1; ++u) syt[u] = mask_breakpoint(t[u]);
+                    // the breakpoint below level index 3 - e is the next fp32 value above -(that of 3 + e)
+                    bool sym = NL == 7;
+                    if constexpr (NL == 7)
+                        for (int e = 0; e < 3; ++e)
+                            sym = sym && t[3 + e] > 0.0f && isfinite(t[3 + e]) &&
+                                  t[2 - e] == __uint_as_float(__float_as_uint(-t[3 + e]) - 1u);
+                    syt[7] = sym ? 1.0f : 0.0f;
                 }
             }
             // sigma of a channel: the sign of its BN scale (+1 for 0); one warp per
@@ -1020,6 +1088,12 @@ __global__ void __launch_bounds__(NT, 1)
                                          : 1.0f;
                 const uint32_t m = __ballot_sync(0xffffffffu, sg > 0.0f);
                 if (lane == 0) ssig[g] = m;
+            }
+        }
+        if (resid) {
+            for (int o = et; o < O32; o += EPI_WARPS * 32) {
+                sthr[o] = o < p.O ? __ldg(p.scale + o) : 0.0f;
+                sthr[O32 + o] = o < p.O ? __ldg(p.shift + o) : 0.0f;
             }
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");   // breakpoints in place
@@ -1037,7 +1111,6 @@ __global__ void __launch_bounds__(NT, 1)
         const int gbeg = half_cols ? gmid : 0, gend = half_cols ? ngrp : gmid;
         // mask epilogue (a layer whose only output is the next layer's levels):
         // this warp's 32-column chunks
-        const bool resid = p.res_codes != nullptr || p.res_f32 != nullptr || p.y_nhwc != nullptr;
         // the accumulator is drained: CTA 1 of a pair tells CTA 0, which issues the MMAs
         auto tempty_arrive = [&](uint64_t *bar) {
             if (PAIR && crank == 1)
@@ -1048,7 +1121,7 @@ __global__ void __launch_bounds__(NT, 1)
         const bool masked = OUTB > 0 && p.ksplit == 1 && p.acc_out == nullptr && p.y_out == nullptr && !resid;
         // residual epilogue without per-element fp32 outputs: the same chunks
         const bool rmasked = p.ksplit == 1 && p.acc_out == nullptr && p.y_out == nullptr && !p.pool && resid &&
-                             p.O % 16 == 0;
+                             p.O % 16 == 0 && p.resal;
         const int nch = (p.BN + 31) >> 5, cmid = (nch + 1) >> 1;
         const int cbeg = half_cols ? cmid : 0, cend = half_cols ? nch : cmid;
         int i = 0;
@@ -1088,20 +1161,12 @@ __global__ void __launch_bounds__(NT, 1)
                     }
                     if (!dead && !mbar_wait(&tfull[ab], use & 1, p.wait_cycles)) dead = true;
                     fence_after();
-                    const bool tres = p.res_codes != nullptr || p.res_f32 != nullptr;
-                    float sc = 0.0f, sh = 0.0f, ny[NL - 1];
-#pragma unroll
-                    for (int u = 0; u < NL - 1; ++u) ny[u] = syt[u];
-                    if (tres && qlive) {
-                        sc = __ldg(p.scale + oc);
-                        sh = __ldg(p.shift + oc);
-                    }
                     // plain block epilogue of 1- and 2-bit outputs: two chunks at a time, their loads,
                     // sign chains, transposes, pooling and stores interleaved (a 3-bit output's six
                     // mask chains per chunk already overlap)
 #pragma unroll
                     for (int k = 0; k < 4; k += 2) {
-                        if (NL > 3 || k >= cq || dead || !qlive || tres) break;
+                        if (NL > 3 || k >= cq || dead || !qlive) break;
                         __syncwarp();
                         uint32_t v0[32], v1[32];
                         const uint32_t ta = tmem_base + ((uint32_t)oq << 16) + (uint32_t)(ab * p.acc_cols + (cb + k) * 32);
@@ -1151,7 +1216,7 @@ __global__ void __launch_bounds__(NT, 1)
                             }
                         }
                     }
-                    for (int c = cb; c < cb + cq && !dead && qlive && (tres || NL > 3); ++c) {
+                    for (int c = cb; c < cb + cq && !dead && qlive && NL > 3; ++c) {
                         __syncwarp();
                         uint32_t v[32];
                         tmem_ld32(tmem_base + ((uint32_t)oq << 16) + (uint32_t)(ab * p.acc_cols + c * 32), v);
@@ -1161,50 +1226,13 @@ __global__ void __launch_bounds__(NT, 1)
                         const int x = xb * p.bw + r % p.bw;
                         const bool valid = b < p.B && y < p.Ho && x < p.Wo;
                         uint32_t M[NL - 1];
-                        if (tres) {
-                            // residual block: y = BN(acc) + shortcut at (pixel j, this lane's channel), then the
-                            // quantizer's breakpoints on y; pixel j's index comes from lane j
-                            // (all 32 loads issue before the first use; a pixel past the batch reads pixel 0)
-                            const long long pix = valid ? (((long long)b * p.Ho + y) * p.Wo + x) * p.O : 0;
-                            float yv[32];
-                            if (p.res_codes != nullptr && p.res4) {
-                                uint32_t cb[32];
 #pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    cb[j] = __ldg(p.res_codes + ((oc + __shfl_sync(0xffffffffu, pix, j)) >> 1));
+                        for (int u = 0; u < NL - 1; ++u) {
+                            uint32_t wd = 0u;          // bit j: [sigma * acc < T_u] at pixel column 32 c + j
 #pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    yv[j] = fmaf(__uint_as_float(v[j]), sc, sh) +
-                                            code_units_e2m1(cb[j] >> (4 * (oc & 1))) * p.res_unit;
-                            } else if (p.res_codes != nullptr) {
-                                uint32_t cb[32];
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) cb[j] = __ldg(p.res_codes + oc + __shfl_sync(0xffffffffu, pix, j));
-#pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    yv[j] = fmaf(__uint_as_float(v[j]), sc, sh) + code_units(cb[j]) * p.res_unit;
-                            } else {
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) yv[j] = __ldg(p.res_f32 + oc + __shfl_sync(0xffffffffu, pix, j));
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) yv[j] = fmaf(__uint_as_float(v[j]), sc, sh) + yv[j];
-                            }
-#pragma unroll
-                            for (int u = 0; u < NL - 1; ++u) {
-                                uint32_t wd = 0u;
-#pragma unroll
-                                for (int j = 31; j >= 0; --j) wd = __funnelshift_l(__float_as_uint(yv[j] + ny[u]), wd, 1);
-                                M[u] = transpose32(wd, lane);
-                            }
-                        } else {
-#pragma unroll
-                            for (int u = 0; u < NL - 1; ++u) {
-                                uint32_t wd = 0u;          // bit j: [sigma * acc < T_u] at pixel column 32 c + j
-#pragma unroll
-                                for (int j = 31; j >= 0; --j)
-                                    wd = __funnelshift_l(__float_as_uint(fmaf(__uint_as_float(v[j]), sg, nt[u])), wd, 1);
-                                M[u] = transpose32(wd, lane);     // lane j: bit k = channel oq + k at column 32 c + j
-                            }
+                            for (int j = 31; j >= 0; --j)
+                                wd = __funnelshift_l(__float_as_uint(fmaf(__uint_as_float(v[j]), sg, nt[u])), wd, 1);
+                            M[u] = transpose32(wd, lane);     // lane j: bit k = channel oq + k at column 32 c + j
                         }
                         if (p.pool) {
 #pragma unroll
@@ -1271,14 +1299,22 @@ __global__ void __launch_bounds__(NT, 1)
                 }
             }
             if (rmasked) {
+                // a chunk's shortcut codes load one chunk ahead, the first while the MMAs run
+                const bool rcodes = OUTB > 0 && p.res_codes != nullptr;
+                ResCodes rc{};
+                if (rcodes) rc = load_res_codes(p, o0 + cbeg * 32, opix, writer, cbeg * 32 + 32 <= p.BN);
                 if (!dead && !mbar_wait(&tfull[ab], use & 1, p.wait_cycles)) dead = true;
                 fence_after();
                 for (int c = cbeg; c < cend && !dead; ++c) {
                     const int ob = o0 + c * 32;
                     if (ob >= p.O) break;
+                    ResCodes nx{};
+                    if (rcodes && c + 1 < cend) nx = load_res_codes(p, ob + 32, opix, writer, c * 32 + 64 <= p.BN);
                     __syncwarp();
                     resid_chunk<OUTB>(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * p.BN + c * 32),
-                                      c * 32 + 32 <= p.BN, p, ob, opix, writer, syt, NWo);
+                                      c * 32 + 32 <= p.BN, p, ob, opix, writer, sthr, sthr + O32, syt,
+                                      OUTB == 3 && syt[7] != 0.0f, rc, NWo);
+                    rc = nx;
                 }
                 fence_before();
                 __syncwarp();
@@ -1822,8 +1858,7 @@ static bool trans_shape(const ConvArgs &a, Params &p) {
 static bool trans_eligible(const ConvArgs &a) {
     return trans_pref() && (a.O == 128 || a.O == 64) && a.quant_out && (a.codes_out != nullptr || a.planes_out != nullptr) &&
            a.acc_out == nullptr && a.y_out == nullptr && a.y_nhwc == nullptr && a.ksplit <= 1 &&
-           (a.res_codes == nullptr && a.res_f32 == nullptr ||
-            ((a.O == 128 || (a.O == 64 && dup_pref())) && !a.pool));   // residual: all 8 warps hold channels
+           a.res_codes == nullptr && a.res_f32 == nullptr;      // residual epilogues read a pixel's channels together
 }
 
 // encode = false plans the tiles and the split only (no tensor maps: no driver call).
@@ -1886,10 +1921,12 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     }
     p.b_bytes = (uint32_t)((p.pair ? p.BN / 2 : p.BN) * p.cb);   // pairs: each CTA holds half the weight rows
     const size_t o32 = ((size_t)a.O + 31) & ~(size_t)31;
-    const size_t thr_bytes = a.quant_out ? (o32 * p.nlev + o32 / 32 + 10) * sizeof(float) : 0;
+    const bool resid_ = a.res_codes != nullptr || a.res_f32 != nullptr || a.y_nhwc != nullptr;
+    const size_t thr_bytes = a.quant_out ? (o32 * p.nlev + o32 / 32 + 10) * sizeof(float)
+                             : resid_    ? o32 * 2 * sizeof(float)
+                                         : 0;
     // staging tiles of the row-contiguous stores: a layer that may split along K,
     // or whose fp32 output is a fully connected one (1 x 1 images)
-    const bool resid_ = a.res_codes != nullptr || a.res_f32 != nullptr || a.y_nhwc != nullptr;
     const bool rowst_fc = !p.trans && a.y_out != nullptr && a.Ho == 1 && a.Wo == 1 && !a.pool && !a.quant_out &&
                           a.acc_out == nullptr && !resid_;
     const bool may_split = a.workspace != nullptr && !a.pool && !p.trans && !p.pair && !a.upd;
@@ -1956,7 +1993,10 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     p.upd = a.upd; p.upd_lr = a.upd_lr; p.upd_2a = a.upd_2a;
     p.pool = a.pool; p.quant_out = a.quant_out; p.qo = a.qo;
     p.planes_out = a.planes_out; p.codes_out = a.codes_out;
-    p.res_codes = a.res_codes; p.res_unit = a.res_unit; p.res_f32 = a.res_f32; p.y_nhwc = a.y_nhwc;
+    if (a.scale != nullptr) {                             // raw accumulators alone: no BN output to add to
+        p.res_codes = a.res_codes; p.res_unit = a.res_unit; p.res_f32 = a.res_f32; p.y_nhwc = a.y_nhwc;
+    }
+    p.resal = minw_host::aligned16(a.res_codes) && minw_host::aligned16(a.res_f32) && minw_host::aligned16(a.y_nhwc);
     p.ythr = a.ythr;
     p.hb_out = a.hb_out; p.hb_ld = a.hb_ld; p.hb_off = a.hb_off; p.hb_res = a.hb_res; p.hb_z = a.hb_z;
 
