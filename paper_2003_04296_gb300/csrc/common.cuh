@@ -130,29 +130,26 @@ __device__ __forceinline__ uint32_t planes_of_index(int k, int bits) {
     return (uint32_t)((06420357ull >> (3 * k)) & 7ull);     // octal digits, idx 0 = low
 }
 
+// Breakpoint T_j (1 <= j < n) of a channel with BN map (s, t).
+__device__ __forceinline__ float channel_threshold(float s, float t, const QParams &q, int j) {
+    const float sigma = (s < 0.0f) ? -1.0f : 1.0f;
+    const int V = (1 << 24) - 1;                       // |acc| < 2^24 always
+    auto idx = [&](int v) { return level_index_of_y(fmaf((float)v * sigma, s, t), q); };
+    if (idx(-V) >= j) return -INFINITY;
+    if (idx(V) < j) return INFINITY;
+    int lo = -V, hi = V;                               // idx(lo) < j <= idx(hi)
+    while (hi - lo > 1) {
+        const int mid = lo + ((hi - lo) >> 1);
+        if (idx(mid) >= j) hi = mid; else lo = mid;
+    }
+    return (float)hi;
+}
+
 // Breakpoints of channel o: T[0 .. n-2] and sigma, written to out[0 .. n-1].
 __device__ __forceinline__ void channel_thresholds(float s, float t, const QParams &q, float *out) {
-    const float sigma = (s < 0.0f) ? -1.0f : 1.0f;
     const int n = num_levels(q.bits);
-    const int V = (1 << 24) - 1;                       // |acc| < 2^24 always
-    for (int j = 1; j < n; ++j) {
-        auto idx = [&](int v) { return level_index_of_y(fmaf((float)v * sigma, s, t), q); };
-        float T;
-        if (idx(-V) >= j) {
-            T = -INFINITY;
-        } else if (idx(V) < j) {
-            T = INFINITY;
-        } else {
-            int lo = -V, hi = V;                       // idx(lo) < j <= idx(hi)
-            while (hi - lo > 1) {
-                const int mid = lo + ((hi - lo) >> 1);
-                if (idx(mid) >= j) hi = mid; else lo = mid;
-            }
-            T = (float)hi;
-        }
-        out[j - 1] = T;
-    }
-    out[n - 1] = sigma;
+    for (int j = 1; j < n; ++j) out[j - 1] = channel_threshold(s, t, q, j);
+    out[n - 1] = (s < 0.0f) ? -1.0f : 1.0f;
 }
 
 // The same breakpoints for an fp32 accumulator (the first layer, whose input
@@ -188,6 +185,27 @@ __device__ __forceinline__ void channel_thresholds_f32(float s, float t, const Q
         out[j - 1] = T;
     }
     out[n - 1] = sigma;
+}
+
+// The breakpoint T_j of the quantizer on y itself (scale 1, shift 0) by a whole warp: 32 candidates a
+// round, so seven rounds instead of 32 (a search by one thread held a 128-channel block's first tile for
+// 20 us).  Every lane returns it.
+__device__ __forceinline__ float y_threshold_warp(const QParams &q, int j) {
+    const int V = 0x7F7FFFFF;
+    auto idx = [&](int k) { return level_index_of_y(f32_from_order(k), q); };
+    if (idx(-V) >= j) return -INFINITY;
+    if (idx(V) < j) return INFINITY;
+    long long lo = -(long long)V, hi = V;                     // idx(lo) < j <= idx(hi)
+    while (hi - lo > 1) {
+        const long long step = (hi - lo + 32) / 33;           // lo + 33 step >= hi
+        const long long c = lo + ((threadIdx.x & 31) + 1) * step;
+        const uint32_t m = __ballot_sync(0xffffffffu, c >= hi || idx((int)c) >= j);
+        const int f = m ? __ffs(m) - 1 : 32;                  // first candidate at or past the breakpoint
+        const long long nh = lo + (f + 1) * step;
+        if (f < 32 && nh < hi) hi = nh;
+        lo += f * step;
+    }
+    return f32_from_order((int)hi);
 }
 
 // Level index of an accumulator (exact integer held in fp32) from the

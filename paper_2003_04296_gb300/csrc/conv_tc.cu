@@ -1052,10 +1052,11 @@ __global__ void __launch_bounds__(NT, 1)
                     sthr[u * O32 + o] = (u == NL - 1) ? x : mask_breakpoint(x);
                 }
             } else {
-                for (int o = et; o < p.O; o += EPI_WARPS * 32) {
-                    float t[8];
-                    channel_thresholds(__ldg(p.scale + o), __ldg(p.shift + o), p.qo, t);
-                    for (int u = 0; u < NL; ++u) sthr[u * O32 + o] = (u == NL - 1) ? t[u] : mask_breakpoint(t[u]);
+                for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {      // one breakpoint (or sigma) per thread
+                    const int o = i / NL, u = i - o * NL;
+                    const float sc = __ldg(p.scale + o);
+                    sthr[u * O32 + o] = (u == NL - 1) ? (sc < 0.0f ? -1.0f : 1.0f)
+                                                      : mask_breakpoint(channel_threshold(sc, __ldg(p.shift + o), p.qo, u + 1));
                 }
             }
             for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
@@ -1063,13 +1064,19 @@ __global__ void __launch_bounds__(NT, 1)
                 sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
             }
             if (resid) {                                        // level of y = #{u : y >= T_u}
+                float *yt = reinterpret_cast<float *>(tmem_slot + 1);        // T_1 .. T_{n-1}
+                const int w8 = warp - 2;
+                if (w8 < NL - 1) {
+                    const float T = p.ythr != nullptr ? __ldg(p.ythr + w8) : y_threshold_warp(p.qo, w8 + 1);
+                    if (lane == 0) yt[w8] = T;
+                }
+                asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");
                 if (et == 0) {
                     float t[8];
-                    if (p.ythr != nullptr)
-                        for (int u = 0; u < NL - 1; ++u) t[u] = __ldg(p.ythr + u);
-                    else
-                        channel_thresholds_f32(1.0f, 0.0f, p.qo, t);     // a long serial search: callers cache it
-                    for (int u = 0; u < NL - 1; ++u) syt[u] = mask_breakpoint(t[u]);
+                    for (int u = 0; u < NL - 1; ++u) {
+                        t[u] = yt[u];
+                        syt[u] = mask_breakpoint(t[u]);
+                    }
                     // the breakpoint below level index 3 - e is the next fp32 value above -(that of 3 + e)
                     bool sym = NL == 7;
                     if constexpr (NL == 7)
