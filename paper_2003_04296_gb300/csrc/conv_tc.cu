@@ -36,6 +36,7 @@
 #include <stdint.h>
 #include <stdlib.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "kernels.cuh"
@@ -377,6 +378,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
+// Eight columns of this warp's 32 TMEM lanes.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 
@@ -478,23 +487,69 @@ __device__ __forceinline__ void mask_chunk_regs(const uint32_t (&v)[32], bool fu
     store_level_masks<OUTB>(M, nvalid, full32 ? 32 : 16, planes, NWo, codes, codes4);
 }
 
-template <int OUTB>
+// 2- and 3-bit outputs go eight columns at a time in a loop that is not
+// unrolled, last columns first (a mask's bits shift up): straight-line code
+// for 32 columns of six masks is fetched anew by every warp, and fetching it
+// took longer than running it.
+template <int OUTB, bool ROLL = (OUTB > 1)>
 __device__ __forceinline__ void mask_chunk(uint32_t taddr, bool full32, const float *th, int tstride, uint32_t sig,
                                            int pool, int bw, bool writer, int nvalid, uint32_t *planes, int NWo,
                                            uint8_t *codes, bool codes4) {
-    uint32_t v[32];
-    if (full32) {
-        tmem_ld32(taddr, v);
-    } else {
-        uint32_t v16[16];
-        tmem_ld16(taddr, v16);
+    if constexpr (!ROLL) {
+        uint32_t v[32];
+        if (full32) {
+            tmem_ld32(taddr, v);
+        } else {
+            uint32_t v16[16];
+            tmem_ld16(taddr, v16);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            v[j] = v16[j];
-            v[j + 16] = 0u;
+            for (int j = 0; j < 16; ++j) {
+                v[j] = v16[j];
+                v[j + 16] = 0u;
+            }
         }
+        mask_chunk_regs<OUTB>(v, full32, th, tstride, sig, pool, bw, writer, nvalid, planes, NWo, codes, codes4);
+    } else {
+        constexpr int NL = OUTB == 1 ? 2 : OUTB == 2 ? 3 : 7;
+        uint32_t M[NL - 1];
+#pragma unroll
+        for (int u = 0; u < NL - 1; ++u) M[u] = 0u;
+#pragma unroll 1
+        for (int g = full32 ? 3 : 1; g >= 0; --g) {
+            uint32_t v[8];
+            tmem_ld8(taddr + 8u * (uint32_t)g, v);
+#pragma unroll
+            for (int j4 = 1; j4 >= 0; --j4) {
+                const float *t4 = th + 8 * g + 4 * j4;
+                const float4 sg4 = *reinterpret_cast<const float4 *>(t4 + (NL - 1) * tstride);
+                float4 nt4[NL - 1];
+#pragma unroll
+                for (int u = 0; u < NL - 1; ++u) nt4[u] = *reinterpret_cast<const float4 *>(t4 + u * tstride);
+                const float sg[4] = {sg4.x, sg4.y, sg4.z, sg4.w};
+#pragma unroll
+                for (int jj = 3; jj >= 0; --jj) {
+                    const float a = __uint_as_float(v[4 * j4 + jj]);
+#pragma unroll
+                    for (int u = 0; u < NL - 1; ++u) {
+                        const float nt = jj == 0 ? nt4[u].x : jj == 1 ? nt4[u].y : jj == 2 ? nt4[u].z : nt4[u].w;
+                        M[u] = __funnelshift_l(__float_as_uint(fmaf(a, sg[jj], nt)), M[u], 1);
+                    }
+                }
+            }
+        }
+        if (pool) {
+#pragma unroll
+            for (int u = 0; u < NL - 1; ++u) {
+                const uint32_t m = M[u];
+                const uint32_t n1 = __shfl_xor_sync(0xffffffffu, m, 1);
+                const uint32_t a1 = m & n1, o1 = m | n1;
+                const uint32_t a2 = a1 & __shfl_xor_sync(0xffffffffu, a1, bw);
+                const uint32_t o2 = o1 | __shfl_xor_sync(0xffffffffu, o1, bw);
+                M[u] = (sig & a2) | (~sig & o2);
+            }
+        }
+        if (writer) store_level_masks<OUTB>(M, nvalid, full32 ? 32 : 16, planes, NWo, codes, codes4);
     }
-    mask_chunk_regs<OUTB>(v, full32, th, tstride, sig, pool, bw, writer, nvalid, planes, NWo, codes, codes4);
 }
 
 // The shortcut's level codes of 32 channels of one pixel (16 bytes of E2M1
@@ -543,98 +598,104 @@ __device__ __forceinline__ float2 res_pair_e4m3(uint32_t v) {
 // quantizer whose breakpoints mirror (sym: a level and its negative at
 // opposite y) needs four masks instead of six: |y| against the three positive
 // breakpoints and the sign of y give its planes.
+// Eight columns at a time, last ones first, as in mask_chunk.
 template <int OUTB>
 __device__ __forceinline__ void resid_chunk(uint32_t taddr, bool full32, const Params &p, int ob, long long opix,
                                             bool writer, const float *ssc, const float *ssh, const float *syt, bool sym,
                                             const ResCodes &rc, int NWo) {
-    uint32_t v[32];
-    if (full32) {
-        tmem_ld32(taddr, v);
-    } else {
-        uint32_t v16[16];
-        tmem_ld16(taddr, v16);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            v[j] = v16[j];
-            v[j + 16] = 0u;
-        }
-    }
-    if (!writer) return;
+    constexpr int NL = OUTB == 0 ? 1 : OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7);
     const int nvalid = min(32, p.O - ob);                 // a multiple of 16
     const int ncol = full32 ? 32 : 16;
-    float y[32];
-#pragma unroll
-    for (int q4 = 0; q4 < 8; ++q4) {
-        const float4 c = *reinterpret_cast<const float4 *>(ssc + ob + 4 * q4);
-        const float4 h = *reinterpret_cast<const float4 *>(ssh + ob + 4 * q4);
-        y[4 * q4] = fmaf(__uint_as_float(v[4 * q4]), c.x, h.x);
-        y[4 * q4 + 1] = fmaf(__uint_as_float(v[4 * q4 + 1]), c.y, h.y);
-        y[4 * q4 + 2] = fmaf(__uint_as_float(v[4 * q4 + 2]), c.z, h.z);
-        y[4 * q4 + 3] = fmaf(__uint_as_float(v[4 * q4 + 3]), c.w, h.w);
-    }
     const long long base = opix * p.O + ob;
-    if (p.y_nhwc != nullptr) {
-        float4 *dst = reinterpret_cast<float4 *>(p.y_nhwc + base);
+    uint32_t M[NL];                                       // NL - 1 masks, or |y| below levels 1, 2, 4 and y < 0
 #pragma unroll
-        for (int q4 = 0; q4 < 8; ++q4)
-            if (q4 * 4 < nvalid && q4 * 4 < ncol) dst[q4] = make_float4(y[4 * q4], y[4 * q4 + 1], y[4 * q4 + 2], y[4 * q4 + 3]);
+    for (int u = 0; u < NL; ++u) M[u] = 0u;
+    float nt[NL];
+#pragma unroll
+    for (int u = 0; u < NL - 1; ++u) nt[u] = OUTB > 0 ? syt[u] : 0.0f;
+    // this group's codes: the last eight channels' bytes, moved up group by group
+    uint32_t c0 = rc.lo.x, c1 = rc.lo.y, c2 = rc.lo.z, c3 = rc.lo.w, d0 = rc.hi.x, d1 = rc.hi.y, d2 = rc.hi.z,
+             d3 = rc.hi.w;
+    if (!full32) {                                        // 16 columns: their codes sit in the first half
+        if (p.res4) {
+            c3 = c1;
+            c2 = c0;
+        } else {
+            d3 = c3; d2 = c2; d1 = c1; d0 = c0;
+        }
+    }
+#pragma unroll 1
+    for (int g = full32 ? 3 : 1; g >= 0; --g) {
+        uint32_t v[8];
+        __syncwarp();
+        tmem_ld8(taddr + 8u * (uint32_t)g, v);
+        float y[8];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float4 c = *reinterpret_cast<const float4 *>(ssc + ob + 8 * g + 4 * k);
+            const float4 h = *reinterpret_cast<const float4 *>(ssh + ob + 8 * g + 4 * k);
+            y[4 * k] = fmaf(__uint_as_float(v[4 * k]), c.x, h.x);
+            y[4 * k + 1] = fmaf(__uint_as_float(v[4 * k + 1]), c.y, h.y);
+            y[4 * k + 2] = fmaf(__uint_as_float(v[4 * k + 2]), c.z, h.z);
+            y[4 * k + 3] = fmaf(__uint_as_float(v[4 * k + 3]), c.w, h.w);
+        }
+        const bool live = writer && 8 * g < nvalid;
+        if (p.y_nhwc != nullptr && live) {
+            float4 *dst = reinterpret_cast<float4 *>(p.y_nhwc + base + 8 * g);
+            dst[0] = make_float4(y[0], y[1], y[2], y[3]);
+            dst[1] = make_float4(y[4], y[5], y[6], y[7]);
+        }
+        if constexpr (OUTB > 0) {
+            if (p.res_codes != nullptr && p.res4) {
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const float2 r = res_pair_e2m1(c3 >> (4 * j));
+                    y[j] = fmaf(r.x, p.res_unit, y[j]);
+                    y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
+                }
+                c3 = c2; c2 = c1; c1 = c0;
+            } else if (p.res_codes != nullptr) {
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const float2 r = res_pair_e4m3((j < 4 ? d2 : d3) >> (8 * (j & 3)));
+                    y[j] = fmaf(r.x, p.res_unit, y[j]);
+                    y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
+                }
+                d3 = d1; d2 = d0; d1 = c3; d0 = c2; c3 = c1; c2 = c0;
+            } else if (p.res_f32 != nullptr && live) {
+                const float4 *src = reinterpret_cast<const float4 *>(p.res_f32 + base + 8 * g);
+                const float4 a = __ldg(src), b = __ldg(src + 1);
+                y[0] += a.x; y[1] += a.y; y[2] += a.z; y[3] += a.w;
+                y[4] += b.x; y[5] += b.y; y[6] += b.z; y[7] += b.w;
+            }
+            if (OUTB == 3 && sym) {
+#pragma unroll
+                for (int j = 7; j >= 0; --j) {
+                    M[0] = __funnelshift_l(__float_as_uint(fabsf(y[j]) + nt[NL > 3 ? 3 : 0]), M[0], 1);
+                    M[1] = __funnelshift_l(__float_as_uint(fabsf(y[j]) + nt[NL > 4 ? 4 : 0]), M[1], 1);
+                    M[NL > 2 ? 2 : 0] = __funnelshift_l(__float_as_uint(fabsf(y[j]) + nt[NL > 5 ? 5 : 0]), M[NL > 2 ? 2 : 0], 1);
+                    M[NL > 3 ? 3 : 0] = __funnelshift_l(__float_as_uint(y[j]), M[NL > 3 ? 3 : 0], 1);
+                }
+            } else {
+#pragma unroll
+                for (int j = 7; j >= 0; --j)
+#pragma unroll
+                    for (int u = 0; u < NL - 1; ++u) M[u] = __funnelshift_l(__float_as_uint(y[j] + nt[u]), M[u], 1);
+            }
+        }
     }
     if constexpr (OUTB > 0) {
-        if (p.res_codes != nullptr && p.res4) {
-            const uint32_t cw[4] = {rc.lo.x, rc.lo.y, rc.lo.z, rc.lo.w};
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-                const float2 r = res_pair_e2m1(cw[j >> 3] >> (4 * (j & 7)));
-                y[j] = fmaf(r.x, p.res_unit, y[j]);
-                y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
-            }
-        } else if (p.res_codes != nullptr) {
-            const uint32_t cw[8] = {rc.lo.x, rc.lo.y, rc.lo.z, rc.lo.w, rc.hi.x, rc.hi.y, rc.hi.z, rc.hi.w};
-#pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-                const float2 r = res_pair_e4m3(cw[j >> 2] >> (8 * (j & 3)));
-                y[j] = fmaf(r.x, p.res_unit, y[j]);
-                y[j + 1] = fmaf(r.y, p.res_unit, y[j + 1]);
-            }
-        } else if (p.res_f32 != nullptr) {
-            const float4 *src = reinterpret_cast<const float4 *>(p.res_f32 + base);
-#pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4) {
-                if (q4 * 4 >= nvalid || q4 * 4 >= ncol) break;
-                const float4 r = __ldg(src + q4);
-                y[4 * q4] += r.x;
-                y[4 * q4 + 1] += r.y;
-                y[4 * q4 + 2] += r.z;
-                y[4 * q4 + 3] += r.w;
-            }
-        }
-        constexpr int NL = OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7);
+        if (!writer) return;
         uint32_t *planes = p.planes_out ? p.planes_out + (opix * OUTB) * NWo + (ob >> 5) : nullptr;
         uint8_t *codes = p.codes_out ? p.codes_out + (p.out4 ? base / 2 : base) : nullptr;
-        if (OUTB == 3 && sym) {
-            const float t1 = syt[3], t2 = syt[4], t3 = syt[5];       // -T of levels 1, 2 and 4 (units)
-            uint32_t n1 = 0u, n2 = 0u, n3 = 0u, ng = 0u;             // |y| below each; y below zero
-#pragma unroll
-            for (int j = 31; j >= 0; --j) {
-                n1 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t1), n1, 1);
-                n2 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t2), n2, 1);
-                n3 = __funnelshift_l(__float_as_uint(fabsf(y[j]) + t3), n3, 1);
-                ng = __funnelshift_l(__float_as_uint(y[j]), ng, 1);
+        if constexpr (OUTB == 3) {
+            if (sym) {
+                const uint32_t n1 = M[0], n2 = M[1], n3 = M[2], ng = M[3];
+                const uint32_t P[3] = {ng & ~n1, ~n1 & (n2 | ~n3), ~n2};
+                store_level_planes<3>(P, nvalid, ncol, planes, NWo, codes, p.out4 != 0);
+                return;
             }
-            const uint32_t P[3] = {ng & ~n1, ~n1 & (n2 | ~n3), ~n2};
-            store_level_planes<3>(P, nvalid, ncol, planes, NWo, codes, p.out4 != 0);
-            return;
         }
-        float nt[NL - 1];
-#pragma unroll
-        for (int u = 0; u < NL - 1; ++u) nt[u] = syt[u];
-        uint32_t M[NL - 1];
-#pragma unroll
-        for (int u = 0; u < NL - 1; ++u) M[u] = 0u;
-#pragma unroll
-        for (int j = 31; j >= 0; --j)
-#pragma unroll
-            for (int u = 0; u < NL - 1; ++u) M[u] = __funnelshift_l(__float_as_uint(y[j] + nt[u]), M[u], 1);
         store_level_masks<OUTB>(M, nvalid, ncol, planes, NWo, codes, p.out4 != 0);
     }
 }
@@ -741,6 +802,79 @@ __device__ __forceinline__ void rows_store16(uint32_t *sw, const uint32_t (&u)[1
                 if (c + 2 < ncols) d[2] = x.z;
                 if (c + 3 < ncols) d[3] = x.w;
             }
+        }
+    }
+}
+
+// Tables of the epilogue warps (2 .. 9), filled by them all: the output
+// quantizer's breakpoints per channel, its sigma words, and for residual
+// blocks the BN maps and the breakpoints on y.  yt: scratch for T_1 .. T_{n-1}.
+template <int OUTB>
+__device__ __forceinline__ void epi_tables(const Params &p, bool resid, float *sthr, uint32_t *ssig, float *syt, float *yt,
+                                           int O32, int thr_floats, int sig_words, int et, int warp, int lane) {
+    constexpr int NL = OUTB == 0 ? 1 : (OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7));
+    // output-quantizer breakpoints of every channel, in shared memory
+    if constexpr (OUTB > 0) {
+        // held as (-T_1 .. -T_{n-1}, sigma) with -0 stored as +0, so that
+        // fmaf(acc, sigma, -T) is never -0 and its sign bit is [sigma * acc < T]
+        // rows u = 0 .. NL - 1 of O32 channels each (channel fastest: four channels per 128-bit load)
+        if (resid) {
+            // a residual block quantizes y + shortcut: no per-channel breakpoints on acc
+        } else if (p.thr != nullptr) {
+            for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {
+                const float x = __ldg(p.thr + i);
+                const int o = i / NL, u = i - o * NL;
+                sthr[u * O32 + o] = (u == NL - 1) ? x : mask_breakpoint(x);
+            }
+        } else {
+            for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {      // one breakpoint (or sigma) per thread
+                const int o = i / NL, u = i - o * NL;
+                const float sc = __ldg(p.scale + o);
+                sthr[u * O32 + o] = (u == NL - 1) ? (sc < 0.0f ? -1.0f : 1.0f)
+                                                  : mask_breakpoint(channel_threshold(sc, __ldg(p.shift + o), p.qo, u + 1));
+            }
+        }
+        for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
+            const int k = i - p.O * NL, o = p.O + k / NL, u = k % NL;
+            sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
+        }
+        if (resid) {                                        // level of y = #{u : y >= T_u}
+            const int w8 = warp - 2;
+            if (w8 < NL - 1) {
+                const float T = p.ythr != nullptr ? __ldg(p.ythr + w8) : y_threshold_warp(p.qo, w8 + 1);
+                if (lane == 0) yt[w8] = T;
+            }
+            asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");
+            if (et == 0) {
+                float t[8];
+                for (int u = 0; u < NL - 1; ++u) {
+                    t[u] = yt[u];
+                    syt[u] = mask_breakpoint(t[u]);
+                }
+                // the breakpoint below level index 3 - e is the next fp32 value above -(that of 3 + e)
+                bool sym = NL == 7;
+                if constexpr (NL == 7)
+                    for (int e = 0; e < 3; ++e)
+                        sym = sym && t[3 + e] > 0.0f && isfinite(t[3 + e]) &&
+                              t[2 - e] == __uint_as_float(__float_as_uint(-t[3 + e]) - 1u);
+                syt[7] = sym ? 1.0f : 0.0f;
+            }
+        }
+        // sigma of a channel: the sign of its BN scale (+1 for 0); one warp per
+        // 32-channel word, a lane per channel (one load latency for the word)
+        for (int g = warp - 2; g < sig_words; g += EPI_WARPS) {
+            const int o = g * 32 + lane;
+            const float sg = o < p.O ? (p.thr != nullptr ? __ldg(p.thr + o * NL + NL - 1)
+                                                         : (__ldg(p.scale + o) < 0.0f ? -1.0f : 1.0f))
+                                     : 1.0f;
+            const uint32_t m = __ballot_sync(0xffffffffu, sg > 0.0f);
+            if (lane == 0) ssig[g] = m;
+        }
+    }
+    if (resid) {
+        for (int o = et; o < O32; o += EPI_WARPS * 32) {
+            sthr[o] = o < p.O ? __ldg(p.scale + o) : 0.0f;
+            sthr[O32 + o] = o < p.O ? __ldg(p.shift + o) : 0.0f;
         }
     }
 }
@@ -1038,71 +1172,8 @@ __global__ void __launch_bounds__(NT, 1)
                 }
             }
         }
-        // output-quantizer breakpoints of every channel, in shared memory
-        if constexpr (OUTB > 0) {
-            // held as (-T_1 .. -T_{n-1}, sigma) with -0 stored as +0, so that
-            // fmaf(acc, sigma, -T) is never -0 and its sign bit is [sigma * acc < T]
-            // rows u = 0 .. NL - 1 of O32 channels each (channel fastest: four channels per 128-bit load)
-            if (resid) {
-                // a residual block quantizes y + shortcut: no per-channel breakpoints on acc
-            } else if (p.thr != nullptr) {
-                for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {
-                    const float x = __ldg(p.thr + i);
-                    const int o = i / NL, u = i - o * NL;
-                    sthr[u * O32 + o] = (u == NL - 1) ? x : mask_breakpoint(x);
-                }
-            } else {
-                for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {      // one breakpoint (or sigma) per thread
-                    const int o = i / NL, u = i - o * NL;
-                    const float sc = __ldg(p.scale + o);
-                    sthr[u * O32 + o] = (u == NL - 1) ? (sc < 0.0f ? -1.0f : 1.0f)
-                                                      : mask_breakpoint(channel_threshold(sc, __ldg(p.shift + o), p.qo, u + 1));
-                }
-            }
-            for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
-                const int k = i - p.O * NL, o = p.O + k / NL, u = k % NL;
-                sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
-            }
-            if (resid) {                                        // level of y = #{u : y >= T_u}
-                float *yt = reinterpret_cast<float *>(tmem_slot + 1);        // T_1 .. T_{n-1}
-                const int w8 = warp - 2;
-                if (w8 < NL - 1) {
-                    const float T = p.ythr != nullptr ? __ldg(p.ythr + w8) : y_threshold_warp(p.qo, w8 + 1);
-                    if (lane == 0) yt[w8] = T;
-                }
-                asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");
-                if (et == 0) {
-                    float t[8];
-                    for (int u = 0; u < NL - 1; ++u) {
-                        t[u] = yt[u];
-                        syt[u] = mask_breakpoint(t[u]);
-                    }
-                    // the breakpoint below level index 3 - e is the next fp32 value above -(that of 3 + e)
-                    bool sym = NL == 7;
-                    if constexpr (NL == 7)
-                        for (int e = 0; e < 3; ++e)
-                            sym = sym && t[3 + e] > 0.0f && isfinite(t[3 + e]) &&
-                                  t[2 - e] == __uint_as_float(__float_as_uint(-t[3 + e]) - 1u);
-                    syt[7] = sym ? 1.0f : 0.0f;
-                }
-            }
-            // sigma of a channel: the sign of its BN scale (+1 for 0); one warp per
-            // 32-channel word, a lane per channel (one load latency for the word)
-            for (int g = warp - 2; g < sig_words; g += EPI_WARPS) {
-                const int o = g * 32 + lane;
-                const float sg = o < p.O ? (p.thr != nullptr ? __ldg(p.thr + o * NL + NL - 1)
-                                                             : (__ldg(p.scale + o) < 0.0f ? -1.0f : 1.0f))
-                                         : 1.0f;
-                const uint32_t m = __ballot_sync(0xffffffffu, sg > 0.0f);
-                if (lane == 0) ssig[g] = m;
-            }
-        }
-        if (resid) {
-            for (int o = et; o < O32; o += EPI_WARPS * 32) {
-                sthr[o] = o < p.O ? __ldg(p.scale + o) : 0.0f;
-                sthr[O32 + o] = o < p.O ? __ldg(p.shift + o) : 0.0f;
-            }
-        }
+        epi_tables<OUTB>(p, resid, sthr, ssig, syt, reinterpret_cast<float *>(tmem_slot + 1), O32, thr_floats, sig_words, et,
+                         warp, lane);
         asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");   // breakpoints in place
         pdl_wait();                               // outputs, shortcuts and partial sums are shared with other kernels
         const int q = warp & 3;                   // TMEM lane quarter of this warp
@@ -1617,6 +1688,211 @@ __global__ void __launch_bounds__(NT, 1)
     }
 }
 
+// ---------------------------------------------------------------------------
+// 3 x 3, stride 1, pad 1 on tiles with their halo: the input of a 16 x 8-pixel
+// tile crosses the TMA unit once, as a box of 18 x 10 pixels, instead of once
+// per tap (180 rows of 64 or 128 bytes against 1152, at 3 to 4 cycles a row
+// what bounds conv_tc_kernel on 64- and 128-channel layers), and the weights
+// of the CTA's channel tile stay in shared memory.  Tap (dy, dx) of the tile
+// is the box at a start address (10 dy + dx) rows on: eight pixels of an
+// image row are an 8-row group of the MMA operand, the next image row is the
+// next group (stride 10 rows), and the swizzle, a function of the address
+// alone, is the same for the TMA's writes and the MMA's reads at any start.
+// Two or three accumulators: an epilogue overlaps the next tiles' MMAs.
+// Roles (576 threads): warp 0 TMA, warp 1 MMA, warps 2-17 epilogue in two sets
+// of eight that take the tiles in turn (the epilogue's dependent instructions
+// set these layers' time: eight warps issued 1.7 a clock), a pixel's channels
+// per lane (pool windows sit in lanes l, l ^ 1, l ^ 8, l ^ 9).
+// ---------------------------------------------------------------------------
+namespace halo {
+constexpr int SETS = 2;
+constexpr int NT = 32 * (2 + SETS * EPI_WARPS);
+constexpr int BX = 10, BY = 18;            // box pixels
+constexpr int NACC = 3;
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
+}  // namespace halo
+
+template <int OUTB, int FMT>
+__global__ void __launch_bounds__(halo::NT, 1)
+    conv_halo_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ Params p) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    constexpr int NL = OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7);
+    const int O32 = (p.O + 31) & ~31;
+    const bool resid = p.res_codes != nullptr || p.res_f32 != nullptr;
+    uint8_t *wres = smem + (size_t)p.S * p.stage_bytes;
+    float *sthr = reinterpret_cast<float *>(wres + (size_t)p.nk * p.b_bytes);
+    const int thr_floats = O32 * NL, sig_words = O32 / 32;
+    uint32_t *ssig = reinterpret_cast<uint32_t *>(sthr + thr_floats);
+    float *syt = reinterpret_cast<float *>(ssig + ((sig_words + 1) & ~1));
+    __shared__ uint64_t full[8], empty[8], tfull[halo::NACC], tempty[halo::NACC], wfull, sfready, tstall;
+    __shared__ uint32_t tmem_slot;
+    __shared__ float yt[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int i = 0; i < halo::NACC; ++i) {
+            mbar_init(&tfull[i], 1);
+            mbar_init(&tempty[i], EPI_WARPS);
+        }
+        mbar_init(&wfull, 1);
+        mbar_init(&sfready, 4);
+        mbar_init(&tstall, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(&tmem_slot)));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    pdl_trigger();
+    // unit u keeps channel tile u % ntn and walks pixel tiles u / ntn, + units per channel tile, ...
+    const int tiles = p.nbx * p.nby * p.nbb, upt = (int)gridDim.x / p.ntn;
+    const int tn = (int)blockIdx.x % p.ntn, t0 = (int)blockIdx.x / p.ntn;
+    const int o0 = tn * p.BN;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
+            // a network's weights (its breakpoints are precomputed too) were written long ago; a standalone
+            // call's may come from the kernel before
+            if (p.thr == nullptr) pdl_wait();
+            mbar_expect_tx(&wfull, (uint32_t)p.nk * p.b_bytes);
+            for (int k = 0; k < p.nk; ++k) tma_load_2d(wres + (size_t)k * p.b_bytes, &tmB, &wfull, k * p.cb, o0);
+            if (p.thr != nullptr) pdl_wait();
+            int s = 0, lap = 0, g = 0;
+            for (int t = t0; t < tiles; t += upt, ++g) {
+                if (lap > 0 && !mbar_wait(&empty[s], (lap - 1) & 1, p.wait_cycles)) break;
+                const int xb = t % p.nbx, yb = (t / p.nbx) % p.nby, b = t / (p.nbx * p.nby);
+                mbar_expect_tx(&full[s], p.a_bytes);
+                tma_load_4d(smem + (size_t)s * p.stage_bytes, &tmA, &full[s], 0, xb * 8 - 1, yb * 16 - 1, b);
+                if (++s == p.S) { s = 0; ++lap; }
+            }
+            for (int j = g > p.S ? g - p.S : 0; j < g; ++j)       // every load has landed before the CTA can exit
+                if (!mbar_wait(&full[j % p.S], (j / p.S) & 1, p.wait_cycles)) break;
+            mbar_wait(&wfull, 0u, p.wait_cycles);
+        }
+    } else if (warp == 1) {
+        bool alive = true;
+        if (p.stall && !__all_sync(0xffffffffu, mbar_wait(&tstall, 0u, p.wait_cycles))) alive = false;
+        if (FMT == 2 && alive && !__all_sync(0xffffffffu, mbar_wait(&sfready, 0u, p.wait_cycles))) alive = false;
+        if (alive && !__all_sync(0xffffffffu, mbar_wait(&wfull, 0u, p.wait_cycles))) alive = false;
+        fence_after();
+        const uint32_t sfa = tmem_base + p.sf_col, sfb = sfa + 32u;
+        // unrolled over the taps and the K steps of a row (p.cb = 32 NJ bytes), so that every descriptor is a
+        // uniform base plus a constant: with a runtime loop each MMA took about 210 cycles to issue
+        auto run = [&](auto nj_) {
+            constexpr int NJ = decltype(nj_)::value, CB = 32 * NJ;
+            // operand groups of eight pixels lie ten pixels apart
+            const uint64_t strip = ~((uint64_t)0x3FFF << 32), sbo = (uint64_t)((halo::BX * CB) >> 4) << 32;
+            const uint64_t ad0 = (sw_desc(smem_u32(smem), CB) & strip) | sbo, bd0 = sw_desc(smem_u32(wres), CB);
+            const uint32_t bstep = p.b_bytes >> 4, idesc = p.idesc;
+            int s = 0, i = 0;
+            uint32_t phase = 0u;
+            for (int t = t0; t < tiles && alive; t += upt, ++i) {
+                const int ab = i % p.nacc, use = i / p.nacc;
+                if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&tempty[ab], (use - 1) & 1, p.wait_cycles))) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(&full[s], phase, p.wait_cycles))) break;
+                fence_after();
+                const uint32_t d = tmem_base + (uint32_t)(ab * p.acc_cols);
+                const uint64_t ad = ad0 + (uint64_t)((uint32_t)s * (p.stage_bytes >> 4));
+                uint64_t bd = bd0;
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap) {
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j) {
+                        const uint64_t a_ = ad + (uint64_t)((halo::BX * (tap / 3) + tap % 3) * (CB >> 4) + 2 * j);
+                        if constexpr (FMT == 2)
+                            mma_f4(d, a_, bd + 2u * j, idesc, tap + j > 0 ? 1u : 0u, sfa, sfb);
+                        else
+                            mma_f8(d, a_, bd + 2u * j, idesc, tap + j > 0 ? 1u : 0u);
+                    }
+                    bd += bstep;
+                }
+                mma_commit(&empty[s]);
+                mma_commit(&tfull[ab]);
+                if (++s == p.S) { s = 0; phase ^= 1u; }
+            }
+        };
+        if (p.cb == 64) run(halo::Int<2>{});
+        else run(halo::Int<4>{});
+    } else {
+        const int et = threadIdx.x - 64;
+        if constexpr (FMT == 2) {
+            if (warp < 6) {                                      // unit scale factors, as in conv_tc_kernel
+                const uint32_t ta = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + p.sf_col;
+#pragma unroll
+                for (int c = 0; c < 64; c += 8)
+                    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};\n" ::"r"(
+                                     ta + (uint32_t)c),
+                                 "r"(0x7F7F7F7Fu));
+                asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sfready);
+            }
+        }
+        const int set = (warp - 2) / EPI_WARPS;
+        if (set == 0) epi_tables<OUTB>(p, resid, sthr, ssig, syt, yt, O32, thr_floats, sig_words, et, warp, lane);
+        asm volatile("bar.sync 2, %0;\n" ::"n"(halo::SETS * EPI_WARPS * 32) : "memory");
+        pdl_wait();
+        const int q = warp & 3, half = ((warp - 2) >> 2) & 1, r = q * 32 + lane;
+        const int Hp = p.pool ? p.Ho / 2 : p.Ho, Wp = p.pool ? p.Wo / 2 : p.Wo, NWo = (p.O + 31) >> 5;
+        const int nch = p.BN >> 5, cmid = (nch + 1) >> 1, cbeg = half ? cmid : 0, cend = half ? nch : cmid;
+        const bool rcodes = p.res_codes != nullptr, sym = OUTB == 3 && resid && syt[7] != 0.0f;
+        int i = 0;
+        bool dead = false;
+        for (int t = t0; t < tiles; t += upt, ++i) {
+            if (i % halo::SETS != set) continue;
+            const int ab = i % p.nacc, use = i / p.nacc;
+            const int xb = t % p.nbx, yb = (t / p.nbx) % p.nby, b = t / (p.nbx * p.nby);
+            const int y = yb * 16 + (r >> 3), x = xb * 8 + (r & 7);
+            const bool valid = y < p.Ho && x < p.Wo;
+            const bool writer = valid && (!p.pool || ((x & 1) == 0 && (y & 1) == 0));
+            const long long opix = ((long long)b * Hp + (p.pool ? y >> 1 : y)) * Wp + (p.pool ? x >> 1 : x);
+            ResCodes rc{};
+            if (rcodes && cbeg < cend) rc = load_res_codes(p, o0 + cbeg * 32, opix, writer, true);
+            if (!dead && !mbar_wait(&tfull[ab], use & 1, p.wait_cycles)) dead = true;
+            fence_after();
+            for (int c = cbeg; c < cend && !dead; ++c) {
+                const int ob = o0 + c * 32;
+                if (ob >= p.O) break;
+                const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * p.acc_cols + c * 32);
+                if (resid) {
+                    ResCodes nx{};
+                    if (rcodes && c + 1 < cend) nx = load_res_codes(p, ob + 32, opix, writer, true);
+                    __syncwarp();
+                    resid_chunk<OUTB>(ta, true, p, ob, opix, writer, sthr, sthr + O32, syt, sym, rc, NWo);
+                    rc = nx;
+                } else {
+                    __syncwarp();
+                    mask_chunk<OUTB, true>(ta, true, sthr + ob, O32, p.pool ? ssig[ob >> 5] : 0u, p.pool, 8, writer, p.O - ob,
+                                     p.planes_out ? p.planes_out + (opix * OUTB) * NWo + (ob >> 5) : nullptr, NWo,
+                                     p.codes_out ? p.codes_out + ((opix * p.O + ob) >> p.out4) : nullptr, p.out4 != 0);
+                }
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0 && !dead) mbar_arrive(&tempty[ab]);
+        }
+    }
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem_base));
+    }
+}
+
 // Split-K second pass: sums the K slices of every accumulator and runs the
 // block epilogue (no pooling).  Thread = one tile row (output pixel) x four
 // channels; eight consecutive lanes cover 32 channels of one row, so the
@@ -2082,6 +2358,105 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     return MINW_OK;
 }
 
+// The plan of conv_halo_kernel, or false where conv_tc_kernel keeps the layer.
+// It takes 3 x 3 layers of stride 1 and padding 1 on rows of 64 or 128 bytes
+// whose only outputs are levels (with or without a shortcut), where its 16 x 8
+// tiles cover at least MIN_COVER of the computed pixels and give at least
+// MIN_TILES tiles per SM: below that the weights' load and the idle rows
+// outweigh the taps' loads.
+static bool halo_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
+    constexpr double MIN_COVER = 0.6, MIN_TILES = 0.5;
+    if (a.bf16 || a.kh != 3 || a.kw != 3 || a.stride != 1 || a.pad != 1 || !a.quant_out || a.acc_out != nullptr ||
+        a.y_out != nullptr || a.y_nhwc != nullptr || a.n128 || a.pair_n128 || a.upd || a.ksplit > 1 || a.O % 32 != 0)
+        return false;
+    const int rowb = a.fp4 ? a.C / 2 : a.C;
+    if (rowb != 64 && rowb != 128) return false;
+    if (!minw_host::plan_options().channel_major) return false;
+    Params &p = pl.p;
+    p = Params{};
+    p.bw = 8; p.bh = 16; p.bb = 1;
+    p.nbx = (a.Wo + 7) / 8;
+    p.nby = (a.Ho + 15) / 16;
+    p.nbb = a.B;
+    const double cover = (double)a.Wo * a.Ho / ((double)p.nbx * p.nby * 128);
+    p.ntn = (a.O + 127) / 128;
+    if (a.O % p.ntn != 0 || (a.O / p.ntn) % 32 != 0) return false;
+    p.BN = a.O / p.ntn;
+    const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
+    const long long tiles = (long long)p.nbx * p.nby * p.nbb;
+    if (cover < MIN_COVER || (double)tiles * p.ntn < MIN_TILES * sms || tiles >= (1ll << 31)) return false;
+    if (p.ntn > sms) return false;
+    if ((a.res_codes != nullptr || a.res_f32 != nullptr) &&
+        (a.pool || !minw_host::aligned16(a.res_codes) || !minw_host::aligned16(a.res_f32)))
+        return false;
+    p.B = a.B; p.C = a.C; p.H = a.H; p.W = a.W; p.O = a.O; p.kh = 3; p.kw = 3; p.pad = 1;
+    p.Ho = a.Ho; p.Wo = a.Wo; p.stride = 1;
+    p.fp4 = a.fp4 ? 1 : 0;
+    p.out4 = a.codes_out4 ? 1 : 0;
+    p.res4 = a.res_codes4 ? 1 : 0;
+    p.cb = rowb;
+    p.nk = 9;
+    p.ksplit = 1;
+    p.cl = 1;
+    p.a_bytes = (uint32_t)(halo::BX * halo::BY * rowb);
+    p.stage_bytes = (p.a_bytes + 1023u) & ~1023u;
+    p.b_bytes = (uint32_t)(p.BN * rowb);
+    p.nlev = num_levels(a.qo.bits);
+    p.thr = a.thr;
+    p.acc_cols = p.BN;
+    p.tmem_cols = 512;
+    // accumulators below the E2M1 scale factors at column 448
+    p.sf_col = 448;
+    p.nacc = std::min(halo::NACC, 448 / p.BN);
+    p.idesc = p.fp4 ? (1u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | (1u << 23) | (8u << 24)
+                    : (1u << 4) | ((uint32_t)(p.BN >> 3) << 17) | (8u << 24);
+    p.scale = a.scale; p.shift = a.shift;
+    p.pool = a.pool; p.quant_out = 1; p.qo = a.qo;
+    p.planes_out = a.planes_out; p.codes_out = a.codes_out;
+    p.res_codes = a.res_codes; p.res_unit = a.res_unit; p.res_f32 = a.res_f32; p.ythr = a.ythr;
+    const size_t o32 = ((size_t)a.O + 31) & ~(size_t)31;
+    const size_t thr_bytes = (o32 * p.nlev + o32 / 32 + 10) * sizeof(float);
+    const size_t fixed = (size_t)p.nk * p.b_bytes + thr_bytes + 1024, limit = 224 * 1024;
+    if (fixed + 2 * (size_t)p.stage_bytes > limit) return false;
+    p.S = (int)std::min<size_t>(8, (limit - fixed) / p.stage_bytes);
+    pl.smem = fixed + (size_t)p.S * p.stage_bytes;
+    if (pl.smem < 120 * 1024) pl.smem = 120 * 1024;           // one CTA (and one tensor-memory allocation) per SM
+    const long long units = std::min<long long>(sms / p.ntn, tiles);
+    pl.grid = dim3((unsigned)(units * p.ntn));
+    pl.thr_ws = nullptr;
+    if (!encode) return true;
+    minw_host::EncodeTiledFn enc = minw_host::tensor_map_encoder();
+    if (enc == nullptr) return false;
+    const CUtensorMapSwizzle swz = rowb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    const cuuint64_t rb = (cuuint64_t)rowb;
+    const cuuint64_t ad[4] = {rb, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
+    const cuuint64_t as[3] = {rb, (cuuint64_t)a.W * rb, (cuuint64_t)a.H * a.W * rb};
+    const cuuint32_t abox[4] = {(cuuint32_t)rowb, halo::BX, halo::BY, 1u}, one[4] = {1u, 1u, 1u, 1u};
+    const cuuint64_t bd[2] = {9 * rb, (cuuint64_t)a.O}, bs[1] = {9 * rb};
+    const cuuint32_t bbox[2] = {(cuuint32_t)rowb, (cuuint32_t)p.BN};
+    return enc(&pl.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<uint8_t *>(a.act8), ad, as, abox, one,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
+           enc(&pl.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(a.wgt8), bd, bs, bbox, one,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+static minw_status launch_halo(const Plan &pl, cudaStream_t s) {
+    typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const Params);
+    static const Kernel kernels[2][3] = {
+        {conv_halo_kernel<1, 0>, conv_halo_kernel<2, 0>, conv_halo_kernel<3, 0>},
+        {conv_halo_kernel<1, 2>, conv_halo_kernel<2, 2>, conv_halo_kernel<3, 2>}};
+    const Kernel kern = kernels[pl.p.fp4][pl.p.qo.bits - 1];
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess)
+        return MINW_ECUDA;
+    Params pm = pl.p;
+    pm.wait_cycles = (long long)minw_host::plan_options().wait_cycles;
+    pm.stall = minw_host::take_stall(MINW_STALL_CONV_TC);
+    return minw_host::launch_pdl(kern, pl.grid, dim3(halo::NT), pl.smem, s, pl.tmA, pl.tmB, pm) == cudaSuccess ? MINW_OK
+                                                                                                              : MINW_ECUDA;
+}
+
 // Resident clusters of cl CTAs for a launch of kern with smem bytes (cached:
 // the answer depends only on these three).
 static int max_active_clusters(const void *kern, int cl, size_t smem, const cudaLaunchConfig_t &cfg) {
@@ -2172,6 +2547,7 @@ bool conv_tc_n128(const ConvArgs &a) {
 int conv_tc_launches(const ConvArgs &a) {
     if (a.workspace == nullptr || a.pool) return 1;
     tc::Plan pl;
+    if (tc::halo_plan(a, pl, false)) return 1;
     if (tc::make_plan(a, pl) != MINW_OK || pl.p.ksplit < 2) return 1;
     // main pass + reduction, plus the breakpoints when the reduction needs them
     return (a.quant_out && a.thr == nullptr && !conv_tc_residual(a)) ? 3 : 2;
@@ -2187,6 +2563,7 @@ minw_status launch_conv_tc(const ConvArgs &a, cudaStream_t s) {
     if (!a.act8 || !a.wgt8) return MINW_EINVAL;
     if (!conv_tc_supported(a)) return MINW_EUNSUPPORTED;
     tc::Plan pl;
+    if (tc::halo_plan(a, pl)) return tc::launch_halo(pl, s);
     minw_status st = tc::make_plan(a, pl);
     if (st != MINW_OK) return st;
     const int outb = a.quant_out ? a.qo.bits : 0;
