@@ -1766,10 +1766,11 @@ __global__ void __launch_bounds__(halo::NT, 1)
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             // a network's weights (its breakpoints are precomputed too) were written long ago; a standalone
             // call's may come from the kernel before
-            if (p.thr == nullptr) pdl_wait();
+            const bool planned = p.thr != nullptr || p.ythr != nullptr;
+            if (!planned) pdl_wait();
             mbar_expect_tx(&wfull, (uint32_t)p.nk * p.b_bytes);
             for (int k = 0; k < p.nk; ++k) tma_load_2d(wres + (size_t)k * p.b_bytes, &tmB, &wfull, k * p.cb, o0);
-            if (p.thr != nullptr) pdl_wait();
+            if (planned) pdl_wait();
             int s = 0, lap = 0, g = 0;
             for (int t = t0; t < tiles; t += upt, ++g) {
                 if (lap > 0 && !mbar_wait(&empty[s], (lap - 1) & 1, p.wait_cycles)) break;

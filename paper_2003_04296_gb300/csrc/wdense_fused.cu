@@ -220,29 +220,46 @@ __global__ void __launch_bounds__(NT, 1) wdense_fused_kernel(const __grid_consta
         uint32_t rph = 0u, hph = 0u;
         const uint32_t rbase = su32(ring);
         // rows ty of a 1x1 convolution with np output columns per tile, tile tx of the rows at column col + tx np
-        auto rows1x1 = [&](const Feat &f, int ty, int cin, uint32_t wbase, int np, uint32_t col) {
+        // (unrolled over the tiles of a row: uniform descriptors plus constants)
+        auto rows_n = [&](auto ntx_, const Feat &f, int ty, int cin, uint32_t wbase, int np, uint32_t col) {
+            constexpr int NTX = decltype(ntx_)::value;
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(np >> 3) << 17) | (8u << 24);
-            const uint64_t bd0 = desc_ns(wbase, (uint32_t)np * 16u, 128u);
-            const uint32_t chunk = (uint32_t)(f.rows(ty) * f.S) * 16u;
-            const int nk = (cin + 15) >> 4, KS = f.ks(), ntx = (f.S + 7) >> 3;
+            uint64_t bd = desc_ns(wbase, (uint32_t)np * 16u, 128u);
+            const uint32_t chunk = (uint32_t)(f.rows(ty) * f.S) * 16u, kstep = chunk >> 3, bstep = 2u * (uint32_t)np;
+            const int nk = (cin + 15) >> 4, KS = f.ks();
+            const uint32_t d = tmem + col;
+            const uint64_t adr = desc_ns(rbase, chunk, (uint32_t)f.S * 16u);
+            uint32_t acc = 0u;
             for (int ks = 0; ks < nk; ks += KS) {
                 const int n = min(KS, nk - ks);
                 warp_wait(&sh.rfull[s], rph, p.wait_cycles, dead);
                 if (!dead) {
                     fence_after();
-                    const uint64_t ad0 = desc_ns(rbase + (uint32_t)s * STAGE_BYTES, chunk, (uint32_t)f.S * 16u);
+                    uint64_t ad = adr + (uint64_t)((uint32_t)s * (STAGE_BYTES >> 4));
                     for (int kk = 0; kk < n; ++kk) {
-                        const uint64_t ad = ad0 + (uint64_t)(((uint32_t)(2 * kk) * chunk) >> 4);
-                        const uint64_t bd = bd0 + (uint64_t)(uint32_t)(2 * (ks + kk) * np);
-                        for (int tx = 0; tx < ntx; ++tx)
-                            mma_bf16(tmem + col + (uint32_t)(tx * np), ad + (uint64_t)(8 * tx), bd, idesc,
-                                     ks + kk > 0 ? 1u : 0u);
+                        uint32_t dt = d;
+#pragma unroll
+                        for (int tx = 0; tx < NTX; ++tx) {
+                            mma_bf16(dt, ad + (uint64_t)(8 * tx), bd, idesc, acc);
+                            dt += (uint32_t)np;
+                        }
+                        acc = 1u;
+                        ad += kstep;
+                        bd += bstep;
                     }
                     mma_commit(&sh.rempty[s]);
                 }
                 if (++s == RING) { s = 0; rph ^= 1u; }
             }
             if (!dead) mma_commit(&sh.hb[ty]);
+        };
+        auto rows1x1 = [&](const Feat &f, int ty, int cin, uint32_t wbase, int np, uint32_t col) {
+            switch ((f.S + 7) >> 3) {
+                case 1: rows_n(Int<1>{}, f, ty, cin, wbase, np, col); break;
+                case 2: rows_n(Int<2>{}, f, ty, cin, wbase, np, col); break;
+                case 3: rows_n(Int<3>{}, f, ty, cin, wbase, np, col); break;
+                default: rows_n(Int<4>{}, f, ty, cin, wbase, np, col); break;
+            }
         };
         for (int b = 0; b < 3; ++b) {
             const Feat f(p.hw >> b);
