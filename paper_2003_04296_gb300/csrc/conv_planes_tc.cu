@@ -26,8 +26,8 @@
 // operand row) and, for raw outputs, the int32 / fp32 stores.  The popcount
 // kernel spends 2 P_a P_w popcounts per 32 products at 16 a clock and SM; on a
 // 256 x 512 x 14 x 14, 3x3, 3-bit x 3-bit layer (quantize + convolve, raw and
-// fp32 outputs) it took 8.24 ms, this kernel 0.38 ms; a 4 x 128 x 32 x 32,
-// 1-bit x 1-bit layer 32.8 -> 20.5 us.
+// fp32 outputs) it took 8.24 ms, this kernel 0.26 ms (0.33 before loads by pairs
+// of lanes); a 4 x 128 x 32 x 32, 1-bit x 1-bit layer 32.8 -> 19.5 us.
 //
 // Every mbarrier wait is bounded; one that runs out sets this file's error
 // flag (read by minw_get_last_device_error) and the CTA winds down.
@@ -214,41 +214,93 @@ __device__ __forceinline__ void load_chunk(Chunk<P> &ch, Cursor &k, const ConvAr
     }
 }
 
-// The producer loop of one thread: every chunk of its row, expanded into the
-// ring slot's 64-byte row (chunk j of four at j ^ ((row >> 1) & 3): the 64-byte
-// swizzle, and no bank conflict between eight neighbouring rows).
+// Expands a chunk of row r into a ring slot (chunk word j of four at j ^ ((r
+// >> 1) & 3): the 64-byte swizzle, and no bank conflict between eight
+// neighbouring rows), once the MMAs of the slot's previous lap released it, and
+// arrives for the warp.
+struct Ring {
+    uint8_t *dst;
+    uint64_t *full, *empty;
+    int r, s, lap;
+    bool write, lane0;
+};
+template <int P>
+__device__ __forceinline__ bool put_chunk(const Params &p, Ring &g, const Chunk<P> &c) {
+    uint4 v[CW];
+#pragma unroll
+    for (int j = 0; j < CW; ++j) v[j] = expand<P>(c.w + j, (c.valid >> j) & 1u);
+    if (g.lap > 0 && !__all_sync(0xffffffffu, bar_wait(&g.empty[g.s], (g.lap - 1) & 1, p.wait_cycles))) return false;
+    if (g.write) {
+        uint4 *d = reinterpret_cast<uint4 *>(g.dst + (size_t)g.s * p.stage_bytes + g.r * ROWB);
+        const int sw = (g.r >> 1) & 3;
+#pragma unroll
+        for (int j = 0; j < CW; ++j) d[j ^ sw] = v[j];
+    }
+    fence_async_smem();
+    __syncwarp();
+    if (g.lane0) bar_arrive(&g.full[g.s]);
+    if (++g.s == p.S) { g.s = 0; ++g.lap; }
+    return true;
+}
+
+// The producer loop of one thread: every chunk of its row, two in flight.
 template <int P, bool ACT, bool VEC>
-__device__ __forceinline__ bool produce(const Params &p, uint8_t *dst, int r, bool write, bool live, int64_t row,
-                                        int y0, int x0, uint64_t *full, uint64_t *empty) {
+__device__ __forceinline__ void produce(const Params &p, Ring &g, bool live, int64_t row, int y0, int x0) {
     const ConvArgs &a = p.a;
     Cursor k{0, 0, 0};
     Chunk<P> c[2];
     load_chunk<P, ACT, VEC>(c[0], k, a, live, row, y0, x0);
     load_chunk<P, ACT, VEC>(c[1], k, a, live, row, y0, x0);
-    const uint32_t sw = (uint32_t)((r >> 1) & 3);
-    const bool lane0 = (threadIdx.x & 31) == 0;
-    int s = 0, lap = 0;
     for (int i = 0; i < p.nchunks; i += 2) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (i + h >= p.nchunks) break;
-            uint4 v[CW];
-#pragma unroll
-            for (int j = 0; j < CW; ++j) v[j] = expand<P>(c[h].w + j, (c[h].valid >> j) & 1u);
+            if (!put_chunk<P>(p, g, c[h])) return;
             load_chunk<P, ACT, VEC>(c[h], k, a, live, row, y0, x0);
-            if (lap > 0 && !__all_sync(0xffffffffu, bar_wait(&empty[s], (lap - 1) & 1, p.wait_cycles))) return false;
-            if (write) {
-                uint4 *d = reinterpret_cast<uint4 *>(dst + (size_t)s * p.stage_bytes + r * ROWB);
-#pragma unroll
-                for (int j = 0; j < CW; ++j) d[j ^ sw] = v[j];
-            }
-            fence_async_smem();
-            __syncwarp();
-            if (lane0) bar_arrive(&full[s]);
-            if (++s == p.S) { s = 0; ++lap; }
         }
     }
-    return true;
+}
+
+// The same where NW is a multiple of eight: an odd and an even lane load the
+// two 16-byte halves of eight words of one row and then of another, so that a
+// load instruction touches 16 lines instead of 32 (its lines, looked up one a
+// clock, held the 512-channel layers), and exchange halves by shuffles.  Lane l
+// of the warp holds row (l >> 1) + 16 (l & 1) of its 32.  rowA, yA, xA and
+// rowB, yB, xB: rows l >> 1 and (l >> 1) + 16.
+template <int P, bool ACT>
+__device__ __forceinline__ void produce_pair(const Params &p, Ring &g, bool liveA, int64_t rowA, int yA, int xA, bool liveB,
+                                             int64_t rowB, int yB, int xB) {
+    const ConvArgs &a = p.a;
+    const bool odd = threadIdx.x & 1;
+    // each lane's cursor starts at its half and steps by eight words
+    Cursor k{0, 0, odd ? CW : 0};
+    Chunk<P> A, B;
+    auto load = [&]() {
+        Cursor ka = k, kb = k;
+        load_chunk<P, ACT, true>(A, ka, a, liveA, rowA, yA, xA);
+        load_chunk<P, ACT, true>(B, kb, a, liveB, rowB, yB, xB);
+        k.w += 2 * CW;
+        if (k.w >= a.NW) {
+            k.w -= a.NW;
+            if (++k.kx == a.kw) { k.kx = 0; ++k.ky; }
+        }
+    };
+    load();
+    for (int i = 0; i < p.nchunks; i += 2) {             // nchunks is even: kh kw NW / 4
+        // the even lane gives its half of row B for the odd lane's half of row A
+        Chunk<P> c0, c1;
+#pragma unroll
+        for (int j = 0; j < P * CW; ++j) {
+            const uint32_t o = __shfl_xor_sync(0xffffffffu, odd ? A.w[j] : B.w[j], 1);
+            c0.w[j] = odd ? o : A.w[j];
+            c1.w[j] = odd ? B.w[j] : o;
+        }
+        const uint32_t ov = __shfl_xor_sync(0xffffffffu, odd ? A.valid : B.valid, 1);
+        c0.valid = odd ? ov : A.valid;
+        c1.valid = odd ? B.valid : ov;
+        load();
+        if (!put_chunk<P>(p, g, c0) || !put_chunk<P>(p, g, c1)) return;
+    }
 }
 
 // Level planes of BN output y of one channel (bits 0 .. OUTB - 1), the fp32
@@ -330,7 +382,8 @@ __device__ __forceinline__ void store_pooled(const ConvArgs &a, const float *acc
     }
 }
 
-template <bool VEC, int OUTB>
+// MODE: loads of single words (0), of four words of a row (1: NW % 4 == 0), of eight by two lanes (2: NW % 8 == 0).
+template <int MODE, int OUTB>
 __global__ void __launch_bounds__(NT, 2) conv_planes_tc_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (su32(smem_raw) & 1023u)) & 1023u);
@@ -395,27 +448,51 @@ __global__ void __launch_bounds__(NT, 2) conv_planes_tc_kernel(const __grid_cons
         }
         if (alive) mma_commit(&tfull);
     } else {
-        const int r = threadIdx.x & (BM - 1);
+        // this thread's row of the operand, and for paired loads the two rows it loads from
+        constexpr bool PAIR = MODE == 2;
+        const int w32 = (warp & 3) * 32;
+        const int rA = PAIR ? w32 + (lane >> 1) : w32 + lane, rB = rA + 16;
+        Ring g{warp < 4 ? smem : smem + BM * ROWB, full, empty, PAIR ? (lane & 1 ? rB : rA) : rA, 0, 0, true, lane == 0};
         if (warp < 4) {
-            const long long m = m0 + r;
-            const bool live = m < a.M;
             const int HoWo = a.Ho * a.Wo;
-            const int b = live ? (int)(m / HoWo) : 0;
-            const int pix = live ? (int)(m - (long long)b * HoWo) : 0;
-            const int yo = pix / a.Wo, xo = pix - yo * a.Wo;
-            const int64_t row = (int64_t)b * a.H * a.W;
-            const int y0 = yo * a.stride - a.pad, x0 = xo * a.stride - a.pad;
-            if (a.bits_a == 1) produce<1, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
-            else if (a.bits_a == 2) produce<2, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
-            else produce<3, true, VEC>(p, smem, r, true, live, row, y0, x0, full, empty);
+            auto place = [&](int r, bool &live, int64_t &row, int &y0, int &x0) {
+                const long long m = m0 + r;
+                live = m < a.M;
+                const int b = live ? (int)(m / HoWo) : 0;
+                const int pix = live ? (int)(m - (long long)b * HoWo) : 0;
+                const int yo = pix / a.Wo, xo = pix - yo * a.Wo;
+                row = (int64_t)b * a.H * a.W;
+                y0 = yo * a.stride - a.pad;
+                x0 = xo * a.stride - a.pad;
+            };
+            bool lA, lB = false;
+            int64_t wA, wB = 0;
+            int yA, xA, yB = 0, xB = 0;
+            place(rA, lA, wA, yA, xA);
+            if constexpr (PAIR) {
+                place(rB, lB, wB, yB, xB);
+                if (a.bits_a == 1) produce_pair<1, true>(p, g, lA, wA, yA, xA, lB, wB, yB, xB);
+                else if (a.bits_a == 2) produce_pair<2, true>(p, g, lA, wA, yA, xA, lB, wB, yB, xB);
+                else produce_pair<3, true>(p, g, lA, wA, yA, xA, lB, wB, yB, xB);
+            } else {
+                if (a.bits_a == 1) produce<1, true, MODE == 1>(p, g, lA, wA, yA, xA);
+                else if (a.bits_a == 2) produce<2, true, MODE == 1>(p, g, lA, wA, yA, xA);
+                else produce<3, true, MODE == 1>(p, g, lA, wA, yA, xA);
+            }
         } else {
-            const int o = o0 + r;
-            const bool write = r < p.BN, live = write && o < a.O;
-            const int64_t row = (int64_t)o * a.kh * a.kw;
-            uint8_t *dst = smem + BM * ROWB;
-            if (a.bits_w == 1) produce<1, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
-            else if (a.bits_w == 2) produce<2, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
-            else produce<3, false, VEC>(p, dst, r, write, live, row, 0, 0, full, empty);
+            g.write = g.r < p.BN;
+            const int taps = a.kh * a.kw;
+            const bool lA = rA < p.BN && o0 + rA < a.O, lB = rB < p.BN && o0 + rB < a.O;
+            const int64_t wA = (int64_t)(o0 + rA) * taps, wB = (int64_t)(o0 + rB) * taps;
+            if constexpr (PAIR) {
+                if (a.bits_w == 1) produce_pair<1, false>(p, g, lA, wA, 0, 0, lB, wB, 0, 0);
+                else if (a.bits_w == 2) produce_pair<2, false>(p, g, lA, wA, 0, 0, lB, wB, 0, 0);
+                else produce_pair<3, false>(p, g, lA, wA, 0, 0, lB, wB, 0, 0);
+            } else {
+                if (a.bits_w == 1) produce<1, false, MODE == 1>(p, g, lA, wA, 0, 0);
+                else if (a.bits_w == 2) produce<2, false, MODE == 1>(p, g, lA, wA, 0, 0);
+                else produce<3, false, MODE == 1>(p, g, lA, wA, 0, 0);
+            }
         }
         __syncwarp();
         // a wait that ran out (here or in the MMA warp) leaves tfull open: no output is written
@@ -488,12 +565,15 @@ minw_status launch_planes_tc(const ConvArgs &a, cudaStream_t s) {
     if (smem < pool) smem = pool;
     smem += 1024;
     typedef void (*Kernel)(const ptc::Params);
-    static const Kernel kernels[2][4] = {
-        {ptc::conv_planes_tc_kernel<false, 0>, ptc::conv_planes_tc_kernel<false, 1>,
-         ptc::conv_planes_tc_kernel<false, 2>, ptc::conv_planes_tc_kernel<false, 3>},
-        {ptc::conv_planes_tc_kernel<true, 0>, ptc::conv_planes_tc_kernel<true, 1>,
-         ptc::conv_planes_tc_kernel<true, 2>, ptc::conv_planes_tc_kernel<true, 3>}};
-    const Kernel kern = kernels[a.NW % ptc::CW == 0][a.quant_out ? a.qo.bits : 0];
+    static const Kernel kernels[3][4] = {
+        {ptc::conv_planes_tc_kernel<0, 0>, ptc::conv_planes_tc_kernel<0, 1>, ptc::conv_planes_tc_kernel<0, 2>,
+         ptc::conv_planes_tc_kernel<0, 3>},
+        {ptc::conv_planes_tc_kernel<1, 0>, ptc::conv_planes_tc_kernel<1, 1>, ptc::conv_planes_tc_kernel<1, 2>,
+         ptc::conv_planes_tc_kernel<1, 3>},
+        {ptc::conv_planes_tc_kernel<2, 0>, ptc::conv_planes_tc_kernel<2, 1>, ptc::conv_planes_tc_kernel<2, 2>,
+         ptc::conv_planes_tc_kernel<2, 3>}};
+    const int mode = a.NW % (2 * ptc::CW) == 0 ? 2 : a.NW % ptc::CW == 0 ? 1 : 0;
+    const Kernel kern = kernels[mode][a.quant_out ? a.qo.bits : 0];
     constexpr int SMEM_MAX = ptc::SMAX * (ptc::BM + 128) * ptc::ROWB + 1024;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess)
         return MINW_ECUDA;
