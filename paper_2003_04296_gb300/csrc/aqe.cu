@@ -23,6 +23,8 @@ __device__ __forceinline__ float aqe_fwd1(float x, float alpha, float oma, const
 __global__ void __launch_bounds__(256) aqe_forward_kernel(const float *__restrict__ x,
                                                           float *__restrict__ y, int64_t n,
                                                           float alpha, float oma, QParams q) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t n4 = n >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
@@ -123,6 +125,8 @@ __device__ __forceinline__ float aqe_bwd1(float x, float g, float two_alpha) {
 __global__ void __launch_bounds__(256) aqe_backward_kernel(const float *__restrict__ x,
                                                            const float *gy, float *gx,
                                                            int64_t n, float two_alpha) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t n4 = n >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
@@ -145,6 +149,8 @@ __global__ void __launch_bounds__(256) aqe_backward_kernel(const float *__restri
 __global__ void __launch_bounds__(256) aqe_backward_masked_kernel(const uint32_t *__restrict__ mask,
                                                                   const float *gy, float *gx,
                                                                   int64_t n, float two_alpha) {
+    pdl_trigger();
+    pdl_wait();
     const int64_t n4 = n >> 2;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const float4 *g4 = reinterpret_cast<const float4 *>(gy);
@@ -185,8 +191,9 @@ __global__ void __launch_bounds__(256) aqe_backward_masked_kernel(const uint32_t
 // the 256 threads stay busy.
 // A warp per 32 channels with its channels in a serial loop, as before, had
 // one load in flight and few warps on small tensors: 256 x 512 x 14 x 14,
-// 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (51 and 4 us here; instruction issue bounds
-// the first, at 45 % of the resident warps).
+// 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (38 and 4 us here; instruction
+// issue bounds the first, so plane bits are collected as signs of differences:
+// 51 us with a compare and a select each).
 // ---------------------------------------------------------------------------
 
 enum QuantOut { OUT_PLANES, OUT_E4M3, OUT_E2M1 };
@@ -218,6 +225,7 @@ __device__ __forceinline__ uint32_t plane_bytes(float u, const QParams &q) {
 // The level's value (level_value with the bit width known: no integer conversion).
 template <int BITS>
 __device__ __forceinline__ float level_of(float u, const QParams &q) {
+    if constexpr (BITS == 2) return ((u > q.thr0) ? 1.0f : 0.0f) - ((u < -q.thr0) ? 1.0f : 0.0f);
     constexpr float one = BITS == 3 ? 0.25f : 1.0f;
     const float s = (u > 0.0f) ? 1.0f : -1.0f;
     return s * pick<BITS, float>(fabsf(u), q, 0.0f, one, 0.5f, 1.0f);
@@ -302,16 +310,53 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
             load(it);
         }
         uint32_t w[V];
-#pragma unroll
-        for (int i = 0; i < V; ++i) w[i] = 0u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        if constexpr (OUT == OUT_PLANES) {
+            // a comparison's bit is the sign of a difference (exact, and +0 at equality), shifted into the
+            // pixel's nibble: two instructions; NaN, whose differences carry no sign, takes the selects
+            float any = 0.0f;
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                const float u = v[k][i] * q.scale;
-                if constexpr (OUT == OUT_PLANES) w[i] |= plane_bytes<BITS>(u, q) << k;
-                else if constexpr (OUT == OUT_E2M1) w[i] |= code_of<BITS, true>(u, q) << (4 * k);
-                else w[i] |= code_of<BITS, false>(u, q) << (8 * k);
+                uint32_t s0 = 0u, s1 = 0u, s2 = 0u, s3 = 0u;
+#pragma unroll
+                for (int k = 3; k >= 0; --k) {
+                    const float u = v[k][i] * q.scale;
+                    asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(any) : "f"(u));
+                    if constexpr (BITS == 1) {
+                        s0 = __funnelshift_l(__float_as_uint(0.0f - u), s0, 1);              // u > 0
+                    } else if constexpr (BITS == 2) {
+                        s0 = __funnelshift_l(__float_as_uint(u + q.thr0), s0, 1);            // u < -D
+                        s1 = __funnelshift_l(__float_as_uint(q.thr0 - u), s1, 1);            // u > D
+                    } else {
+                        const float m = fabsf(u);
+                        s0 = __funnelshift_l(__float_as_uint(u), s0, 1);                     // u < 0
+                        s1 = __funnelshift_l(__float_as_uint(q.thr2 - m), s1, 1);            // |u| > D_3, D_2, D_1
+                        s2 = __funnelshift_l(__float_as_uint(q.thr1 - m), s2, 1);
+                        s3 = __funnelshift_l(__float_as_uint(q.thr0 - m), s3, 1);
+                    }
+                }
+                if constexpr (BITS == 1) w[i] = s0 ^ 0xFu;
+                else if constexpr (BITS == 2) w[i] = s0 | ((s0 | s1) << 8);
+                else w[i] = (s0 & s1) | ((s1 & (~s2 | s3)) << 8) | (s2 << 16);
+            }
+            if (any != any) {
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    w[i] = 0u;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w[i] |= plane_bytes<BITS>(v[k][i] * q.scale, q) << k;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < V; ++i) w[i] = 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const float u = v[k][i] * q.scale;
+                    if constexpr (OUT == OUT_E2M1) w[i] |= code_of<BITS, true>(u, q) << (4 * k);
+                    else w[i] |= code_of<BITS, false>(u, q) << (8 * k);
+                }
             }
         }
         // this thread's channels of the tensor (planes: bits of channels past C stay zero)
@@ -339,36 +384,37 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
                 }
             }
             if (mask != nullptr) {
-                // 32 consecutive pixels of a channel row sit in 32 / V neighbouring lanes of one warp
+                // 32 consecutive pixels of a channel row sit in 32 / V neighbouring lanes of one warp; lane k of
+                // them stores channel k's word
+                uint32_t mk = 0u;
+                const int rl = V == 4 ? threadIdx.x & 7 : threadIdx.x & 31;       // lane in the run
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     uint32_t m = 0u;
-                    const bool in = k < nst;
 #pragma unroll
                     for (int i = 0; i < V; ++i) m |= (fabsf(v[k][i]) <= 1.0f ? 1u : 0u) << i;
-                    m = in ? m : 0u;
-                    bool first;                                   // run's first lane
+                    m = pin ? m : 0u;
                     if constexpr (V == 4) {
-                        m <<= (threadIdx.x & 7) * 4;
+                        m <<= rl * 4;
                         m |= __shfl_xor_sync(0xffffffffu, m, 1);
                         m |= __shfl_xor_sync(0xffffffffu, m, 2);
                         m |= __shfl_xor_sync(0xffffffffu, m, 4);
-                        first = (threadIdx.x & 7) == 0;
                     } else {
                         m = __ballot_sync(0xffffffffu, m);
-                        first = (threadIdx.x & 31) == 0;
                     }
-                    if (first && in) {                            // flat bit offset of the run's first pixel
-                        const int64_t at = off + (int64_t)k * HW;
-                        uint32_t *mw = mask + (at >> 5);
-                        const uint32_t sh = (uint32_t)at & 31u;
-                        const uint32_t hi = __funnelshift_l(m, 0u, sh);     // bits past the first word
-                        if (!mask_atomic) {
-                            *mw = m;
-                        } else {
-                            atomicOr(mw, m << sh);
-                            if (hi) atomicOr(mw + 1, hi);
-                        }
+                    mk = rl == k ? m : mk;
+                }
+                const int pr = p - V * rl;                        // the run's first pixel
+                if (rl < nc && pr < HW) {
+                    const int64_t at = (b * C + c + rl) * HW + pr;
+                    uint32_t *mw = mask + (at >> 5);
+                    const uint32_t sh = (uint32_t)at & 31u;
+                    const uint32_t hi = __funnelshift_l(mk, 0u, sh);     // bits past the first word
+                    if (!mask_atomic) {
+                        *mw = mk;
+                    } else {
+                        atomicOr(mw, mk << sh);
+                        if (hi) atomicOr(mw + 1, hi);
                     }
                 }
             }
@@ -634,8 +680,8 @@ minw_status aqe_forward(const float *x, float *y, int64_t n, float alpha, const 
     if (!x || !y || !aligned16(x) || !aligned16(y)) return MINW_EINVAL;
     const QParams qp = to_qparams(q);
     const int64_t g = grid_for(n / 4 + 1, 256);
-    aqe_forward_kernel<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, y, n, alpha, 1.0f - alpha, qp);
-    return launch_status();
+    return launch_pdl(aqe_forward_kernel, dim3((unsigned)g), dim3(256), 0, (cudaStream_t)stream, x, y, n, alpha,
+                      1.0f - alpha, qp) == cudaSuccess ? launch_status() : MINW_ECUDA;
 }
 
 minw_status aqe_forward_stochastic(const float *x, float *y, int64_t n, float alpha, uint64_t seed,
@@ -655,8 +701,8 @@ minw_status aqe_backward(const float *x, const float *gy, float *gx, int64_t n, 
     if (n == 0) return MINW_OK;
     if (!x || !gy || !gx || !aligned16(x) || !aligned16(gy) || !aligned16(gx)) return MINW_EINVAL;
     const int64_t g = grid_for(n / 4 + 1, 256);
-    aqe_backward_kernel<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(x, gy, gx, n, 2.0f * alpha);
-    return launch_status();
+    return launch_pdl(aqe_backward_kernel, dim3((unsigned)g), dim3(256), 0, (cudaStream_t)stream, x, gy, gx, n,
+                      2.0f * alpha) == cudaSuccess ? launch_status() : MINW_ECUDA;
 }
 
 minw_status aqe_backward_masked(const uint32_t *mask, const float *gy, float *gx, int64_t n,
@@ -665,9 +711,8 @@ minw_status aqe_backward_masked(const uint32_t *mask, const float *gy, float *gx
     if (n == 0) return MINW_OK;
     if (!mask || !gy || !gx || !aligned16(gy) || !aligned16(gx)) return MINW_EINVAL;
     const int64_t g = grid_for(n / 4 + 1, 256);
-    aqe_backward_masked_kernel<<<(unsigned)g, 256, 0, (cudaStream_t)stream>>>(mask, gy, gx, n,
-                                                                            2.0f * alpha);
-    return launch_status();
+    return launch_pdl(aqe_backward_masked_kernel, dim3((unsigned)g), dim3(256), 0, (cudaStream_t)stream, mask, gy, gx, n,
+                      2.0f * alpha) == cudaSuccess ? launch_status() : MINW_ECUDA;
 }
 
 minw_status aqe_quantize_pack(const float *x, int32_t B, int32_t C, int32_t H, int32_t W,

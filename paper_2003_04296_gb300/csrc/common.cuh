@@ -357,6 +357,9 @@ int take_stall(int which);          // 1 once after minw_test_stall_next_launch(
 // no L1 / shared-memory reconfiguration of the SM between them, so the next
 // kernel's CTAs start as soon as an SM frees up.
 void max_shared_carveout(const void *kern);
+// Allows kern bytes of dynamic shared memory (set once per kernel and device: the attribute call costs the
+// host about as much as a launch).
+bool allow_shared(const void *kern, int bytes);
 
 // cuTensorMapEncodeTiled from the driver (nullptr when it is unavailable).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,

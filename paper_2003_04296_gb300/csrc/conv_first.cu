@@ -185,6 +185,7 @@ template <int OUTB, int KH, int KW, int S, bool TM>
 __global__ void __launch_bounds__(FIRST_NT, 2)
     conv_first_kernel(const FirstArgs a, const FirstTile tl, const __grid_constant__ CUtensorMap tmX) {
     extern __shared__ float4 smem4[];
+    if (!a.planned) pdl_wait();                                   // the weights too may come from an earlier kernel
     const int kh = KH ? KH : a.kh, kw = KW ? KW : a.kw, st = S ? S : a.stride;
     const int OCB = tl.OCB, K = tl.K, RP = tl.RP, Ws = tl.Ws;
     const size_t patch = (size_t)tl.pstride;

@@ -100,6 +100,7 @@ struct Params {
     int codes4;
     long long wait_cycles;
     int stall;
+    int planned;           // see FirstArgs
 };
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -464,6 +465,7 @@ __global__ void __launch_bounds__(NT, 1)
     } else if (warp < REC0) {
         // ---------------- epilogue warps: weight preparation, then the epilogue ----------------
         const int et = threadIdx.x - EPI0 * 32;   // 0 .. 255
+        if (!p.planned) pdl_wait();
         // the chain's fp32 weights, [O][Ks]
         for (int i = et; i < K * O; i += NEPI * 32) {
             const int k = i / O, o = i - k * O;
@@ -866,6 +868,7 @@ minw_status launch_first_tc(const FirstArgs &a, cudaStream_t s) {
     p.planes_out = a.planes_out; p.codes_out = a.codes_out; p.codes4 = a.codes4;
     p.wait_cycles = (long long)minw_host::plan_options().wait_cycles;
     p.stall = minw_host::take_stall(MINW_STALL_CONV_FIRST);
+    p.planned = a.planned;
     CUtensorMap tm;
     memset(&tm, 0, sizeof(tm));
     const cuuint64_t dims[4] = {(cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.C, (cuuint64_t)a.B};

@@ -575,8 +575,7 @@ minw_status launch_planes_tc(const ConvArgs &a, cudaStream_t s) {
     const int mode = a.NW % (2 * ptc::CW) == 0 ? 2 : a.NW % ptc::CW == 0 ? 1 : 0;
     const Kernel kern = kernels[mode][a.quant_out ? a.qo.bits : 0];
     constexpr int SMEM_MAX = ptc::SMAX * (ptc::BM + 128) * ptc::ROWB + 1024;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX) != cudaSuccess)
-        return MINW_ECUDA;
+    if (!minw_host::allow_shared(reinterpret_cast<const void *>(kern), SMEM_MAX)) return MINW_ECUDA;
     if (minw_host::launch_pdl(kern, dim3((unsigned)(tiles_m * p.ntn)), dim3(ptc::NT), smem, s, p) != cudaSuccess)
         return MINW_ECUDA;
     return cudaGetLastError() == cudaSuccess ? MINW_OK : MINW_ECUDA;

@@ -87,6 +87,7 @@ struct Params {
     const float *res_f32;      // shortcut as fp32 NHWC [B][Hp][Wp][O] (nullable)
     float *y_nhwc;             // BN output (before the shortcut) as fp32 NHWC (nullable)
     const float *ythr;         // breakpoints of the output quantizer on y (nullable: computed here)
+    int planned;               // see ConvArgs
     int resal;                 // the shortcut and y_nhwc start on 16 bytes (wide accesses)
     uint16_t *hb_out;          // bf16 operands: HardTanh(BN(acc) [+ hb_res]) as bf16 NHWC rows of hb_ld, at hb_off
     int hb_ld, hb_off;
@@ -977,6 +978,7 @@ __global__ void __launch_bounds__(NT, 1)
             const bool arrive = !PAIR || crank == 0;
             const int nissue = p.wres ? 2 * p.tlanes : p.tlanes;          // issuers of this operand
             const int myid = (p.wres && wwarp) ? p.tlanes + lane : lane;
+            if (!p.planned) pdl_wait();
             if (p.wres && wwarp && lane == 0) {
                 // the channel tile's weights, all K blocks, once
                 const int o0 = (((int)blockIdx.x / p.cl) % p.ntn) * p.BN;
@@ -995,7 +997,7 @@ __global__ void __launch_bounds__(NT, 1)
                 }
             }
             if (act) pdl_wait();                  // activations come from the previous kernel
-                                                  // (the weights above do not: they load before)
+                                                  // (a network's weights do not: they load before)
             int g = 0, s = 0, lap = 0;             // stages walked, ring slot, ring lap
             bool alive = true;
             for (int n = 0, w; alive && (w = cta_item(p, n, items, tiles_m, crank)) >= 0; ++n) {
@@ -1172,6 +1174,7 @@ __global__ void __launch_bounds__(NT, 1)
                 }
             }
         }
+        if (!p.planned) pdl_wait();
         epi_tables<OUTB>(p, resid, sthr, ssig, syt, reinterpret_cast<float *>(tmem_slot + 1), O32, thr_floats, sig_words, et,
                          warp, lane);
         asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");   // breakpoints in place
@@ -1764,13 +1767,10 @@ __global__ void __launch_bounds__(halo::NT, 1)
     if (warp == 0) {
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
-            // a network's weights (its breakpoints are precomputed too) were written long ago; a standalone
-            // call's may come from the kernel before
-            const bool planned = p.thr != nullptr || p.ythr != nullptr;
-            if (!planned) pdl_wait();
+            if (!p.planned) pdl_wait();
             mbar_expect_tx(&wfull, (uint32_t)p.nk * p.b_bytes);
             for (int k = 0; k < p.nk; ++k) tma_load_2d(wres + (size_t)k * p.b_bytes, &tmB, &wfull, k * p.cb, o0);
-            if (planned) pdl_wait();
+            if (p.planned) pdl_wait();
             int s = 0, lap = 0, g = 0;
             for (int t = t0; t < tiles; t += upt, ++g) {
                 if (lap > 0 && !mbar_wait(&empty[s], (lap - 1) & 1, p.wait_cycles)) break;
@@ -1844,6 +1844,7 @@ __global__ void __launch_bounds__(halo::NT, 1)
             }
         }
         const int set = (warp - 2) / EPI_WARPS;
+        if (!p.planned) pdl_wait();
         if (set == 0) epi_tables<OUTB>(p, resid, sthr, ssig, syt, yt, O32, thr_floats, sig_words, et, warp, lane);
         asm volatile("bar.sync 2, %0;\n" ::"n"(halo::SETS * EPI_WARPS * 32) : "memory");
         pdl_wait();
@@ -2188,6 +2189,7 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     }
     p.nlev = a.quant_out ? num_levels(a.qo.bits) : 0;
     p.thr = a.thr;
+    p.planned = a.planned;
     // CTA pairs (MINW_TC_PAIR): 256-channel tiles of a layer that is not split along K
     {
         const int sms_ = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
@@ -2404,6 +2406,7 @@ static bool halo_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     p.b_bytes = (uint32_t)(p.BN * rowb);
     p.nlev = num_levels(a.qo.bits);
     p.thr = a.thr;
+    p.planned = a.planned;
     p.acc_cols = p.BN;
     p.tmem_cols = 512;
     // accumulators below the E2M1 scale factors at column 448
@@ -2449,8 +2452,7 @@ static minw_status launch_halo(const Plan &pl, cudaStream_t s) {
         {conv_halo_kernel<1, 0>, conv_halo_kernel<2, 0>, conv_halo_kernel<3, 0>},
         {conv_halo_kernel<1, 2>, conv_halo_kernel<2, 2>, conv_halo_kernel<3, 2>}};
     const Kernel kern = kernels[pl.p.fp4][pl.p.qo.bits - 1];
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess)
-        return MINW_ECUDA;
+    if (!minw_host::allow_shared(reinterpret_cast<const void *>(kern), 224 * 1024)) return MINW_ECUDA;
     Params pm = pl.p;
     pm.wait_cycles = (long long)minw_host::plan_options().wait_cycles;
     pm.stall = minw_host::take_stall(MINW_STALL_CONV_TC);

@@ -239,8 +239,7 @@ __global__ void __launch_bounds__(256) wgrad_update_kernel(const float *__restri
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int R = C * ntaps, r0 = blockIdx.x * 32;
     const size_t n = (size_t)R * O;
-    pdl_trigger();
-    pdl_wait();
+    pdl_wait();                       // (and no early start of a dependent: it may read W before it waits)
     for (int o0 = blockIdx.y * 32; o0 < O; o0 += gridDim.y * 32) {
         float acc[4];
         const float *src[4];
@@ -351,9 +350,7 @@ minw_status launch_conv_wgrad(const WgradArgs &a, float *part, float lr, float t
     };
     if (!encode(&tmG, a.gd, a.Op, a.Hd, a.Wd) || !encode(&tmA, a.ab, a.C, a.H, a.W)) return MINW_ECUDA;
     const size_t smem = (size_t)p.S * p.stage_bytes + 1024;
-    if (cudaFuncSetAttribute(wg::conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=
-        cudaSuccess)
-        return MINW_ECUDA;
+    if (!minw_host::allow_shared(reinterpret_cast<const void *>(wg::conv_wgrad_kernel), 220 * 1024)) return MINW_ECUDA;
     const unsigned grid = (unsigned)(p.nm * p.nn * p.ntg * p.slices);
     if (minw_host::launch_pdl(wg::conv_wgrad_kernel, dim3(grid), dim3(wg::NT), smem, s, tmG, tmA, p) != cudaSuccess)
         return MINW_ECUDA;

@@ -50,6 +50,9 @@ struct ConvArgs {
                            // tensor memory beside the scale factors)
     int pair_n128;         // E2M1: CTA pairs of 256 pixels x 128 channels (two accumulators fit the tensor
                            // memory beside the scale factors, so the epilogue overlaps the next MMAs)
+    int planned;           // a network's layer: weights, BN maps and breakpoints were written at its creation, so
+                           // the kernel may read them while the kernel before it still runs (else it waits first:
+                           // a pass before a standalone call may have written them)
     int ldc;               // bf16 operands: elements between pixel rows of act8 (0: C); the product reads
                            // channels 0 .. C of each row (the first C of a wider feature buffer)
     // bf16 operands, in place of y_out: HardTanh(BN(acc)) rounded to bf16 into NHWC rows of hb_ld
@@ -77,6 +80,7 @@ struct FirstArgs {
     float *y_out;              // [B][O][Ho][Wo] (nullable)
     const float *thr;          // fp32 breakpoints [O][8] (nullable: computed in-kernel)
     const float *wt;           // prepared weights [K][O] (levels when quantized; nullable: from w)
+    int planned;               // as ConvArgs::planned
     long long wait_cycles;     // limit of the bounded patch waits (set by the launcher)
     int stall;                 // timeout-path test: first wait on a barrier nothing completes (set by the launcher)
 };

@@ -417,6 +417,7 @@ static minw_status forward_enqueue(minw_net *net, const float *x, int32_t B, flo
         minw_status st;
         if (l == 0) {
             FirstArgs a{};
+            a.planned = 1;
             a.x = x; a.w = P.wlatent; a.cscale = P.wscale;
             a.quant_w = P.d.bits_w > 0;
             if (a.quant_w) a.qw = to_qparams(&P.qw);
@@ -435,6 +436,7 @@ static minw_status forward_enqueue(minw_net *net, const float *x, int32_t B, flo
         } else {
             const void *src = net->buf[cur ^ 1];
             ConvArgs a{};
+            a.planned = 1;
             a.B = B; a.C = P.C; a.H = P.H; a.W = P.W; a.O = P.O; a.kh = P.kh; a.kw = P.kw;
             a.stride = P.stride; a.pad = P.pad; a.Ho = P.Ho; a.Wo = P.Wo; a.NW = P.C / 32;
             a.bits_a = P.d.bits_in; a.bits_w = P.d.bits_w;

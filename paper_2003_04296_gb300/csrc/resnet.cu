@@ -237,6 +237,7 @@ static minw_status copy_owned(minw_net *n, float **dst, const float *src, size_t
 
 static ConvArgs conv_args(const ResConv &c, int B) {
     ConvArgs a{};
+    a.planned = 1;
     a.B = B; a.C = c.C; a.H = c.H; a.W = c.W; a.O = c.O; a.kh = c.k; a.kw = c.k;
     a.stride = c.stride; a.pad = c.pad; a.Ho = c.Ho; a.Wo = c.Wo; a.NW = c.C / 32;
     a.M = (long long)B * c.Ho * c.Wo;
@@ -464,6 +465,7 @@ minw_status resnet_forward(minw_net *net, const float *x, int B, float *logits, 
     // stem convolution -> level codes [B][Hs][Hs][64]
     {
         FirstArgs a{};
+        a.planned = 1;
         a.x = x; a.w = R->stem_w; a.quant_w = 0;
         a.B = B; a.C = 3; a.H = R->hw; a.W = R->hw; a.O = 64; a.kh = 7; a.kw = 7; a.stride = 2; a.pad = 3;
         a.Ho = R->Hs; a.Wo = R->Hs;

@@ -15,7 +15,9 @@
 
 #include <atomic>
 #include <mutex>
+#include <set>
 #include <unordered_set>
+#include <utility>
 
 #include "kernels.cuh"
 
@@ -56,6 +58,19 @@ bool pdl_enabled() { return plan_options().pdl != 0; }
 int take_stall(int which) {
     int expected = which;
     return g_stall.compare_exchange_strong(expected, 0) ? 1 : 0;
+}
+
+bool allow_shared(const void *kern, int bytes) {
+    static std::mutex mu;
+    static std::set<std::pair<int, const void *>> done;      // the attribute belongs to a device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    const std::pair<int, const void *> key(dev, kern);
+    if (done.count(key)) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done.insert(key);
+    return true;
 }
 
 void max_shared_carveout(const void *kern) {

@@ -329,6 +329,7 @@ minw_status wresnet_forward(minw_net *net, const float *x, int B, float *logits,
     const int hw = R->hw;
     {
         FirstArgs a{};
+        a.planned = 1;
         a.x = x; a.w = R->stem_w; a.quant_w = 0;
         a.B = B; a.C = 3; a.H = hw; a.W = hw; a.O = 16; a.kh = 3; a.kw = 3; a.stride = 1; a.pad = 1;
         a.Ho = hw; a.Wo = hw;
@@ -647,6 +648,7 @@ minw_status wdense_forward(minw_net *net, const float *x, int B, float *logits, 
     const int c0 = 2 * D->growth, k4 = 4 * D->growth;
     {
         FirstArgs a{};
+        a.planned = 1;
         a.x = x; a.w = D->stem_w; a.quant_w = 0;
         a.B = B; a.C = 3; a.H = D->hw; a.W = D->hw; a.O = c0; a.kh = 3; a.kw = 3; a.stride = 1; a.pad = 1;
         a.Ho = D->hw; a.Wo = D->hw;
