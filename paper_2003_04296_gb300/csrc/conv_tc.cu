@@ -2364,11 +2364,14 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
 // The plan of conv_halo_kernel, or false where conv_tc_kernel keeps the layer.
 // It takes 3 x 3 layers of stride 1 and padding 1 on rows of 64 or 128 bytes
 // whose only outputs are levels (with or without a shortcut), where its 16 x 8
-// tiles cover at least MIN_COVER of the computed pixels and give at least
-// MIN_TILES tiles per SM: below that the weights' load and the idle rows
-// outweigh the taps' loads.
+// tiles cover at least MIN_COVER of the pixels they compute, or ONE_WAVE_COVER
+// where every tile has an SM of its own.  Measured, quantizer pass included,
+// against conv_tc_kernel: 1 x 128 x 32 x 32 8.3 : 9.1 us, 64 x 256 x 8 x 8
+// (half covered, one wave) 11.6 : 12.9, 256 x 256 x 8 x 8 (half covered, three
+// waves) 17.8 : 15.3, 128 x 256 x 14 x 14 20.0 : 22.7, 128 x 64 x 56 x 56 with
+// a shortcut 61 : 120.
 static bool halo_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
-    constexpr double MIN_COVER = 0.6, MIN_TILES = 0.5;
+    constexpr double MIN_COVER = 0.6, ONE_WAVE_COVER = 0.45;
     if (a.bf16 || a.kh != 3 || a.kw != 3 || a.stride != 1 || a.pad != 1 || !a.quant_out || a.acc_out != nullptr ||
         a.y_out != nullptr || a.y_nhwc != nullptr || a.n128 || a.pair_n128 || a.upd || a.ksplit > 1 || a.O % 32 != 0)
         return false;
@@ -2387,7 +2390,7 @@ static bool halo_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     p.BN = a.O / p.ntn;
     const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
     const long long tiles = (long long)p.nbx * p.nby * p.nbb;
-    if (cover < MIN_COVER || (double)tiles * p.ntn < MIN_TILES * sms || tiles >= (1ll << 31)) return false;
+    if (cover < (tiles * p.ntn <= sms ? ONE_WAVE_COVER : MIN_COVER) || tiles >= (1ll << 31)) return false;
     if (p.ntn > sms) return false;
     if ((a.res_codes != nullptr || a.res_f32 != nullptr) &&
         (a.pool || !minw_host::aligned16(a.res_codes) || !minw_host::aligned16(a.res_f32)))
