@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(256) train_weights_kernel(const float *__restr
                                                             int Op, float alpha, QParams q, uint16_t *__restrict__ wf,
                                                             uint16_t *__restrict__ wd, float *__restrict__ ones,
                                                             float *__restrict__ zeros, int M) {
+    pdl_wait();
     // element counts below 2^31 (checked by the host): 32-bit index arithmetic
     const float oma = 1.0f - alpha;
     const int khw = kh * kw;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(256) train_grad_kernel(const float *__restrict
                                                          int O, int HoWo, int Wo, int stride, int Hd, int Wd, int Op,
                                                          float alpha, int quant_a, QParams qa,
                                                          float *__restrict__ a_out, uint16_t *__restrict__ gd) {
+    pdl_wait();
     __shared__ float tile[64][33];
     const int b = blockIdx.z;
     const int o0 = blockIdx.y * 64, p0 = blockIdx.x * 32;
@@ -258,8 +260,10 @@ minw_status minw_conv_train_step(const float *A, float *Wt, const float *g_out, 
     const int M = std::max(std::max(O, C), sh.Kw);
 #define TRY(x) do { if ((st = (x)) != MINW_OK) return st; } while (0)
     // W^ (Eq. weight) in both layouts; the input as bf16 NHWC
-    train_weights_kernel<<<grid_for((int64_t)O * kh * kw * C), 256, 0, s>>>(Wt, O, C, kh, kw, sh.Op, alpha, qw, wf,
-                                                                             wd, ones, zeros, M);
+    // (these passes start while the kernel before drains, and let no dependent start early)
+    if (launch_pdl(train_weights_kernel, dim3(grid_for((int64_t)O * kh * kw * C)), dim3(256), 0, s, (const float *)Wt, O, C,
+                   kh, kw, sh.Op, alpha, qw, wf, wd, ones, zeros, M) != cudaSuccess)
+        return MINW_ECUDA;
     TRY(launch_status());
     TRY(minw_to_bf16_nhwc(A, B, C, H, W, ab, stream));
     // a~ = a * W^ (fp32 NCHW [B][O][Ho][Wo]); the last layer emits a~ itself
@@ -271,8 +275,9 @@ minw_status minw_conv_train_step(const float *A, float *Wt, const float *g_out, 
         if (cudaMemsetAsync(gd, 0, (size_t)B * sh.Hd * sh.Wd * sh.Op * 2, s) != cudaSuccess) return MINW_ECUDA;
     {
         const dim3 grid((unsigned)((sh.Ho * sh.Wo + 31) / 32), (unsigned)(sh.Op / 64), (unsigned)B);
-        train_grad_kernel<<<grid, 256, 0, s>>>(q_a ? at : g_out, g_out, O, sh.Ho * sh.Wo, sh.Wo, stride, sh.Hd, sh.Wd,
-                                               sh.Op, alpha, q_a ? 1 : 0, qa, a_out, gd);
+        if (launch_pdl(train_grad_kernel, grid, dim3(256), 0, s, (const float *)(q_a ? at : g_out), g_out, O, sh.Ho * sh.Wo,
+                       sh.Wo, stride, sh.Hd, sh.Wd, sh.Op, alpha, q_a ? 1 : 0, qa, a_out, gd) != cudaSuccess)
+            return MINW_ECUDA;
         TRY(launch_status());
     }
     // the input gradient: the stride-1 convolution of the spread g~ with the flipped weights (NCHW [B][C][H][W])

@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const float *__restrict__ X, 
                                                    uint16_t *__restrict__ vb, uint16_t *__restrict__ vtb,
                                                    float *__restrict__ a_out, float *__restrict__ ones,
                                                    float *__restrict__ zeros, int M) {
+    pdl_wait();       // starts while the kernel before drains; lets no dependent start early (its output is weights too)
     __shared__ float tile[32][65];
     const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 64;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;     // columns 4 tx .. 4 tx + 3 of rows ty, ty + 16
@@ -272,10 +273,13 @@ minw_status minw_fc_train_step(const float *A, float *W, const float *g_out, int
     minw_status st;
 #define TRY(x) do { if ((st = (x)) != MINW_OK) return st; } while (0)
     // 1.1 forward: W^ = alpha h(W) + (1 - alpha) W as bf16 [O][K] and [K][Op]; a as bf16 [B][K] and [K][B]
-    prep_kernel<0><<<dim3((unsigned)(K / 64), (unsigned)(Op / 32)), 256, 0, s>>>(
-        W, nullptr, O, K, K, Op, alpha, qw, wb, wtb, nullptr, ones, zeros, M);
-    prep_kernel<1><<<dim3((unsigned)(K / 64), (unsigned)(B / 32)), 256, 0, s>>>(
-        A, nullptr, B, K, K, B, 0.0f, qw, ab, atb, nullptr, nullptr, nullptr, 0);
+    const float *none = nullptr;
+    float *fnone = nullptr;
+    if (launch_pdl(prep_kernel<0>, dim3((unsigned)(K / 64), (unsigned)(Op / 32)), dim3(256), 0, s, (const float *)W, none, O,
+                   K, K, Op, alpha, qw, wb, wtb, fnone, ones, zeros, M) != cudaSuccess ||
+        launch_pdl(prep_kernel<1>, dim3((unsigned)(K / 64), (unsigned)(B / 32)), dim3(256), 0, s, A, none, B, K, K, B, 0.0f,
+                   qw, ab, atb, fnone, fnone, fnone, 0) != cudaSuccess)
+        return MINW_ECUDA;
     TRY(launch_status());
     // a~ = a W^T  ([B][O], reduction over K); the last layer emits a~ itself
     float *fwd_out = q_a ? at : a_out;
@@ -283,8 +287,10 @@ minw_status minw_fc_train_step(const float *A, float *W, const float *g_out, int
                     nullptr, s));
     // 1.2 backward through the activation AQE (Eq. activation): g_a~ = 2 alpha g 1[|a~| <= 1], as bf16
     // [B][Op] and [O][B]; a_l = alpha h(a~) + (1 - alpha) a~
-    prep_kernel<2><<<dim3((unsigned)(Op / 64), (unsigned)(B / 32)), 256, 0, s>>>(
-        q_a ? at : g_out, g_out, B, O, Op, B, alpha, qa, gb, gtb, q_a ? a_out : nullptr, nullptr, nullptr, 0);
+    if (launch_pdl(prep_kernel<2>, dim3((unsigned)(Op / 64), (unsigned)(B / 32)), dim3(256), 0, s,
+                   (const float *)(q_a ? at : g_out), g_out, B, O, Op, B, alpha, qa, gb, gtb, q_a ? a_out : fnone, fnone,
+                   fnone, 0) != cudaSuccess)
+        return MINW_ECUDA;
     TRY(launch_status());
     if (g_in)                                          // g_a = g_a~ W^  ([B][K], reduction over O)
         TRY(conv2d_bf16(gb, B, Op, 1, 1, wtb, K, 1, 1, q_w->bits, 1, 0, 0, ones, zeros, g_in, split, L.split_bytes,
