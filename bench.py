@@ -595,7 +595,8 @@ def run_gpu(args, rank, world, local_rank):
 
     # roofline of the dominant kernel: the quantized convolution (every op in q_ops_idx)
     variants = net.layer_variants()
-    q_ms = float(sum(layer_ms[i] for i in q_ops_idx))
+    fused = wl.name in ("wresnet110", "wdense100") and net.kernels == 1     # the forward is one kernel
+    q_ms = ms_max if fused else float(sum(layer_ms[i] for i in q_ops_idx))
     q_ops = 2.0 * sum(macs[i] for i in q_ops_idx) * BATCH
     achieved = q_ops / (q_ms * 1e-3) / 1e12
     tc_kind = {minw.VARIANT_TC: "e4m3", minw.VARIANT_TC_E2M1: "e2m1", minw.VARIANT_TC_E2M1_PAIRS: "e2m1",
@@ -604,20 +605,23 @@ def run_gpu(args, rank, world, local_rank):
         tc_kind = {minw.VARIANT_TC: "bf16"}
     all_tc = all(variants[i] in tc_kind for i in q_ops_idx)
     if wl.name == "wresnet110":
-        roofline = {"bound": "tensor", "kernel": "conv_tc_kernel<0, *, bf16> (tcgen05 kind::f16, the 110 block "
-                                                 "and shortcut convolutions)",
+        roofline = {"bound": "tensor", "kernel": "wres_fused_kernel (the whole forward; tcgen05 kind::f16)" if fused
+                    else "conv_tc_kernel<0, *, bf16> (tcgen05 kind::f16, the 110 block and shortcut convolutions)",
                     "achieved": achieved, "peak": BF16_TFLOPS, "unit": "TFLOP/s", "frac": achieved / BF16_TFLOPS,
                     "traffic": None, "layer_kinds": ["bf16"] * len(q_ops_idx),
                     "peak_basis": "measured dense bf16 TFLOP/s (burst), of measured; achieved counts the unpadded "
-                                  "MACs (16- and 32-channel layers run on operands padded to 64 channels)"}
+                                  "MACs of the quantized convolutions" + ("" if fused else " (16- and 32-channel "
+                                  "layers run on operands padded to 64 channels)")}
     elif wl.name == "wdense100":
-        roofline = {"bound": "tensor", "kernel": "conv_tc_kernel<0, *, bf16> (tcgen05 kind::f16, the 96 "
-                                                 "bottleneck-layer and 2 transition convolutions)",
+        roofline = {"bound": "tensor", "kernel": "wdense_fused_kernel (the whole forward; tcgen05 kind::f16)" if fused
+                    else "conv_tc_kernel<0, *, bf16> (tcgen05 kind::f16, the 96 bottleneck-layer and 2 transition "
+                         "convolutions)",
                     "achieved": achieved, "peak": BF16_TFLOPS, "unit": "TFLOP/s", "frac": achieved / BF16_TFLOPS,
                     "traffic": None, "layer_kinds": ["bf16"] * len(q_ops_idx),
                     "peak_basis": "measured dense bf16 TFLOP/s (burst), of measured; achieved counts the unpadded "
-                                  "MACs (each 1x1 reads its channels padded to a multiple of 64, the 3x3 its 48 "
-                                  "padded to 64, and the 3x3 computes 12 output channels of a 16-wide MMA)"}
+                                  "MACs of the quantized convolutions (the 3x3 computes 12 output channels of a "
+                                  "16-wide MMA" + (")" if fused else "; each 1x1 reads its channels padded to a "
+                                  "multiple of 64, the 3x3 its 48 padded to 64)")}
     elif all_tc:
         roofline = tensor_roofline([2.0 * macs[i] * BATCH for i in q_ops_idx],
                                    [tc_kind[variants[i]] for i in q_ops_idx],
@@ -652,7 +656,8 @@ def run_gpu(args, rank, world, local_rank):
             "eff_tops": eff_tops,
             "layer_ms": [round(v, 5) for v in layer_ms.tolist()],
             "layer_ms_note": "per-op CUDA-event durations from a second pass of the same steps with an event "
-                             "after every op; the timed steps run without them",
+                             "after every op; the timed steps run without them" +
+                             (" (and as one kernel, while a timed forward goes layer by layer)" if fused else ""),
             "roofline": roofline, "cpu_baseline": cpu, "cpu_baseline_all_cores": cpu_all,
             "e2e": {"value": replica_throughput(BATCH, world, e2e_sec), "unit": "images/s",
                     "h2d_bytes_per_step": int(x_host.numel() * 4),

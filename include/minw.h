@@ -800,8 +800,9 @@ MINW_API minw_status minw_get_last_device_error(void *stream);
  * to networks created after it (a network keeps the plan it was created
  * with, except pdl and graph, read at every forward).
  * - cta_pairs: 256-channel layers with long K loops as CTA pairs (cta_group::2).
- * - channel_major: 64- and 128-channel layers as 128-channel x 256-pixel tiles
- *   when at least channel_major_min_tiles_per_sm such tiles per SM exist.
+ * - channel_major: 3 x 3 layers of stride 1 on rows of 64 or 128 bytes as 16 x 8-pixel
+ *   tiles loaded once with their halo; other 64- and 128-channel layers as 128-channel x
+ *   256-pixel tiles when at least channel_major_min_tiles_per_sm such tiles per SM exist.
  * - dup_weights: a 64-channel channel-major tile loads its weight rows twice
  *   (else pads with zero rows).
  * - kblocks_per_stage: K blocks per pipeline stage of the tensor-core kernel (1 or 2).
