@@ -1413,22 +1413,42 @@ __global__ void __launch_bounds__(NT, 1)
                     }
                 }
                 const int ob = o0 + ch * 16;
+                // NCHW outputs: one address and a channel stride, and the group's BN maps in wide loads (an address
+                // and two loads per element held the fp32 products of the convolutional training step: 78 us
+                // each at 256 x 256 x 16 x 16, 62 here)
                 if (p.acc_out != nullptr && valid) {
+                    int32_t *d = p.acc_out + (((long long)b * p.O + ob) * p.Ho + y) * p.Wo + x;
+                    const long long cst = (long long)p.Ho * p.Wo;
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
-                        if (ob + j < p.O)
-                            p.acc_out[(((long long)b * p.O + ob + j) * p.Ho + y) * p.Wo + x] = __float2int_rn(a[j]);
+                        if (ob + j < p.O) d[j * cst] = __float2int_rn(a[j]);
                 }
                 const bool resid = p.res_codes != nullptr || p.res_f32 != nullptr || p.y_nhwc != nullptr;
                 if (p.y_out != nullptr && writer && !resid) {
+                    float *d = p.y_out + (((long long)b * p.O + ob) * Hp + yp) * Wp + xp;
+                    const long long cst = (long long)Hp * Wp;
+                    const float *sp = p.scale + ob, *hp = p.shift + ob;
+                    if (ob + 16 <= p.O && ((reinterpret_cast<uintptr_t>(sp) | reinterpret_cast<uintptr_t>(hp)) & 15) == 0) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int o = ob + j;
-                        if (o < p.O) {
-                            float yv = fmaf(a[j], __ldg(p.scale + o), __ldg(p.shift + o));
-                            if (OUTB > 0) yv = fminf(fmaxf(yv, -1.0f), 1.0f);
-                            p.y_out[(((long long)b * p.O + o) * Hp + yp) * Wp + xp] = yv;
+                        for (int k = 0; k < 4; ++k) {
+                            const float4 c = __ldg(reinterpret_cast<const float4 *>(sp) + k);
+                            const float4 h = __ldg(reinterpret_cast<const float4 *>(hp) + k);
+                            const float cc[4] = {c.x, c.y, c.z, c.w}, hh[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                float yv = fmaf(a[4 * k + e], cc[e], hh[e]);
+                                if (OUTB > 0) yv = fminf(fmaxf(yv, -1.0f), 1.0f);
+                                d[(4 * k + e) * cst] = yv;
+                            }
                         }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            if (ob + j < p.O) {
+                                float yv = fmaf(a[j], __ldg(sp + j), __ldg(hp + j));
+                                if (OUTB > 0) yv = fminf(fmaxf(yv, -1.0f), 1.0f);
+                                d[j * cst] = yv;
+                            }
                     }
                 }
                 if (p.hb_out != nullptr && writer) {
