@@ -26,8 +26,8 @@
 // operand row) and, for raw outputs, the int32 / fp32 stores.  The popcount
 // kernel spends 2 P_a P_w popcounts per 32 products at 16 a clock and SM; on a
 // 256 x 512 x 14 x 14, 3x3, 3-bit x 3-bit layer (quantize + convolve, raw and
-// fp32 outputs) it took 8.24 ms, this kernel 0.26 ms (0.33 before loads by pairs
-// of lanes); a 4 x 128 x 32 x 32, 1-bit x 1-bit layer 32.8 -> 19.5 us.
+// fp32 outputs) it took 8.24 ms, this kernel 0.24 ms (0.33 before loads by pairs
+// of lanes and BN maps in wide loads); a 4 x 128 x 32 x 32, 1-bit x 1-bit layer 32.8 -> 19.5 us.
 //
 // Every mbarrier wait is bounded; one that runs out sets this file's error
 // flag (read by minw_get_last_device_error) and the CTA winds down.
@@ -328,10 +328,8 @@ __device__ __forceinline__ void store_group(const ConvArgs &a, const uint32_t (&
     }
     if (a.y_out == nullptr && OUTB == 0) return;
     uint32_t w[3] = {0u, 0u, 0u};
-#pragma unroll
-    for (int c = 0; c < 32; ++c) {
-        if (c >= nv) break;
-        const float y = fmaf(__uint_as_float(v[c]), __ldg(a.scale + o0 + c), __ldg(a.shift + o0 + c));
+    auto one = [&](int c, float sc, float sh) {
+        const float y = fmaf(__uint_as_float(v[c]), sc, sh);
         if constexpr (OUTB > 0) {
             const uint32_t pb = planes_of_y<OUTB>(y, a.qo);
 #pragma unroll
@@ -339,6 +337,23 @@ __device__ __forceinline__ void store_group(const ConvArgs &a, const uint32_t (&
         }
         if (a.y_out != nullptr)
             __stcs(a.y_out + at + (long long)c * HoWo, OUTB > 0 ? fminf(fmaxf(y, -1.0f), 1.0f) : y);
+    };
+    const float *sp = a.scale + o0, *hp = a.shift + o0;
+    if (nv == 32 && ((reinterpret_cast<uintptr_t>(sp) | reinterpret_cast<uintptr_t>(hp)) & 15) == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 s = __ldg(reinterpret_cast<const float4 *>(sp) + k), h = __ldg(reinterpret_cast<const float4 *>(hp) + k);
+            one(4 * k, s.x, h.x);
+            one(4 * k + 1, s.y, h.y);
+            one(4 * k + 2, s.z, h.z);
+            one(4 * k + 3, s.w, h.w);
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+            if (c >= nv) break;
+            one(c, __ldg(sp + c), __ldg(hp + c));
+        }
     }
     if constexpr (OUTB > 0) {
         const int NWo = (a.O + 31) >> 5;
