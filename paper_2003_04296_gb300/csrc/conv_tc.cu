@@ -2200,18 +2200,24 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     p.nk = a.kh * a.kw * p.nck;
     p.nbb = (a.B + p.bb - 1) / p.bb;
     p.ntn = (a.O + p.BN - 1) / p.BN;
-    // the weight update of a fully connected layer is bound by its epilogue, whose time is waves x columns per
-    // warp: the width with the least of it (1024 x 8192 on 152 SMs: 296 tiles of 224 columns, two full waves,
-    // instead of 256 of 256: 29.4 -> 28.1 us cold, the step 84.6 -> 82.5)
-    if (a.upd && !p.trans) {
+    // fp32 outputs of a fully connected product of bf16 operands: the tile width with the least waves x columns
+    // per epilogue warp (weight update 1024 x 8192 on 152 SMs: 296 tiles of 224 columns, two full waves, instead of
+    // 256 of 256: 29.4 -> 28.1 us cold; input gradient 256 x 8192: 128 tiles of 128 instead of 64 of 256); where the
+    // product splits along K, half the width halves the slices and their partial sums
+    if (a.bf16 && !p.trans && a.Ho == 1 && a.Wo == 1 && a.y_out != nullptr && !a.pool && p.BN > 128) {
         const int sms_ = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
-        long long best = -1;
-        for (int bn = p.BN, first = bn; bn >= 128 || bn == first; bn -= 16) {
-            const long long t = (long long)p.nbx * p.nby * p.nbb * ((a.O + bn - 1) / bn);
-            const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
-            if (best < 0 || cost < best) {
-                best = cost;
-                p.BN = bn;
+        const long long tm = (long long)p.nbx * p.nby * p.nbb;
+        if (a.workspace != nullptr && !a.upd && auto_ksplit((int)std::min<long long>(tm * p.ntn, 1 << 30), p.nk, sms_) > 1) {
+            p.BN = 128;
+        } else {
+            long long best = -1;
+            for (int bn = p.BN, first = bn; bn >= 128 || bn == first; bn -= 16) {
+                const long long t = tm * ((a.O + bn - 1) / bn);
+                const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    p.BN = bn;
+                }
             }
         }
         p.ntn = (a.O + p.BN - 1) / p.BN;
