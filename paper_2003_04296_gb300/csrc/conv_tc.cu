@@ -2202,22 +2202,22 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     p.ntn = (a.O + p.BN - 1) / p.BN;
     // fp32 outputs of a fully connected product of bf16 operands: the tile width with the least waves x columns
     // per epilogue warp (weight update 1024 x 8192 on 152 SMs: 296 tiles of 224 columns, two full waves, instead of
-    // 256 of 256: 29.4 -> 28.1 us cold; input gradient 256 x 8192: 128 tiles of 128 instead of 64 of 256); where the
-    // product splits along K, half the width halves the slices and their partial sums
+    // 256 of 256: 29.4 -> 28.1 us cold; input gradient 256 x 8192: 128 tiles of 128 instead of 64 of 256).  A product
+    // that splits along K keeps its full width: the number of tiles sets the slices and with them the order of the
+    // fp32 sums (128 columns on the 256 x 8192 -> 1024 forward, 9 slices instead of 19: the step 74.2 us instead of
+    // 78.6, and levels of a~ that lie at a threshold flip)
     if (a.bf16 && !p.trans && a.Ho == 1 && a.Wo == 1 && a.y_out != nullptr && !a.pool && p.BN > 128) {
         const int sms_ = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
         const long long tm = (long long)p.nbx * p.nby * p.nbb;
-        if (a.workspace != nullptr && !a.upd && auto_ksplit((int)std::min<long long>(tm * p.ntn, 1 << 30), p.nk, sms_) > 1) {
-            p.BN = 128;
-        } else {
-            long long best = -1;
-            for (int bn = p.BN, first = bn; bn >= 128 || bn == first; bn -= 16) {
-                const long long t = tm * ((a.O + bn - 1) / bn);
-                const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
-                if (best < 0 || cost < best) {
-                    best = cost;
-                    p.BN = bn;
-                }
+        const bool split = a.workspace != nullptr && !a.upd &&
+                           auto_ksplit((int)std::min<long long>(tm * p.ntn, 1 << 30), p.nk, sms_) > 1;
+        long long best = -1;
+        for (int bn = p.BN, first = bn; !split && (bn >= 128 || bn == first); bn -= 16) {
+            const long long t = tm * ((a.O + bn - 1) / bn);
+            const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
+            if (best < 0 || cost < best) {
+                best = cost;
+                p.BN = bn;
             }
         }
         p.ntn = (a.O + p.BN - 1) / p.BN;

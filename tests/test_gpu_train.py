@@ -189,6 +189,39 @@ def test_train_step(dev, M, case, last):
     assert np.abs(W1).max() <= 1.0
 
 
+def _sliced_sum(A, slices):
+    """Row sums of A over its blocks of 64 columns as K slices give them: each
+    slice exact, the slices added in order in fp32."""
+    nk = A.shape[1] // 64
+    t = np.zeros(A.shape[0], np.float32)
+    for s in range(slices):
+        part = A[:, 64 * (s * nk // slices):64 * ((s + 1) * nk // slices)].astype(np.float64).sum(1)
+        assert (np.abs(part) < 2 ** 24).all()
+        t = t + part.astype(np.float32)
+    return t
+
+
+def test_forward_slices(dev, M):
+    """The K slices of the step's forward product are those of its full-width
+    tiles (256 x 256 outputs a column of tiles, one slice per SM and tile), so
+    that a~ keeps the order of its fp32 sums.  W^ = 1 and whole inputs below
+    2^24 a slice: every slice is exact and only the additions between slices
+    round, which another number of slices would show."""
+    B, K, O_ = 256, 8192, 1024
+    r = np.random.default_rng(3)
+    A = np.where(r.random((B, K)) < 0.5, 16384.0, 1.0 + 2.0 * r.integers(0, 64, (B, K))).astype(np.float32)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slices = sms // ((B // 128) * (O_ // 256))
+    want = _sliced_sum(A, slices)
+    assert (want != _sliced_sum(A, slices // 2)).any()
+    W = torch.full((O_, K), 0.5, device=dev)
+    G, a1, pre = (torch.zeros((B, O_), device=dev) for _ in range(3))
+    ws = torch.empty(M.minw_fc_train_workspace_bytes(B, K, O_), dtype=torch.uint8, device=dev)
+    M.minw_fc_train_step(dev_tensor(A, dev), W, G, 1.0, 0.0, M.quant(1, DEFAULT_THR[1]), M.quant(1, DEFAULT_THR[1]), a1,
+                         None, ws, a_pre=pre)
+    assert np.array_equal(pre.cpu().numpy(), np.repeat(want[:, None], O_, 1))
+
+
 def test_train_step_errors(dev, M):
     A = torch.zeros((64, 100), device=dev)
     W = torch.zeros((8, 100), device=dev)
