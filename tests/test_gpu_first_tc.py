@@ -102,6 +102,94 @@ def test_first_tc_levels(dev, M, restore, case, bits_out):
     assert np.array_equal(_gpu_planes(dev, M, x, w, s, pad, scale, shift, bits_out, bw, cs, tc=False), ref)
 
 
+def _breakpoint(bits):
+    """The smallest fp32 y of the quantizer's top level (its last breakpoint on BN outputs)."""
+    lo, hi = np.float32(-1.0), np.float32(1.0)
+    top = O.quantize(np.array([hi]), bits, DEFAULT_THR[bits])[0]
+    while np.nextafter(lo, hi) < hi:
+        mid = np.float32((lo.astype(np.float64) + hi) / 2)
+        mid = np.nextafter(lo, hi) if mid <= lo or mid >= hi else mid
+        if O.quantize(np.array([mid]), bits, DEFAULT_THR[bits])[0] == top:
+            hi = mid
+        else:
+            lo = mid
+    return hi
+
+
+def _close_decisions(seed, B, C, hw, O_, k, close, bits_out):
+    """Inputs 1 + 2^-19 N(0, 1) and, on every ``close``-th channel, weights
+    that sum to zero with a breakpoint at acc = 0: there the fp32 chain's
+    rounding decides a good share of the outputs, against the exact sum."""
+    r = np.random.default_rng(seed)
+    x = (1.0 + 2.0 ** -19 * r.standard_normal((B, C, hw, hw))).astype(np.float32)
+    w = r.normal(0, 0.05, (O_, C, k, k)).astype(np.float32)
+    w[::close] -= w[::close].mean(axis=(1, 2, 3), keepdims=True)
+    scale, shift = _bn(r, O_, C * k * k)
+    scale[::close], shift[::close] = 1.0, _breakpoint(bits_out)
+    return x, w, scale, shift
+
+
+# B, C, image, O, k, stride, patch slots of the plan (shared memory left after the weights), open decisions per tile
+SLOTS = [
+    (16, 3, 128, 128, 7, 2, "1 slot"),
+    (60, 3, 32, 256, 5, 1, "1 slot, no lists"),
+    (240, 4, 16, 192, 5, 1, "1 slot"),
+    (60, 3, 64, 128, 7, 2, "2 slots"),
+    (240, 8, 16, 192, 3, 1, "3 slots"),
+    (60, 3, 32, 64, 3, 1, "4 slots"),
+]
+
+
+@pytest.mark.parametrize("close", [64, 8], ids=["listed", "overflow"])
+@pytest.mark.parametrize("case", SLOTS, ids=lambda c: "x".join(map(str, c[:6])) + " " + c[6])
+def test_first_tc_tiles_in_turn(dev, M, restore, case, close):
+    """At least three tiles per CTA, so that patch slots and lists of open
+    decisions are used again, at every number of slots; one channel in 64 whose
+    outputs are all open fills half a list per 64 channels, one in 8
+    overflows it.  Against the CUDA-core kernel on every image, the oracle on the
+    first and the last."""
+    B, C, hw, O_, k, s, _ = case
+    bits_out = 1 + (hw + O_ // 64 + close) % 3
+    x, w, scale, shift = _close_decisions(hw + close, B, C, hw, O_, k, close, bits_out)
+    got = _gpu_planes(dev, M, x, w, s, k // 2, scale, shift, bits_out)
+    pick = [0, B - 1]
+    ref = _ref_planes(x[pick], w, s, k // 2, scale, shift, bits_out)
+    assert np.array_equal(got[pick], ref)
+    # the chain, not the exact sum, decided some of them
+    exact = O.conv2d_real(x[pick].astype(np.float64), w.astype(np.float64), s, k // 2)
+    assert (O.pack(O.quantize(O.hardtanh(O.affine(exact.astype(np.float32), scale, shift)), bits_out,
+                              DEFAULT_THR[bits_out]), bits_out) != ref).any()
+    assert np.array_equal(got, _gpu_planes(dev, M, x, w, s, k // 2, scale, shift, bits_out, tc=False))
+
+
+@pytest.mark.parametrize("variant", ["VARIANT_TC_E2M1", "VARIANT_TC_E4M3"])
+@pytest.mark.parametrize("close", [64, 8], ids=["listed", "overflow"])
+@pytest.mark.parametrize("bits", [1, 2, 3])
+def test_first_tc_codes(dev, M, restore, bits, close, variant):
+    """The corrections on level codes, E2M1 nibbles and E4M3 bytes, through a
+    network's first layer of four tiles per CTA: logits equal the oracle's on
+    the first and last image, and the CUDA-core first layer's on all."""
+    B, hw, O_ = 76, 32, 128
+    p = convnet_params(31 + bits, bits_a=bits, bits_w=2, widths=(O_, 64), pools=(False, True), fcs=(), hw=hw)
+    x, _, _, _ = _close_decisions(bits, B, 3, hw, O_, 3, close, bits)
+    r = np.random.default_rng(bits)
+    l0 = p["layers"][0]
+    for o in range(0, O_, close):                        # levels +-1 and one 0 that sum to zero
+        l0["w"][o] = r.permutation([0.1] * 13 + [-0.1] * 13 + [0.0]).reshape(3, 3, 3)
+        l0["w_scale"][o], l0["scale"][o], l0["shift"][o] = 10.0, 1.0, _breakpoint(bits)
+    got = []
+    for tc in (1, 0):
+        M.set_plan_options(first_tensor_cores=tc)
+        net = M.Net(M.layer_descs(p, dev), max_batch=B, variant=getattr(M, variant))
+        logits = torch.empty((B, 10), dtype=torch.float32, device=dev)
+        net.forward(dev_tensor(x, dev), logits)
+        assert M.minw_get_last_device_error() == M.MINW_OK
+        got.append(logits.cpu().numpy())
+        net.close()
+    assert np.array_equal(got[0], got[1])
+    assert np.array_equal(got[0][[0, B - 1]], N.convnet_forward(p, x[[0, B - 1]]))
+
+
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 def test_first_tc_exact_ties(dev, M, restore, sign):
     """Inputs on the 2^-6 grid and +-1 weights: every accumulator is an exact
