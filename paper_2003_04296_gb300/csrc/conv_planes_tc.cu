@@ -48,7 +48,7 @@ constexpr int NT = NPROD + 32;
 constexpr int ROWB = 64;                 // bytes of one operand row of a chunk: 128 E2M1 channels
 constexpr int CW = 4;                    // 32-channel words per chunk
 constexpr int SMAX = 6;
-constexpr int POOL_LD = BM + 1;          // padded channel row of the pooling stage
+constexpr int POOL_LD = BM + 2;          // padded channel row of the pooling stage (pairs of pixels load at once)
 
 struct Params {
     ConvArgs a;
@@ -364,36 +364,43 @@ __device__ __forceinline__ void store_group(const ConvArgs &a, const uint32_t (&
 }
 
 // Epilogue of one 32-channel group with the 2x2 max pool: the group's
-// accumulators in shared memory [channel][pixel], lane = channel, warp q of
-// four takes pooled pixels q, q + 4, ... of the tile's 32.
+// accumulators in shared memory [channel][pixel], lane = one of the tile's 32
+// pooled pixels (consecutive in the output), warp q of four takes channels 8 q
+// .. 8 q + 7: one byte of each plane word, and whole lines of y_out.  With a
+// channel per lane and the pixels in turn a 1x1 layer of 32 -> 32 channels, 2 x 2
+// bits, 160 images of 32 x 32, took 29.1 us (1-bit planes) and 28.8 (fp32) against
+// 25.1 and 18.6 of the popcount kernel; 19.9 and 19.8 here.
 template <int OUTB>
 __device__ __forceinline__ void store_pooled(const ConvArgs &a, const float *acc, int o0, long long m0, int q,
                                              int lane) {
-    const int o = o0 + lane, HoWo = a.Ho * a.Wo, half = a.Wo / 2, Wp = half, HpWp = (a.Ho / 2) * Wp;
-    const bool live = o < a.O;
-    const float sc = live ? __ldg(a.scale + o) : 0.0f, sh = live ? __ldg(a.shift + o) : 0.0f;
+    const int HoWo = a.Ho * a.Wo, half = a.Wo / 2, HpWp = (a.Ho / 2) * half;
     const int NWo = (a.O + 31) >> 5;
-    for (int t = q; t < BM / 4; t += 4) {
-        const int pr = t / half, r00 = 2 * pr * a.Wo + 2 * (t - pr * half);
-        const long long m = m0 + r00;
-        if (m >= a.M) break;
-        const long long b = m / HoWo;
-        const int pix = (int)(m - b * HoWo), yo = pix / a.Wo, xo = pix - yo * a.Wo;
-        const long long op = (long long)(yo / 2) * Wp + xo / 2;
-        const float *p = acc + lane * POOL_LD + r00;
-        const float v = fmaxf(fmaxf(p[0], p[1]), fmaxf(p[a.Wo], p[a.Wo + 1]));
-        const float y = fmaf(v, sc, sh);
-        if (a.y_out != nullptr && live)
+    const int pr = lane / half, r00 = 2 * (pr * a.Wo + lane - pr * half);
+    const long long m = m0 + r00;
+    if (m >= a.M) return;
+    const long long b = m / HoWo;
+    const int pix = (int)(m - b * HoWo), yo = pix / a.Wo, xo = pix - yo * a.Wo;
+    const long long op = (long long)(yo / 2) * half + xo / 2;
+    uint32_t w[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int c = 8 * q + e, o = o0 + c;
+        if (o >= a.O) break;
+        const float *p = acc + c * POOL_LD + r00;
+        const float2 r0 = *reinterpret_cast<const float2 *>(p), r1 = *reinterpret_cast<const float2 *>(p + a.Wo);
+        const float y = fmaf(fmaxf(fmaxf(r0.x, r0.y), fmaxf(r1.x, r1.y)), __ldg(a.scale + o), __ldg(a.shift + o));
+        if (a.y_out != nullptr)
             a.y_out[(b * a.O + o) * HpWp + op] = OUTB > 0 ? fminf(fmaxf(y, -1.0f), 1.0f) : y;
         if constexpr (OUTB > 0) {
-            const uint32_t pb = live ? planes_of_y<OUTB>(y, a.qo) : 0u;
-            uint32_t *dst = a.planes_out + ((b * HpWp + op) * OUTB) * NWo + (o0 >> 5);
+            const uint32_t pb = planes_of_y<OUTB>(y, a.qo);
 #pragma unroll
-            for (int u = 0; u < OUTB; ++u) {
-                const uint32_t w = __ballot_sync(0xffffffffu, (pb >> u) & 1u);
-                if (lane == u) dst[u * NWo] = w;
-            }
+            for (int u = 0; u < OUTB; ++u) w[u] |= ((pb >> u) & 1u) << e;
         }
+    }
+    if constexpr (OUTB > 0) {
+        uint8_t *dst = reinterpret_cast<uint8_t *>(a.planes_out + (b * HpWp + op) * OUTB * NWo + (o0 >> 5)) + q;
+#pragma unroll
+        for (int u = 0; u < OUTB; ++u) dst[4 * u * NWo] = (uint8_t)w[u];
     }
 }
 

@@ -117,6 +117,50 @@ def test_exact_against_oracle(M, ba, bw):
         assert np.array_equal(acc.cpu().numpy(), ref)
 
 
+def _replay_us(call):
+    """Least time of a pass, 20 of them in a graph."""
+    call()
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        for _ in range(20):
+            call()
+    best = float("inf")
+    for _ in range(12):
+        a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+        a.record()
+        g.replay()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 50)
+    return best
+
+
+# B, C, side, O, bits of activations, weights and outputs (0: fp32), pool
+SHORT = [
+    (160, 32, 32, 64, 2, 2, 1, 1),
+    (160, 32, 32, 64, 1, 1, 3, 1),
+    (160, 64, 32, 96, 2, 1, 0, 1),
+]
+
+
+@pytest.mark.parametrize("case", SHORT)
+def test_auto_is_not_slower_than_popcount(M, case):
+    """1x1 layers of one or two words, where a tile's fixed cost and its
+    epilogue are all there is: the kernel that the automatic choice runs takes
+    at most a tenth more than the popcount kernel."""
+    B, C, side, O_, ba, bw, bo, pool = case
+    _, _, act, wgt, scale, shift = _operands(M, B, C, side, side, O_, 1, ba, bw, sum(case))
+    h = side >> pool
+    y = torch.empty((B, O_, h, h), device="cuda")
+    planes = torch.empty(M.packed_words(B, O_, h, h, max(bo, 1)), dtype=torch.int32, device="cuda")
+    q = M.quant(bo, DEFAULT_THR[bo]) if bo else None
+    us = [_replay_us(lambda: M.minw_conv_block(act, B, C, side, side, ba, wgt, O_, 1, 1, bw, 1, 0, pool, scale, shift, q,
+                                               planes if bo else None, None if bo else y, variant=v))
+          for v in (M.VARIANT_AUTO, M.VARIANT_POPC)]
+    assert us[0] <= 1.1 * us[1], us
+
+
 def test_timeout_path(M):
     """A stalled MMA issuer: the bounded waits run out, the status is reported
     once, and the next launch is correct."""
