@@ -173,8 +173,9 @@ enum {
  * y_out (nullable): fp32 NCHW, y = fmaf((float)acc, scale[o], shift[o]);
  *   scale/shift (length O) are required when y_out is given.
  * variant: MINW_VARIANT_AUTO (the tensor cores, the planes expanded to level
- * codes inside the kernel, for kh kw C < 2^20; else the popcount path) or
- * MINW_VARIANT_POPC; both give the same bits.  At least one output must be
+ * codes inside the kernel, for kh kw C < 2^20 except the shortest 1 x 1
+ * contractions; else the popcount path) or MINW_VARIANT_POPC; both give the
+ * same bits.  At least one output must be
  * non-null.
  * Errors: MINW_EINVAL (sizes, pointers, bits), MINW_EUNSUPPORTED (C % 32,
  * a variant that does not cover the shape). */

@@ -44,13 +44,38 @@ int choose_variant(const ConvArgs &a, int requested) {
     return conv_tc_supported(a) ? MINW_VARIANT_TC : MINW_VARIANT_POPC;
 }
 
-// Packed-plane operands: the popcount path on request, else the tensor cores
-// with the planes expanded on the way (conv_planes_tc.cu) wherever that kernel
-// covers the shape.  The kernels on level codes (MINW_VARIANT_TC) take their
-// operands in the codes layout (minw_conv2d_codes / minw_conv_block_codes).
+// Contractions too short for the tensor cores' fixed cost per tile (set-up,
+// expansion of a chunk of four words that is not filled, tensor memory,
+// epilogue): 1x1 kernels of one to three words and few output channels, where
+// popcounts cost less.  A word pair's work is in tenths of the 1-bit one's, as
+// measured; the limits are where the two kernels meet.  160 images of 32 x 32,
+// raw accumulators, popcount : tensor cores in us: 32 -> 8 channels, 2 x 1 bits
+// 9.6 : 16.6; 32 -> 64, 1 x 1 14.9 : 19.1; 32 -> 32, 3 x 1 14.6 : 17.8; 64 -> 32,
+// 1 x 1 14.2 : 17.2; 96 -> 8, 2 x 1 15.5 : 16.6; past the limits 32 -> 32, 1 x 3
+// 19.5 : 17.4; 32 -> 96, 1 x 1 24.6 : 21.5; 96 -> 8, 1 x 1 20.0 : 16.9.  Below two
+// tiles per SM nothing is gained.
+static bool popcount_shorter(const ConvArgs &a) {
+    const int work[3][3] = {{11, 16, 0}, {9, 15, 0}, {20, 0, 0}};       // [activation bits - 1][weight bits - 1]
+    const int w = work[a.bits_a - 1][a.bits_w - 1] * a.NW;
+    if (a.kh != 1 || a.kw != 1 || w == 0) return false;
+    const int sms = num_sms() > 0 ? num_sms() : 152;
+    const long long tiles = (a.M + 127) / 128;
+    if (tiles < 2 * sms) return false;
+    if (a.O <= 8) return w <= (tiles < 4 * sms ? 24 : 30);
+    if (a.O <= 16) return w <= (!a.pool || !a.quant_out ? 22 : a.qo.bits == 1 ? 16 : 0);
+    if (a.O <= 64 && !a.quant_out)                                     // the popcount kernel's fp32 epilogue is the longer one
+        return w <= (a.y_out == nullptr ? 22 : a.acc_out == nullptr ? 15 : 0);
+    return false;
+}
+
+// Packed-plane operands: the popcount path on request and for the shortest
+// contractions, else the tensor cores with the planes expanded on the way
+// (conv_planes_tc.cu) wherever that kernel covers the shape.  The kernels on
+// level codes (MINW_VARIANT_TC) take their operands in the codes layout
+// (minw_conv2d_codes / minw_conv_block_codes).
 minw_status run_conv(const ConvArgs &a, int variant, cudaStream_t s) {
     if (variant == MINW_VARIANT_TC) return MINW_EUNSUPPORTED;
-    if (variant != MINW_VARIANT_POPC && planes_tc_supported(a)) return launch_planes_tc(a, s);
+    if (variant != MINW_VARIANT_POPC && planes_tc_supported(a) && !popcount_shorter(a)) return launch_planes_tc(a, s);
     return launch_conv_popc(a, s);
 }
 

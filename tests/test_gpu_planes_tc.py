@@ -136,11 +136,16 @@ def _replay_us(call):
     return best
 
 
-# B, C, side, O, bits of activations, weights and outputs (0: fp32), pool
+# B, C, side, O, bits of activations, weights and outputs (0: fp32, None: raw accumulators), pool
 SHORT = [
     (160, 32, 32, 64, 2, 2, 1, 1),
     (160, 32, 32, 64, 1, 1, 3, 1),
     (160, 64, 32, 96, 2, 1, 0, 1),
+    (160, 32, 32, 8, 2, 1, 2, 0),
+    (160, 32, 32, 16, 1, 1, 0, 0),
+    (160, 64, 32, 4, 2, 2, 1, 1),
+    (160, 32, 32, 64, 2, 2, None, 0),
+    (40, 64, 32, 40, 2, 1, None, 0),
 ]
 
 
@@ -150,14 +155,21 @@ def test_auto_is_not_slower_than_popcount(M, case):
     epilogue are all there is: the kernel that the automatic choice runs takes
     at most a tenth more than the popcount kernel."""
     B, C, side, O_, ba, bw, bo, pool = case
-    _, _, act, wgt, scale, shift = _operands(M, B, C, side, side, O_, 1, ba, bw, sum(case))
+    _, _, act, wgt, scale, shift = _operands(M, B, C, side, side, O_, 1, ba, bw, O_ + C)
     h = side >> pool
     y = torch.empty((B, O_, h, h), device="cuda")
-    planes = torch.empty(M.packed_words(B, O_, h, h, max(bo, 1)), dtype=torch.int32, device="cuda")
+    acc = torch.empty((B, O_, h, h), dtype=torch.int32, device="cuda")
+    planes = torch.empty(M.packed_words(B, O_, h, h, bo or 1), dtype=torch.int32, device="cuda")
     q = M.quant(bo, DEFAULT_THR[bo]) if bo else None
-    us = [_replay_us(lambda: M.minw_conv_block(act, B, C, side, side, ba, wgt, O_, 1, 1, bw, 1, 0, pool, scale, shift, q,
-                                               planes if bo else None, None if bo else y, variant=v))
-          for v in (M.VARIANT_AUTO, M.VARIANT_POPC)]
+
+    def call(variant):
+        if bo is None:
+            M.minw_conv2d(act, B, C, side, side, ba, wgt, O_, 1, 1, bw, 1, 0, acc, variant=variant)
+        else:
+            M.minw_conv_block(act, B, C, side, side, ba, wgt, O_, 1, 1, bw, 1, 0, pool, scale, shift, q,
+                              planes if bo else None, None if bo else y, variant=variant)
+
+    us = [_replay_us(lambda: call(v)) for v in (M.VARIANT_AUTO, M.VARIANT_POPC)]
     assert us[0] <= 1.1 * us[1], us
 
 
