@@ -174,13 +174,15 @@ def test_block_e2m1_pool(dev, M, ba, bw, hw, O_):
     assert np.array_equal(decode_e2m1(codes.cpu().numpy(), O_), (lv * 2.0 ** O.units_shift(bo)).transpose(0, 2, 3, 1))
 
 
-@pytest.mark.parametrize("O_,pool,bits", [(128, 1, 1), (128, 0, 3), (64, 0, 2)])
-def test_block_e2m1_channel_major(dev, M, O_, pool, bits):
-    """Codes-only outputs of a 64- or 128-channel layer with enough 256-pixel
-    tiles run as channel-major tiles (128 channels x 256 pixels); the E2M1
+@pytest.mark.parametrize("hw", [32, 20])
+@pytest.mark.parametrize("O_,pool,bits", [(128, 1, 1), (128, 0, 3), (64, 0, 2), (64, 1, 3)])
+def test_block_e2m1_channel_major(dev, M, O_, pool, bits, hw):
+    """Codes-only outputs of a 64- or 128-channel layer: halo tiles at 32 x 32,
+    and where those cover too little, with enough 256-pixel tiles,
+    channel-major ones (128 channels x 256 pixels) at 20 x 20; the E2M1
     output codes equal the E4M3 path's (decoded) on the whole batch, and the
     oracle's on the first and last image."""
-    B, C, hw = 160, 128, 32
+    B, C = (160 if hw == 32 else 208), 128
     p = conv_problem(91 + O_ + pool + bits, B, C, hw, hw, O_, 3, 3, 1, 1, bits, bits, w_sigma=0.5)
     act4, wgt4 = _operands(dev, M, p)
     act8 = torch.empty((B, hw, hw, C), dtype=torch.uint8, device=dev)

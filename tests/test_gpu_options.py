@@ -91,6 +91,22 @@ def test_options_keep_the_logits(dev, M, restore, opts, variant):
     assert M.minw_get_last_device_error() == M.MINW_OK
 
 
+@pytest.mark.parametrize("opts", [dict(), dict(dup_weights=0), dict(kblocks_per_stage=1), dict(tma_lanes=8)],
+                         ids=lambda d: ",".join(f"{k}={v}" for k, v in d.items()) or "default")
+@pytest.mark.parametrize("bits", [1, 3])
+def test_options_of_channel_major_tiles(dev, M, restore, opts, bits):
+    """Hidden layers that run channel-major for a small batch (18 x 18 and 9 x 9
+    images, of which halo tiles would cover 0.42 and 0.32): 64 -> 64 pooled,
+    whose weight rows are doubled or padded, and 64 -> 128."""
+    net_p = convnet_params(63, bits_a=bits, bits_w=bits, widths=(64, 64, 128), pools=(False, True, False),
+                           fcs=(), classes=10, hw=18)
+    x = convnet_input(64, 6, hw=18)
+    M.set_plan_options(channel_major_min_tiles_per_sm=0, **opts)
+    got = _net_logits(dev, M, net_p, x, variant=M.VARIANT_TC_E4M3)
+    assert np.array_equal(got, N.convnet_forward(net_p, x))
+    assert M.minw_get_last_device_error() == M.MINW_OK
+
+
 def test_options_round_trip_and_validation(M, restore):
     d = M.get_plan_options()
     assert d["cta_pairs"] == 1 and d["kblocks_per_stage"] == 2 and d["tma_lanes"] == 1 and d["wait_cycles"] == 1 << 31
