@@ -228,47 +228,51 @@ __global__ void __launch_bounds__(NT, 1)
 
 // W [O][C][taps] -= the step: the slices' partial sums added in order, then
 // Eq. weight's mask, the update and the clip in the fp32 operations of
-// aqe_backward and minw_sgd_clip.  A block takes 32 output channels x 32
+// aqe_backward and minw_sgd_clip.  A block takes 32 output channels x 8 RPT
 // consecutive (c, tap) of their rows through shared memory, as the partial
-// sums run along o and W along (c, tap); a thread has four slices of its four
-// (c, tap) in flight (one element and W strided per thread: 35 us at 256 x 256
-// x 3 x 3 in 16 slices; 19 us here, cold).
+// sums run along o and W along (c, tap); a thread has RPT rows of 16 / RPT slices
+// in flight (one element and W strided per thread: 35 us at 256 x 256 x 3 x 3 in
+// 16 slices; 19 us here, cold).  A small gradient has a slice per SM and few
+// blocks: 64 x 39 x 1 x 1, 96 images of 24 x 24, RPT = 4 the step 119.5 us, RPT = 1
+// 56.2.
+template <int RPT>
 __global__ void __launch_bounds__(256) wgrad_update_kernel(const float *__restrict__ part, int slices, int ntaps, int C,
                                                            int O, float lr, float two_alpha, float *__restrict__ W) {
-    __shared__ float tile[32][33];
+    constexpr int ROWS = 8 * RPT, E = 16 / RPT;
+    __shared__ float tile[ROWS][33];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
-    const int R = C * ntaps, r0 = blockIdx.x * 32;
+    const int R = C * ntaps, r0 = blockIdx.x * ROWS;
     const size_t n = (size_t)R * O;
     pdl_wait();                       // (and no early start of a dependent: it may read W before it waits)
     for (int o0 = blockIdx.y * 32; o0 < O; o0 += gridDim.y * 32) {
-        float acc[4];
-        const float *src[4];
+        float acc[RPT];
+        const float *src[RPT];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < RPT; ++k) {
             const int r = min(r0 + row + 8 * k, R - 1), c = r / ntaps, tap = r - c * ntaps;
             src[k] = part + ((size_t)tap * C + c) * O + min(o0 + lane, O - 1);
             acc[k] = 0.0f;
         }
         int s = 0;
-        for (; s + 4 <= slices; s += 4) {
-            float v[4][4];
+        for (; s + E <= slices; s += E) {
+            float v[E][RPT];
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
+            for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) v[e][k] = __ldcs(src[k] + (size_t)(s + e) * n);
+                for (int k = 0; k < RPT; ++k) v[e][k] = __ldcs(src[k] + (size_t)(s + e) * n);
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
+            for (int e = 0; e < E; ++e)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] += v[e][k];
+                for (int k = 0; k < RPT; ++k) acc[k] += v[e][k];
         }
         for (; s < slices; ++s)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[k] += __ldcs(src[k] + (size_t)s * n);
+            for (int k = 0; k < RPT; ++k) acc[k] += __ldcs(src[k] + (size_t)s * n);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) tile[row + 8 * k][lane] = acc[k];
+        for (int k = 0; k < RPT; ++k) tile[row + 8 * k][lane] = acc[k];
         __syncthreads();
-        for (int i = threadIdx.x; i < 32 * 32; i += 256) {
-            const int r = i & 31, o = i >> 5;
+        for (int i = threadIdx.x; i < ROWS * 32; i += 256) {
+            const int r = i % ROWS, o = i / ROWS;
             if (r0 + r < R && o0 + o < O) {
                 float *w = W + (size_t)(o0 + o) * R + r0 + r;
                 const float wi = *w;
@@ -354,9 +358,13 @@ minw_status launch_conv_wgrad(const WgradArgs &a, float *part, float lr, float t
     const unsigned grid = (unsigned)(p.nm * p.nn * p.ntg * p.slices);
     if (minw_host::launch_pdl(wg::conv_wgrad_kernel, dim3(grid), dim3(wg::NT), smem, s, tmG, tmA, p) != cudaSuccess)
         return MINW_ECUDA;
-    const dim3 ugrid((unsigned)((p.C * p.ntaps + 31) / 32), (unsigned)std::min((p.O + 31) / 32, 65535));
-    if (minw_host::launch_pdl(wg::wgrad_update_kernel, ugrid, dim3(256), 0, s, (const float *)part, p.slices, p.ntaps, p.C,
-                              p.O, lr, two_alpha, W) != cudaSuccess)
+    // narrow blocks where there are fewer than two wide ones per SM (the step at 64 images of 16 x 16, 128 -> 256
+    // channels, 288 wide blocks: 88.1 -> 83.0 us; above, the same time)
+    const int R = p.C * p.ntaps, ob = (p.O + 31) / 32;
+    const bool narrow = (long long)((R + 31) / 32) * ob < 2 * (minw_host::num_sms() > 0 ? minw_host::num_sms() : 152);
+    const dim3 ugrid((unsigned)(narrow ? (R + 7) / 8 : (R + 31) / 32), (unsigned)std::min(ob, 65535));
+    if (minw_host::launch_pdl(narrow ? wg::wgrad_update_kernel<1> : wg::wgrad_update_kernel<4>, ugrid, dim3(256), 0, s,
+                              (const float *)part, p.slices, p.ntaps, p.C, p.O, lr, two_alpha, W) != cudaSuccess)
         return MINW_ECUDA;
     return minw_host::launch_status();
 }

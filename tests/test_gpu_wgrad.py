@@ -30,6 +30,8 @@ def M():
     (16, 64, 32, 32, 300, 3, 3, 1, 1),     # two M groups
     (64, 64, 5, 5, 64, 5, 5, 1, 2),
     (1, 64, 64, 64, 32, 3, 3, 1, 1),
+    (96, 64, 24, 24, 39, 1, 1, 1, 0),      # a slice per SM: more than the update has in flight, with a remainder
+    (64, 256, 8, 8, 300, 3, 3, 1, 1),      # a gradient of many elements: the update's wide blocks
 ])
 def test_weight_gradient(M, B, C, H, W, O, kh, kw, stride, pad):
     g = torch.Generator(device="cuda").manual_seed(B + C + H + W + O)
@@ -53,3 +55,30 @@ def test_weight_gradient(M, B, C, H, W, O, kh, kw, stride, pad):
     err = (Wt.double() - (W0.double() - lr * ref)).abs()
     assert (err <= bound).all(), float((err / bound).max())
     assert M.minw_get_last_device_error() == M.MINW_OK
+
+
+def test_short_gradients_are_not_bound_by_the_slice_sums(M):
+    """A 1x1 layer's gradient has few elements, each the sum of a slice per SM:
+    its step takes less than that of the 3x3 layer of the same sizes, which
+    does nine times the products."""
+    B, C, S, O = 96, 64, 24, 39
+    g = torch.Generator(device="cuda").manual_seed(1)
+    A = torch.randn((B, C, S, S), generator=g, device="cuda") * 0.1
+    G = torch.randn((B, O, S, S), generator=g, device="cuda") * 0.1
+    a_out, g_in = torch.empty_like(G), torch.empty_like(A)
+    q = M.quant(2, DEFAULT_THR[2])
+    us = []
+    for k in (1, 3):
+        Wt = torch.rand((O, C, k, k), generator=g, device="cuda") * 2 - 1
+        ws = torch.empty(M.minw_conv_train_workspace_bytes(B, C, S, S, O, k, k, 1, k // 2), dtype=torch.uint8, device="cuda")
+        best = float("inf")
+        for i in range(30):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            for _ in range(5):
+                M.minw_conv_train_step(A, Wt, G, 1, k // 2, 0.75, 1e-4, q, q, a_out, g_in, ws)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 200 if i else best)
+        us.append(best)
+    assert us[0] <= 0.9 * us[1], us
