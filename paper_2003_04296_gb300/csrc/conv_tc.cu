@@ -808,45 +808,41 @@ __device__ __forceinline__ void rows_store16(uint32_t *sw, const uint32_t (&u)[1
 }
 
 // Tables of the epilogue warps (2 .. 9), filled by them all: the output
-// quantizer's breakpoints per channel, its sigma words, and for residual
-// blocks the BN maps and the breakpoints on y.  yt: scratch for T_1 .. T_{n-1}.
+// quantizer's breakpoints per channel (computed ones for the channels olo ..
+// ohi of the CTA's tiles), its sigma words, and for residual blocks the BN maps
+// and the breakpoints on y.  yt: scratch for T_1 .. T_{n-1}.
 template <int OUTB>
 __device__ __forceinline__ void epi_tables(const Params &p, bool resid, float *sthr, uint32_t *ssig, float *syt, float *yt,
-                                           int O32, int thr_floats, int sig_words, int et, int warp, int lane) {
+                                           int O32, int thr_floats, int sig_words, int et, int warp, int lane, int olo,
+                                           int ohi) {
     constexpr int NL = OUTB == 0 ? 1 : (OUTB == 1 ? 2 : (OUTB == 2 ? 3 : 7));
     // output-quantizer breakpoints of every channel, in shared memory
     if constexpr (OUTB > 0) {
         // held as (-T_1 .. -T_{n-1}, sigma) with -0 stored as +0, so that
         // fmaf(acc, sigma, -T) is never -0 and its sign bit is [sigma * acc < T]
         // rows u = 0 .. NL - 1 of O32 channels each (channel fastest: four channels per 128-bit load)
-        if (resid) {
-            // a residual block quantizes y + shortcut: no per-channel breakpoints on acc
-        } else if (p.thr != nullptr) {
+        if (!resid && p.thr != nullptr) {
             for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {
                 const float x = __ldg(p.thr + i);
                 const int o = i / NL, u = i - o * NL;
                 sthr[u * O32 + o] = (u == NL - 1) ? x : mask_breakpoint(x);
             }
         } else {
-            for (int i = et; i < p.O * NL; i += EPI_WARPS * 32) {      // one breakpoint (or sigma) per thread
-                const int o = i / NL, u = i - o * NL;
-                const float sc = __ldg(p.scale + o);
-                sthr[u * O32 + o] = (u == NL - 1) ? (sc < 0.0f ? -1.0f : 1.0f)
-                                                  : mask_breakpoint(channel_threshold(sc, __ldg(p.shift + o), p.qo, u + 1));
-            }
-        }
-        for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
-            const int k = i - p.O * NL, o = p.O + k / NL, u = k % NL;
-            sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
-        }
-        if (resid) {                                        // level of y = #{u : y >= T_u}
+            // the quantizer's own breakpoints on y, level = #{u : y >= T_u}, a warp each
             const int w8 = warp - 2;
             if (w8 < NL - 1) {
-                const float T = p.ythr != nullptr ? __ldg(p.ythr + w8) : y_threshold_warp(p.qo, w8 + 1);
+                const float T = resid && p.ythr != nullptr ? __ldg(p.ythr + w8) : y_threshold_warp(p.qo, w8 + 1);
                 if (lane == 0) yt[w8] = T;
             }
             asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");
-            if (et == 0) {
+            // (a residual block quantizes y + shortcut: no per-channel breakpoints on acc)
+            for (int i = et + olo * NL; i < min(ohi, p.O) * NL && !resid; i += EPI_WARPS * 32) {
+                const int o = i / NL, u = i - o * NL;                            // one breakpoint (or sigma) per thread
+                const float sc = __ldg(p.scale + o);
+                sthr[u * O32 + o] = (u == NL - 1) ? (sc < 0.0f ? -1.0f : 1.0f)
+                                                  : mask_breakpoint(channel_threshold_y(sc, __ldg(p.shift + o), yt[u]));
+            }
+            if (resid && et == 0) {
                 float t[8];
                 for (int u = 0; u < NL - 1; ++u) {
                     t[u] = yt[u];
@@ -860,6 +856,10 @@ __device__ __forceinline__ void epi_tables(const Params &p, bool resid, float *s
                               t[2 - e] == __uint_as_float(__float_as_uint(-t[3 + e]) - 1u);
                 syt[7] = sym ? 1.0f : 0.0f;
             }
+        }
+        for (int i = p.O * NL + et; i < thr_floats && !resid; i += EPI_WARPS * 32) {      // padding channels
+            const int k = i - p.O * NL, o = p.O + k / NL, u = k % NL;
+            sthr[u * O32 + o] = (u == NL - 1) ? 1.0f : 0.0f;
         }
         // sigma of a channel: the sign of its BN scale (+1 for 0); one warp per
         // 32-channel word, a lane per channel (one load latency for the word)
@@ -1175,8 +1175,12 @@ __global__ void __launch_bounds__(NT, 1)
             }
         }
         if (!p.planned) pdl_wait();
+        // channel tiles of this CTA's first and last item
+        const int w0 = cta_item(p, 0, items, tiles_m, crank);
+        const int w1 = p.wres || w0 < 0 ? w0 : w0 + (items - 1 - w0) / (int)gridDim.x * (int)gridDim.x;
         epi_tables<OUTB>(p, resid, sthr, ssig, syt, reinterpret_cast<float *>(tmem_slot + 1), O32, thr_floats, sig_words, et,
-                         warp, lane);
+                         warp, lane, w0 < 0 ? 0 : w0 / p.ksplit / tiles_m * p.BN,
+                         w0 < 0 ? 0 : (w1 / p.ksplit / tiles_m + 1) * p.BN);
         asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");   // breakpoints in place
         pdl_wait();                               // outputs, shortcuts and partial sums are shared with other kernels
         const int q = warp & 3;                   // TMEM lane quarter of this warp
@@ -1865,7 +1869,8 @@ __global__ void __launch_bounds__(halo::NT, 1)
         }
         const int set = (warp - 2) / EPI_WARPS;
         if (!p.planned) pdl_wait();
-        if (set == 0) epi_tables<OUTB>(p, resid, sthr, ssig, syt, yt, O32, thr_floats, sig_words, et, warp, lane);
+        if (set == 0)
+            epi_tables<OUTB>(p, resid, sthr, ssig, syt, yt, O32, thr_floats, sig_words, et, warp, lane, o0, o0 + p.BN);
         asm volatile("bar.sync 2, %0;\n" ::"n"(halo::SETS * EPI_WARPS * 32) : "memory");
         pdl_wait();
         const int q = warp & 3, half = ((warp - 2) >> 2) & 1, r = q * 32 + lane;

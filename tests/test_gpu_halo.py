@@ -145,9 +145,10 @@ def test_unaligned_shortcut(M, restore, res, off):
     _check(M, 3, 64, 16, 16, 64, 3, False, 0, res, off=off)
 
 
-def test_residual_with_bn_output(M, restore):
-    """The BN output before the shortcut as fp32 NHWC beside the levels."""
-    _check(M, 3, 128, 14, 14, 96, 2, False, 0, "codes", want_y=True)
+@pytest.mark.parametrize("res", ["codes", "f32", None])
+def test_residual_with_bn_output(M, restore, res):
+    """The BN output before the shortcut (or without one) as fp32 NHWC beside the levels."""
+    _check(M, 3, 128, 14, 14, 96, 2, False, 0, res, want_y=True)
 
 
 def test_halo_timeout(M, restore):

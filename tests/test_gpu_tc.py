@@ -283,3 +283,63 @@ def test_residual_block_epilogue(dev, M, shortcut, bits):
     assert np.array_equal(y.cpu().numpy(), yr)
     lv = O.quantize(yr, bits, DEFAULT_THR[bits])
     assert np.array_equal(decode_e4m3(codes.cpu().numpy()), (lv * 2.0 ** O.units_shift(bits)).transpose(0, 2, 3, 1))
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3])
+@pytest.mark.parametrize("C", [64, 512])
+def test_breakpoints_of_extreme_bn_maps(dev, M, bits, C):
+    """Per-channel breakpoints found in the kernel, over BN maps whose
+    breakpoints lie inside the accumulators' range, far outside it, at 0, at no
+    accumulator at all (scale 0), or where a rounding of y is worth many
+    accumulators (a large shift): levels equal the oracle's on all of them."""
+    B, hw = 3, 12
+    scales = np.array([0.0, -0.0, 1.0, -1.0, 1e-3, -1e-3, 0.02, -0.02, 3e-8, -3e-8, 1e-30, 1e30, -1e30, 0.25, 7.0, -1e-2],
+                      np.float32)
+    shifts = np.array([0.0, -0.0, 0.25, -0.75, 1e-6, 3.0, -4.0, 100.0, -100.0, 8e3, -8e3, 1e-30, 0.5, -0.125, 0.374999, 20.0],
+                      np.float32)
+    Oc = scales.size * shifts.size
+    p = conv_problem(C + bits, B, C, hw, hw, Oc, 1, 1, 1, 0, bits, bits, w_sigma=0.5)
+    p["scale"], p["shift"] = (a.ravel().copy() for a in np.meshgrid(scales, shifts, indexing="ij"))
+    p["shift"][::3] -= p["scale"][::3] * np.float32(20)        # breakpoints among the accumulators for large shifts too
+    act = torch.empty((B, hw, hw, C), dtype=torch.uint8, device=dev)
+    wgt = torch.empty((Oc, 1, 1, C), dtype=torch.uint8, device=dev)
+    M.aqe_quantize_codes(dev_tensor(p["x"], dev), M.quant(bits, p["thr_a"]), act)
+    M.minw_pack_weight_codes(dev_tensor(p["w"], dev), M.quant(bits, p["thr_w"]), wgt,
+                             channel_scale=dev_tensor(p["w_scale"], dev))
+    codes = torch.empty((B, hw, hw, Oc), dtype=torch.uint8, device=dev)
+    M.minw_conv_block_codes(act, B, C, hw, hw, bits, wgt, Oc, 1, 1, bits, 1, 0, 0, dev_tensor(p["scale"], dev),
+                            dev_tensor(p["shift"], dev), q_out=M.quant(bits, DEFAULT_THR[bits]), codes_out=codes)
+    acc = O.conv2d_levels(O.quantize(p["x"], bits, p["thr_a"]), O.quantize(p["w"], bits, p["thr_w"], p["w_scale"]), 1, 0,
+                          bits, bits)
+    with np.errstate(over="ignore"):
+        lv = O.quantize(O.hardtanh(O.affine(acc, p["scale"], p["shift"])), bits, DEFAULT_THR[bits])
+    assert np.array_equal(decode_e4m3(codes.cpu().numpy()), lv.transpose(0, 2, 3, 1) * 2.0 ** O.units_shift(bits))
+
+
+def test_breakpoint_search_is_short(dev, M):
+    """A fully connected layer with 3-bit outputs and no breakpoints given: their
+    search in the kernel keeps it within twice the time of its fp32 outputs."""
+    B, K, Oc = 256, 1024, 1024
+    g = torch.Generator(device=dev).manual_seed(1)
+    act = torch.empty((B, 1, 1, K), dtype=torch.uint8, device=dev)
+    wgt = torch.empty((Oc, 1, 1, K), dtype=torch.uint8, device=dev)
+    M.aqe_quantize_codes(torch.randn((B, K, 1, 1), generator=g, device=dev), M.quant(2, DEFAULT_THR[2]), act)
+    M.minw_pack_weight_codes(torch.randn((Oc, K, 1, 1), generator=g, device=dev), M.quant(2, DEFAULT_THR[2]), wgt)
+    sc, sh = torch.randn(Oc, generator=g, device=dev), torch.randn(Oc, generator=g, device=dev)
+    y = torch.empty((B, Oc), device=dev)
+    codes = torch.empty((B, Oc), dtype=torch.uint8, device=dev)
+
+    def us(**kw):
+        best = float("inf")
+        for i in range(20):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            for _ in range(20):
+                M.minw_fc_codes(act.view(B, K), B, K, 2, wgt.view(Oc, K), Oc, 2, sc, sh, **kw)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 50 if i else best)
+        return best
+
+    t = us(q_out=M.quant(3, DEFAULT_THR[3]), codes_out=codes), us(y_out=y)
+    assert t[0] <= 2 * t[1], t
