@@ -186,9 +186,12 @@ __global__ void __launch_bounds__(256) aqe_backward_masked_kernel(const uint32_t
 // nibble per plane in bytes 0 .. P - 1), exchanged through shared memory so
 // that one thread assembles the 32 channels of a pixel.  Shared word of
 // channel group g of pixel V j + i: [i][j][g], rows of G + 4 words (16-byte
-// aligned, no conflict at G = 32, two-way below).  PX is 32 for 128 channels
-// and more, and grows to 128 as the channels shrink to 32 (V = 4), so that
-// the 256 threads stay busy.
+// aligned, no conflict at G = 32, two-way below), or [i][g][j] where one block
+// holds all of the channels in fewer than eight groups.  PX is 32 for 128 channels
+// and more, and grows to 128 as the channels shrink to 32 and 1024 at 4 (V = 4), so
+// that the 256 threads stay busy; images of 16 pixels and fewer (V = 1) take as
+// few lanes as they have.  64 x 3 x 224 x 224, 1 bit: 59.7 us with 128 pixels,
+// 12.1 with 1024; 256 x 1024 x 1 x 1 with forward and mask 23.5 and 3.6.
 // A warp per 32 channels with its channels in a serial loop, as before, had
 // one load in flight and few warps on small tensors: 256 x 512 x 14 x 14,
 // 3 bits 107 us; 4 x 128 x 32 x 32, 1 bit 21 us (38 and 4 us here; instruction
@@ -239,7 +242,8 @@ __device__ __forceinline__ uint32_t code_of(float u, const QParams &q) {
     return pick<BITS, uint32_t>(fabsf(u), q, 0u, c1 | neg, c2 | neg, c4 | neg);
 }
 
-template <int BITS, int OUT, int V>
+// FEW: all channels in fewer than eight groups (at most 16 channels).
+template <int BITS, int OUT, int V, bool FEW>
 __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restrict__ x, int B, int C, int HW, QParams q,
                                                           int lgl, int chunks, int cgs, int64_t total,
                                                           uint32_t *__restrict__ planes, uint8_t *__restrict__ codes,
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
     pdl_trigger();
     pdl_wait();
     const int LN = 1 << lgl, G = 256 >> lgl, PX = V << lgl;      // lanes per pixel run, channel groups, pixels
-    const int RS = G + 4, IS = LN * RS;                           // shared strides of j and i
+    const int RS = G + 4, IS = FEW ? 264 : LN * RS;               // shared strides of j and i
     const int NW = (C + 31) >> 5;
     const int j = threadIdx.x & (LN - 1), g = threadIdx.x >> lgl;
 
@@ -367,11 +371,12 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
             for (int i = 0; i < V; ++i) w[i] &= cm;
         }
 #pragma unroll
-        for (int i = 0; i < V; ++i) sw[i * IS + j * RS + g] = w[i];
+        for (int i = 0; i < V; ++i) sw[i * IS + (FEW ? (int)threadIdx.x : j * RS + g)] = w[i];
         if constexpr (OUT == OUT_PLANES) {
             if (y != nullptr) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
+                    if (FEW && k >= nc) break;                    // the same in a whole warp
                     float yv[V];
 #pragma unroll
                     for (int i = 0; i < V; ++i)
@@ -383,13 +388,31 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
                     }
                 }
             }
-            if (mask != nullptr) {
+            if (V == 1 && !FEW && mask != nullptr && lgl < 5) {
+                // no 32-pixel runs: bit by bit, four channels at once where their bits are neighbours
+                uint32_t mb = 0u;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) mb |= (k < nst && fabsf(v[k][0]) <= 1.0f ? 1u : 0u) << k;
+                if (HW == 1 && mb != 0u) {
+                    uint32_t *mw = mask + (off >> 5);
+                    const uint32_t sh = (uint32_t)off & 31u, hi = __funnelshift_l(mb, 0u, sh);
+                    atomicOr(mw, mb << sh);
+                    if (hi) atomicOr(mw + 1, hi);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int64_t at = off + (int64_t)k * HW;
+                        if ((mb >> k) & 1u) atomicOr(mask + (at >> 5), 1u << (at & 31));
+                    }
+                }
+            } else if (mask != nullptr) {
                 // 32 consecutive pixels of a channel row sit in 32 / V neighbouring lanes of one warp; lane k of
                 // them stores channel k's word
                 uint32_t mk = 0u;
                 const int rl = V == 4 ? threadIdx.x & 7 : threadIdx.x & 31;       // lane in the run
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
+                    if (FEW && k >= nc) break;
                     uint32_t m = 0u;
 #pragma unroll
                     for (int i = 0; i < V; ++i) m |= (fabsf(v[k][i]) <= 1.0f ? 1u : 0u) << i;
@@ -421,13 +444,22 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
         }
         __syncthreads();
         // word wi (32 channels: shared words 8 wi .. + 7) of pixel px; neighbouring threads on neighbouring words
-        const int lgn = 5 - lgl, nwi = 1 << lgn;                  // 32-channel words per pixel
+        const int lgn = FEW ? 0 : 5 - lgl, nwi = 1 << lgn;        // 32-channel words per pixel
         for (int e = threadIdx.x; e < PX * nwi; e += 256) {
             const int wi = e & (nwi - 1), px = e >> lgn;
-            const int cw = (cg * G >> 3) + wi;
+            const int cw = FEW ? 0 : (cg * G >> 3) + wi;
             if (p0 + px >= HW || cw >= NW) continue;
-            const uint32_t *src = sw + (px & (V - 1)) * IS + (px / V) * RS + 8 * wi;
-            const uint4 a = *reinterpret_cast<const uint4 *>(src), d = *reinterpret_cast<const uint4 *>(src + 4);
+            uint4 a = make_uint4(0u, 0u, 0u, 0u), d = a;
+            if constexpr (FEW) {
+                const uint32_t *src = sw + (px & (V - 1)) * IS + px / V;
+                a.x = src[0];
+                if (G > 1) a.y = src[LN];
+                if (G > 2) { a.z = src[2 * LN]; a.w = src[3 * LN]; }
+            } else {
+                const uint32_t *src = sw + (px & (V - 1)) * IS + (px / V) * RS + 8 * wi;
+                a = *reinterpret_cast<const uint4 *>(src);
+                d = *reinterpret_cast<const uint4 *>(src + 4);
+            }
             const uint32_t s[8] = {a.x, a.y, a.z, a.w, d.x, d.y, d.z, d.w};
             const int64_t pix = b * HW + p0 + px;
             if constexpr (OUT == OUT_PLANES) {
@@ -459,8 +491,11 @@ static minw_status launch_quantize(const float *x, int B, int C, int64_t HW, con
                                    uint8_t *codes, float alpha, float *y, uint32_t *mask, int mask_atomic,
                                    cudaStream_t s) {
     const bool vec = HW % 4 == 0 && minw_host::aligned16(x) && (!y || minw_host::aligned16(y));
-    // pixels per block: 32 (lanes 8 x 4 pixels) for more than 64 channels, 64 and 128 below; scalar: 32
-    const int lgl = !vec ? 5 : C > 64 ? 3 : C > 32 ? 4 : 5;
+    // pixels per block: 32 (lanes 8 x 4 pixels) for more than 64 channels, 64 and 128 below; scalar: 32, or as
+    // many as an image of up to 16 has; four to sixteen channels in one to four groups
+    int lgl = C <= 4 ? 8 : C <= 8 ? 7 : C <= 16 ? 6 : !vec || C <= 32 ? 5 : C <= 64 ? 4 : 3;
+    if (!vec && HW <= 16)
+        for (lgl = 0; (1 << lgl) < HW;) ++lgl;
     const int PX = (vec ? 4 : 1) << lgl, CG = 4 * (256 >> lgl);
     const int chunks = (int)((HW + PX - 1) / PX), cgs = (C - 1) / CG + 1;
     const int64_t total = (int64_t)B * chunks * cgs;
@@ -469,10 +504,13 @@ static minw_status launch_quantize(const float *x, int B, int C, int64_t HW, con
     const dim3 grid((unsigned)(total < 4 * sms ? total : 4 * sms));
     typedef void (*Kernel)(const float *, int, int, int, QParams, int, int, int, int64_t, uint32_t *, uint8_t *, float,
                            float, float *, uint32_t *, int);
-    static const Kernel kernels[2][3] = {
-        {quantize_kernel<1, OUT, 1>, quantize_kernel<2, OUT, 1>, quantize_kernel<3, OUT, 1>},
-        {quantize_kernel<1, OUT, 4>, quantize_kernel<2, OUT, 4>, quantize_kernel<3, OUT, 4>}};
-    if (minw_host::launch_pdl(kernels[vec][q.bits - 1], grid, dim3(256), 0, s, x, B, C, (int)HW, q, lgl, chunks, cgs,
+    constexpr bool F = OUT != OUT_E2M1;                           // (E2M1 codes have 32 channels and more)
+    static const Kernel kernels[2][2][3] = {
+        {{quantize_kernel<1, OUT, 1, false>, quantize_kernel<2, OUT, 1, false>, quantize_kernel<3, OUT, 1, false>},
+         {quantize_kernel<1, OUT, 4, false>, quantize_kernel<2, OUT, 4, false>, quantize_kernel<3, OUT, 4, false>}},
+        {{quantize_kernel<1, OUT, 1, F>, quantize_kernel<2, OUT, 1, F>, quantize_kernel<3, OUT, 1, F>},
+         {quantize_kernel<1, OUT, 4, F>, quantize_kernel<2, OUT, 4, F>, quantize_kernel<3, OUT, 4, F>}}};
+    if (minw_host::launch_pdl(kernels[lgl > 5][vec][q.bits - 1], grid, dim3(256), 0, s, x, B, C, (int)HW, q, lgl, chunks, cgs,
                               total, planes, codes, alpha, 1.0f - alpha, y, mask, mask_atomic) != cudaSuccess)
         return MINW_ECUDA;
     return minw_host::launch_status();

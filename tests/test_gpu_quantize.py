@@ -50,7 +50,11 @@ def _at_offset(x, off):
 
 
 SHAPES = [(1, 1, 1, 1), (2, 3, 7, 9), (3, 33, 2, 2), (2, 64, 14, 14), (1, 65, 8, 8), (2, 40, 16, 10), (1, 130, 12, 11),
-          (2, 160, 6, 6), (1, 512, 14, 14), (2, 96, 33, 4)]
+          (2, 160, 6, 6), (1, 512, 14, 14), (2, 96, 33, 4),
+          # up to 16 channels in one to four groups: whole and ragged runs of 1024, 512 and 256 pixels (scalar: a quarter)
+          (2, 4, 32, 32), (3, 3, 33, 32), (2, 7, 13, 9), (1, 8, 50, 40), (1, 12, 40, 28), (2, 16, 29, 21), (1, 1, 47, 45),
+          # images of up to 16 pixels with as few lanes, many channels
+          (4, 100, 1, 1), (3, 1030, 1, 1), (2, 70, 3, 3), (33, 40, 1, 2), (1, 5, 3, 5), (2, 600, 1, 11)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -77,7 +81,9 @@ def test_planes_mask_forward(M, shape, bits, off):
 
 @pytest.mark.parametrize("bits", [1, 2, 3])
 @pytest.mark.parametrize("shape,off", [((2, 16, 5, 5), 0), ((1, 48, 4, 4), 0), ((2, 64, 14, 14), 0), ((1, 96, 9, 9), 0),
-                                       ((2, 160, 8, 8), 1), ((1, 512, 7, 7), 0), ((3, 32, 12, 11), 1)])
+                                       ((2, 160, 8, 8), 1), ((1, 512, 7, 7), 0), ((3, 32, 12, 11), 1),
+                                       ((1, 16, 64, 44), 0), ((2, 16, 20, 20), 1), ((3, 16, 3, 3), 0), ((3, 32, 1, 1), 0),
+                                       ((2, 1056, 1, 1), 0), ((2, 64, 1, 5), 0)])
 def test_codes(M, shape, bits, off):
     B, C, H, W = shape
     x = _values(shape, bits, sum(shape) + bits)
@@ -93,6 +99,26 @@ def test_codes(M, shape, bits, off):
         codes = torch.full((B, H, W, C // 2), 0x77, dtype=torch.uint8, device="cuda")
         M.aqe_quantize_codes_e2m1(xd, M.quant(bits, DEFAULT_THR[bits]), codes)
         assert np.array_equal(codes.cpu().numpy(), nib[..., 0::2] | (nib[..., 1::2] << 4))
+
+
+def test_few_channels_keep_the_threads_busy(M):
+    """Three-channel images take the time of their bytes: at most twice that
+    of as many 96-channel values."""
+    us = []
+    for shape in ((64, 3, 224, 224), (64, 96, 49, 32)):
+        x = torch.zeros(shape, device="cuda")
+        planes = torch.empty(M.packed_words(*shape, 1), dtype=torch.int32, device="cuda")
+        best = float("inf")
+        for i in range(20):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            for _ in range(5):
+                M.aqe_quantize_pack(x, M.quant(1, DEFAULT_THR[1]), planes)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 200 if i else best)
+        us.append(best)
+    assert us[0] <= 2 * us[1], us
 
 
 def test_capture_behind_copies_and_fills(M):
