@@ -791,11 +791,20 @@ static bool first_tc_plan(const FirstArgs &a, ftc::Params &p) {
     // shared memory: weight pieces, A ring, patch ring, fp32 weights, channel table, taps, maxabs,
     // recompute lists, barriers (three patches and three A blocks in flight where they fit)
     const size_t limit = 227 * 1024 - 1024;
+    // Lists of open decisions (rather than a patch slot more, or recomputing them in place) where two recompute warps
+    // keep up with them: a decision is open with a chance of about K, and its chain is K long, longer still where the
+    // taps are not unrolled (shapes 0).  In us, lists : none, 64 images, 3 bits: 8 -> 128 channels 3x3 on 96 x 96 (O 6
+    // K^2 = 4.0e6) 225 : 287, 8 -> 192 on 64 x 64 (6.0e6) 217 : 191, 16 -> 64 on 64 x 64 (8.0e6) 154 : 123; the stem,
+    // unrolled, 64 channels on 224 x 224 (8.3e6) 236 : 251.  With one patch slot the recompute would hold the next
+    // patch up: 16 -> 128 on 32 x 32 160 : 93.
+    const bool unrolled = a.C == 3 && ((a.kh == 3 && a.kw == 3 && a.stride == 1) || (a.kh == 7 && a.kw == 7 && a.stride == 2));
+    const bool lists = (long long)a.O * (nl - 1) * p.K * p.K <= (unrolled ? 10000000 : 5000000);
     static const int np_[6] = {4, 3, 3, 2, 2, 1}, sa_[6] = {4, 4, 3, 3, 2, 2};
     for (int cfg = 0; cfg < 12; ++cfg) {
         p.NP = np_[cfg % 6];
         p.SA = sa_[cfg % 6];
-        p.cap = cfg < 6 ? ftc::CAP : 0;         // lists of open decisions where they fit, else recomputed in place
+        p.cap = cfg < 6 ? ftc::CAP : 0;
+        if (p.cap != 0 && (!lists || p.NP < 2)) continue;
         size_t off = (size_t)p.nkb * p.b_block;
         p.off_a = (uint32_t)off;
         off += (size_t)p.SA * 16384u;
