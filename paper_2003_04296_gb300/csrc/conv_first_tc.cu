@@ -679,14 +679,15 @@ __global__ void __launch_bounds__(NT, 1)
         // ---------------- recompute warps: the open decisions of a tile, 32 at a time ----------------
         // About 0.3 % of the stem's decisions are open, a few per 32-channel chunk: chunk by chunk their
         // 147-tap chains kept a warp busy for three lanes' work.
-        // The warps take the tiles in turn, as many of them as there are patch slots: a barrier's parity tells tile n
+        // The warps take the tiles in turn, one of them all where there is one patch slot: a barrier's parity tells tile n
         // from tile n - NP of the same slot only to a warp that has seen the latter done, which holds where its own
         // last tile is n - NP or a later one.
-        const int NWo = (O + 31) >> 5, nrec = min(NREC, p.NP);
+        const int NWo = (O + 31) >> 5;
+        const bool one = p.NP < NREC;
         int n = 0;
         bool dead = false;
         for (int t = blockIdx.x; t < p.tiles && !dead; t += gridDim.x, ++n) {
-            if (n % nrec != warp - REC0) continue;
+            if (one ? warp != REC0 : n % NREC != warp - REC0) continue;
             const int pslot = n % p.NP;
             if (!__all_sync(0xffffffffu, bar_wait(&efull[pslot], (uint32_t)(n / p.NP) & 1u, p.wait_cycles))) { dead = true; break; }
             const int b = t / p.tiles_img, p0 = (t - b * p.tiles_img) * 128, oyf = p0 / p.Wo;
