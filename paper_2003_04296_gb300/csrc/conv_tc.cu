@@ -1175,12 +1175,15 @@ __global__ void __launch_bounds__(NT, 1)
             }
         }
         if (!p.planned) pdl_wait();
-        // channel tiles of this CTA's first and last item
-        const int w0 = cta_item(p, 0, items, tiles_m, crank);
-        const int w1 = p.wres || w0 < 0 ? w0 : w0 + (items - 1 - w0) / (int)gridDim.x * (int)gridDim.x;
+        int olo = 0, ohi = p.O;
+        if (OUTB > 0 && p.thr == nullptr && !resid) {         // channel tiles of this CTA's first and last item
+            const int w0 = max(0, cta_item(p, 0, items, tiles_m, crank));
+            const int w1 = p.wres ? w0 : w0 + (items - 1 - w0) / (int)gridDim.x * (int)gridDim.x;
+            olo = w0 / p.ksplit / tiles_m * p.BN;
+            ohi = (w1 / p.ksplit / tiles_m + 1) * p.BN;
+        }
         epi_tables<OUTB>(p, resid, sthr, ssig, syt, reinterpret_cast<float *>(tmem_slot + 1), O32, thr_floats, sig_words, et,
-                         warp, lane, w0 < 0 ? 0 : w0 / p.ksplit / tiles_m * p.BN,
-                         w0 < 0 ? 0 : (w1 / p.ksplit / tiles_m + 1) * p.BN);
+                         warp, lane, olo, ohi);
         asm volatile("bar.sync 1, %0;\n" ::"n"(EPI_WARPS * 32) : "memory");   // breakpoints in place
         pdl_wait();                               // outputs, shortcuts and partial sums are shared with other kernels
         const int q = warp & 3;                   // TMEM lane quarter of this warp
