@@ -421,8 +421,10 @@ MINW_API size_t minw_conv_train_workspace_bytes(int32_t B, int32_t C, int32_t H,
  * pad < kw (else MINW_EUNSUPPORTED); alpha in [0, 1]; 16-byte aligned
  * pointers; workspace of minw_conv_train_workspace_bytes (scratch: nothing
  * in it survives the call).  All buffers are caller-owned device memory; the
- * call is asynchronous on stream and launches eight to eleven kernels (and a
- * memset of the input gradient's spread image for stride 2 or O % 64 != 0).
+ * call is asynchronous on stream and launches seven kernels, one more for each
+ * of the forward and the input-gradient product that splits along K, one
+ * fewer without g_in (and a memset of the input gradient's spread image for
+ * stride 2 or O % 64 != 0).
  * MINW_EINVAL: null A, W, g_out, a_out, q_w or workspace, an invalid
  * quantizer, alpha outside [0, 1], a misaligned pointer or a short workspace;
  * MINW_EUNSUPPORTED: the shapes above, or sizes past the kernels' index and
@@ -601,7 +603,11 @@ MINW_API minw_status minw_forward_host(minw_net *net, const float *x_host, int32
 /* Per-layer timing: with on != 0 every later minw_forward records a CUDA
  * event after each layer's kernel; minw_net_layer_times then writes the
  * elapsed milliseconds of each layer of the most recent forward into ms
- * (host array of minw_net_launches() floats), synchronising on the events. */
+ * (host array of minw_net_launches() floats), synchronising on the events.
+ * A weight-only network whose forward is one kernel (minw_net_kernels() is 1
+ * without timing) runs layer by layer while timing is on: another forward,
+ * several times slower than the one-kernel one, with logits that may differ
+ * within the products' fp32 sums. */
 MINW_API minw_status minw_net_enable_timing(minw_net *net, int32_t on);
 MINW_API minw_status minw_net_layer_times(minw_net *net, float *ms);
 
@@ -675,10 +681,11 @@ MINW_API minw_status minw_resnet18_create(const minw_resnet18_desc *desc, int32_
  * c2_*[b] [O][O][3][3]; down_*[i] is the shortcut entering stage i + 2
  * [O][C][1][1]; *_wscale: per-output-channel weight prescale (nullable);
  * every block weight is quantized with (bits_w, thr_w) to levels in integer
- * units.  The 16- and 32-channel layers run on operands padded to 64
- * channels.  image_hw: a multiple of 4 (32 for CIFAR).  Device pointers, read
- * during creation only.  minw_forward takes x [B][3][hw][hw] and writes
- * logits [B][num_classes].  Errors: MINW_EINVAL (arguments, n outside
+ * units.  Images of 8 to 32 pixels a side run the whole forward as one kernel;
+ * larger or smaller ones, and forwards with per-layer timing, run layer by layer,
+ * their 16- and 32-channel layers on operands padded to 64 channels.  image_hw: a
+ * multiple of 4 (32 for CIFAR).  Device pointers, read during creation only.
+ * minw_forward takes x [B][3][hw][hw] and writes logits [B][num_classes].  Errors: MINW_EINVAL (arguments, n outside
  * 1 .. MINW_WRESNET_MAX_N), MINW_EUNSUPPORTED (sizes past the 32-bit index
  * range), MINW_ECUDA. */
 #define MINW_WRESNET_MAX_N 18
@@ -735,8 +742,11 @@ MINW_API minw_status minw_wresnet_activation(const minw_net *net, int32_t index,
  * thr_w) to levels in integer units.  Each block's features live in one bf16
  * NHWC buffer of pad64(final c) channels per pixel that the layers append
  * to in place (no concatenation copies); each 1x1 convolution reads the
- * first pad64(c) channels of its rows (zero weights past c).  image_hw: a
- * multiple of 4, at least 8.  Device pointers, read during creation only.
+ * first pad64(c) channels of its rows (zero weights past c).  Growth 4, 8 or 12 on
+ * images of up to 32 pixels a side, where the weights fit its buffers, runs the
+ * whole forward as one kernel on features of its own layout instead (not with
+ * per-layer timing).  image_hw: a multiple of 4, at least 8.  Device pointers,
+ * read during creation only.
  * minw_forward takes x [B][3][hw][hw] and writes logits [B][num_classes].
  * Errors: MINW_EINVAL (arguments; layers outside 1 .. MINW_WDENSE_MAX_LAYERS,
  * growth outside 1 .. 64), MINW_EUNSUPPORTED (sizes past the 32-bit index
@@ -850,9 +860,10 @@ MINW_API minw_status minw_get_plan_options(minw_plan_options *out);
 MINW_API minw_status minw_set_plan_options(const minw_plan_options *opt);
 
 /* Test hook of the timeout path (no counterpart in the paper): the next launch
- * of the named kernel -- MINW_STALL_CONV_TC, the single-CTA tensor-core
- * convolution, or MINW_STALL_CONV_FIRST, the first layer with TMA patches --
- * first waits on a barrier that nothing completes.  That wait runs out after
+ * of the named kernel -- MINW_STALL_CONV_TC, a tensor-core convolution on level
+ * codes (a single CTA's or on halo tiles) or bit-planes, or
+ * MINW_STALL_CONV_FIRST, the first layer with TMA patches or on the tensor
+ * cores -- first waits on a barrier that nothing completes.  That wait runs out after
  * wait_cycles, the kernel skips its work, drains its own loads and frees its
  * tensor memory, and minw_get_last_device_error reports MINW_ETIMEOUT once.
  * One launch only; 0 cancels a pending request.  No GPU fault is involved. */

@@ -27,7 +27,7 @@
 // arrivals on fready, after which its output may be copied.
 //
 // Measured: DenseNet-100, 3-bit weights, batch 128: 1475 us layer by layer,
-// 435 us here.  Block 1 holds most of it: each layer streams its inputs, 256 KB
+// 426 us here.  Block 1 holds most of it: each layer streams its inputs, 256 KB
 // per image on average, and 128 CTAs together draw about 5 TB/s from L2.
 //
 // Same operations as the layer-by-layer path: fp32 stem chain, bf16 features,

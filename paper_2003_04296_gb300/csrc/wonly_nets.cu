@@ -605,7 +605,7 @@ void wdense_variants(const minw_net *net, int32_t *v) {
     v[k++] = 0;
 }
 
-// The sizes wdense_fused.cu covers take its one-kernel forward: 1.473 -> 0.435
+// The sizes wdense_fused.cu covers take its one-kernel forward: 1.475 -> 0.426
 // ms for DenseNet-100 at batch 128.  Other sizes and forwards with per-op
 // timing run layer by layer.
 static bool wdense_fused(const minw_net *net) { return net->wdense->blob != nullptr && !net->timing; }
