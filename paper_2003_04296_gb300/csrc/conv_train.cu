@@ -261,8 +261,8 @@ minw_status minw_conv_train_step(const float *A, float *Wt, const float *g_out, 
 #define TRY(x) do { if ((st = (x)) != MINW_OK) return st; } while (0)
     // W^ (Eq. weight) in both layouts; the input as bf16 NHWC
     // (these passes start while the kernel before drains, and let no dependent start early)
-    if (launch_pdl(train_weights_kernel, dim3(grid_for((int64_t)O * kh * kw * C)), dim3(256), 0, s, (const float *)Wt, O, C,
-                   kh, kw, sh.Op, alpha, qw, wf, wd, ones, zeros, M) != cudaSuccess)
+    if (launch_pdl_stream(false, train_weights_kernel, dim3(grid_for((int64_t)O * kh * kw * C)), dim3(256), 0, s,
+                          (const float *)Wt, O, C, kh, kw, sh.Op, alpha, qw, wf, wd, ones, zeros, M) != cudaSuccess)
         return MINW_ECUDA;
     TRY(launch_status());
     TRY(minw_to_bf16_nhwc(A, B, C, H, W, ab, stream));
@@ -275,8 +275,9 @@ minw_status minw_conv_train_step(const float *A, float *Wt, const float *g_out, 
         if (cudaMemsetAsync(gd, 0, (size_t)B * sh.Hd * sh.Wd * sh.Op * 2, s) != cudaSuccess) return MINW_ECUDA;
     {
         const dim3 grid((unsigned)((sh.Ho * sh.Wo + 31) / 32), (unsigned)(sh.Op / 64), (unsigned)B);
-        if (launch_pdl(train_grad_kernel, grid, dim3(256), 0, s, (const float *)(q_a ? at : g_out), g_out, O, sh.Ho * sh.Wo,
-                       sh.Wo, stride, sh.Hd, sh.Wd, sh.Op, alpha, q_a ? 1 : 0, qa, a_out, gd) != cudaSuccess)
+        if (launch_pdl_stream(false, train_grad_kernel, grid, dim3(256), 0, s, (const float *)(q_a ? at : g_out), g_out, O,
+                              sh.Ho * sh.Wo, sh.Wo, stride, sh.Hd, sh.Wd, sh.Op, alpha, q_a ? 1 : 0, qa, a_out,
+                              gd) != cudaSuccess)
             return MINW_ECUDA;
         TRY(launch_status());
     }

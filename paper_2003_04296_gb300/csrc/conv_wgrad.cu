@@ -363,8 +363,9 @@ minw_status launch_conv_wgrad(const WgradArgs &a, float *part, float lr, float t
     const int R = p.C * p.ntaps, ob = (p.O + 31) / 32;
     const bool narrow = (long long)((R + 31) / 32) * ob < 2 * (minw_host::num_sms() > 0 ? minw_host::num_sms() : 152);
     const dim3 ugrid((unsigned)(narrow ? (R + 7) / 8 : (R + 31) / 32), (unsigned)std::min(ob, 65535));
-    if (minw_host::launch_pdl(narrow ? wg::wgrad_update_kernel<1> : wg::wgrad_update_kernel<4>, ugrid, dim3(256), 0, s,
-                              (const float *)part, p.slices, p.ntaps, p.C, p.O, lr, two_alpha, W) != cudaSuccess)
+    if (minw_host::launch_pdl_stream(false, narrow ? wg::wgrad_update_kernel<1> : wg::wgrad_update_kernel<4>, ugrid,
+                                     dim3(256), 0, s, (const float *)part, p.slices, p.ntaps, p.C, p.O, lr, two_alpha,
+                                     W) != cudaSuccess)
         return MINW_ECUDA;
     return minw_host::launch_status();
 }

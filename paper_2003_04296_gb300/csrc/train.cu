@@ -275,10 +275,10 @@ minw_status minw_fc_train_step(const float *A, float *W, const float *g_out, int
     // 1.1 forward: W^ = alpha h(W) + (1 - alpha) W as bf16 [O][K] and [K][Op]; a as bf16 [B][K] and [K][B]
     const float *none = nullptr;
     float *fnone = nullptr;
-    if (launch_pdl(prep_kernel<0>, dim3((unsigned)(K / 64), (unsigned)(Op / 32)), dim3(256), 0, s, (const float *)W, none, O,
-                   K, K, Op, alpha, qw, wb, wtb, fnone, ones, zeros, M) != cudaSuccess ||
-        launch_pdl(prep_kernel<1>, dim3((unsigned)(K / 64), (unsigned)(B / 32)), dim3(256), 0, s, A, none, B, K, K, B, 0.0f,
-                   qw, ab, atb, fnone, fnone, fnone, 0) != cudaSuccess)
+    if (launch_pdl_stream(false, prep_kernel<0>, dim3((unsigned)(K / 64), (unsigned)(Op / 32)), dim3(256), 0, s,
+                          (const float *)W, none, O, K, K, Op, alpha, qw, wb, wtb, fnone, ones, zeros, M) != cudaSuccess ||
+        launch_pdl_stream(false, prep_kernel<1>, dim3((unsigned)(K / 64), (unsigned)(B / 32)), dim3(256), 0, s, A, none, B,
+                          K, K, B, 0.0f, qw, ab, atb, fnone, fnone, fnone, 0) != cudaSuccess)
         return MINW_ECUDA;
     TRY(launch_status());
     // a~ = a W^T  ([B][O], reduction over K); the last layer emits a~ itself
@@ -287,7 +287,7 @@ minw_status minw_fc_train_step(const float *A, float *W, const float *g_out, int
                     nullptr, s));
     // 1.2 backward through the activation AQE (Eq. activation): g_a~ = 2 alpha g 1[|a~| <= 1], as bf16
     // [B][Op] and [O][B]; a_l = alpha h(a~) + (1 - alpha) a~
-    if (launch_pdl(prep_kernel<2>, dim3((unsigned)(Op / 64), (unsigned)(B / 32)), dim3(256), 0, s,
+    if (launch_pdl_stream(false, prep_kernel<2>, dim3((unsigned)(Op / 64), (unsigned)(B / 32)), dim3(256), 0, s,
                    (const float *)(q_a ? at : g_out), g_out, B, O, Op, B, alpha, qa, gb, gtb, q_a ? a_out : fnone, fnone,
                    fnone, 0) != cudaSuccess)
         return MINW_ECUDA;

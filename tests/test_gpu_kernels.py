@@ -239,3 +239,27 @@ def test_conv2d_adversarial_magnitudes(dev, M):
     for variant in (M.VARIANT_POPC,):
         _, _, acc, _ = _conv_gpu(dev, M, p, variant)
         assert np.array_equal(acc.cpu().numpy(), _conv_ref(p))
+
+
+def test_streaming_passes_keep_their_loads_in_flight():
+    """The AQE backward on 25.7 M values against an addition of the same
+    bytes: the pass streams at the memory's rate."""
+    import __graft_entry__ as g
+    g.build()
+    from paper_2003_04296_gb300 import minw as M
+    n = 256 * 512 * 14 * 14
+    x, gy = torch.randn(n, device="cuda"), torch.randn(n, device="cuda")
+    out = torch.empty_like(x)
+    us = []
+    for call in (lambda: M.aqe_backward(x, gy, out, 0.75), lambda: torch.add(x, gy, out=out)):
+        best = float("inf")
+        for i in range(20):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            for _ in range(5):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 200 if i else best)
+        us.append(best)
+    assert us[0] <= 1.25 * us[1], us
