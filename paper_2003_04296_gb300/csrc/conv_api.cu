@@ -53,7 +53,8 @@ int choose_variant(const ConvArgs &a, int requested) {
 // 9.6 : 16.6; 32 -> 64, 1 x 1 14.9 : 19.1; 32 -> 32, 3 x 1 14.6 : 17.8; 64 -> 32,
 // 1 x 1 14.2 : 17.2; 96 -> 8, 2 x 1 15.5 : 16.6; past the limits 32 -> 32, 1 x 3
 // 19.5 : 17.4; 32 -> 96, 1 x 1 24.6 : 21.5; 96 -> 8, 1 x 1 20.0 : 16.9.  Below two
-// tiles per SM nothing is gained.
+// tiles per SM nothing is gained (one tile, a 7 x 7 image of 32 -> 32 channels, 1 x 1
+// bit, raw 3.4 : 2.8, with planes out 8.7 : 3.5).
 static bool popcount_shorter(const ConvArgs &a) {
     const int work[3][3] = {{11, 16, 0}, {9, 15, 0}, {20, 0, 0}};       // [activation bits - 1][weight bits - 1]
     const int w = work[a.bits_a - 1][a.bits_w - 1] * a.NW;
