@@ -605,9 +605,8 @@ MINW_API minw_status minw_forward_host(minw_net *net, const float *x_host, int32
  * elapsed milliseconds of each layer of the most recent forward into ms
  * (host array of minw_net_launches() floats), synchronising on the events.
  * A weight-only network whose forward is one kernel (minw_net_kernels() is 1
- * without timing) runs layer by layer while timing is on: another forward,
- * several times slower than the one-kernel one, with logits that may differ
- * within the products' fp32 sums. */
+ * without timing) runs layer by layer while timing is on: another forward of
+ * the same operations, several times slower than the one-kernel one. */
 MINW_API minw_status minw_net_enable_timing(minw_net *net, int32_t on);
 MINW_API minw_status minw_net_layer_times(minw_net *net, float *ms);
 
