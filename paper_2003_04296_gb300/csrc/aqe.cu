@@ -242,13 +242,17 @@ __device__ __forceinline__ uint32_t code_of(float u, const QParams &q) {
     return pick<BITS, uint32_t>(fabsf(u), q, 0u, c1 | neg, c2 | neg, c4 | neg);
 }
 
-// FEW: all channels in fewer than eight groups (at most 16 channels).
-template <int BITS, int OUT, int V, bool FEW>
+// SPLIT: SPLIT_WIDE as above, SPLIT_FEW all channels in fewer than eight groups (at most 16 channels), SPLIT_TINY
+// fewer than 32 lanes per pixel run (V = 1, images of at most 16 pixels; a kernel of its own as its bitwise mask
+// cost the others' scalar loads 10 %).
+enum QuantSplit { SPLIT_WIDE, SPLIT_FEW, SPLIT_TINY };
+template <int BITS, int OUT, int V, int SPLIT>
 __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restrict__ x, int B, int C, int HW, QParams q,
                                                           int lgl, int chunks, int cgs, int64_t total,
                                                           uint32_t *__restrict__ planes, uint8_t *__restrict__ codes,
                                                           float alpha, float oma, float *__restrict__ y,
                                                           uint32_t *__restrict__ mask, int mask_atomic) {
+    constexpr bool FEW = SPLIT == SPLIT_FEW;
     __shared__ __align__(16) uint32_t sw[V * (256 + 4 * 32)];
     pdl_trigger();
     pdl_wait();
@@ -388,7 +392,7 @@ __global__ void __launch_bounds__(256, 4) quantize_kernel(const float *__restric
                     }
                 }
             }
-            if (V == 1 && !FEW && mask != nullptr && lgl < 5) {
+            if (SPLIT == SPLIT_TINY && mask != nullptr) {
                 // no 32-pixel runs: bit by bit, four channels at once where their bits are neighbours
                 uint32_t mb = 0u;
 #pragma unroll
@@ -504,17 +508,21 @@ static minw_status launch_quantize(const float *x, int B, int C, int64_t HW, con
     const dim3 grid((unsigned)(total < 4 * sms ? total : 4 * sms));
     typedef void (*Kernel)(const float *, int, int, int, QParams, int, int, int, int64_t, uint32_t *, uint8_t *, float,
                            float, float *, uint32_t *, int);
-    constexpr bool F = OUT != OUT_E2M1;                           // (E2M1 codes have 32 channels and more)
-    static const Kernel kernels[2][2][3] = {
-        {{quantize_kernel<1, OUT, 1, false>, quantize_kernel<2, OUT, 1, false>, quantize_kernel<3, OUT, 1, false>},
-         {quantize_kernel<1, OUT, 4, false>, quantize_kernel<2, OUT, 4, false>, quantize_kernel<3, OUT, 4, false>}},
-        {{quantize_kernel<1, OUT, 1, F>, quantize_kernel<2, OUT, 1, F>, quantize_kernel<3, OUT, 1, F>},
-         {quantize_kernel<1, OUT, 4, F>, quantize_kernel<2, OUT, 4, F>, quantize_kernel<3, OUT, 4, F>}}};
+    constexpr int F = OUT != OUT_E2M1 ? SPLIT_FEW : SPLIT_WIDE;   // (E2M1 codes have 32 channels and more)
+    static const Kernel wide[2][3] = {
+        {quantize_kernel<1, OUT, 1, SPLIT_WIDE>, quantize_kernel<2, OUT, 1, SPLIT_WIDE>, quantize_kernel<3, OUT, 1, SPLIT_WIDE>},
+        {quantize_kernel<1, OUT, 4, SPLIT_WIDE>, quantize_kernel<2, OUT, 4, SPLIT_WIDE>, quantize_kernel<3, OUT, 4, SPLIT_WIDE>}};
+    static const Kernel few[2][3] = {
+        {quantize_kernel<1, OUT, 1, F>, quantize_kernel<2, OUT, 1, F>, quantize_kernel<3, OUT, 1, F>},
+        {quantize_kernel<1, OUT, 4, F>, quantize_kernel<2, OUT, 4, F>, quantize_kernel<3, OUT, 4, F>}};
+    static const Kernel tiny[3] = {quantize_kernel<1, OUT, 1, SPLIT_TINY>, quantize_kernel<2, OUT, 1, SPLIT_TINY>,
+                                   quantize_kernel<3, OUT, 1, SPLIT_TINY>};
+    const Kernel kern = lgl > 5 ? few[vec][q.bits - 1] : !vec && lgl < 5 ? tiny[q.bits - 1] : wide[vec][q.bits - 1];
     // the pass of a training layer (forward and mask beside the planes) moves 2.5 times the bytes and reads through
     // L1: 256 x 512 x 14 x 14, 2 bits 58.3 -> 40.9 us; alone, the packing is bound by issue, and a change of the
     // carve-out delays a convolution behind it by 1 to 2 us
     const bool stream = y != nullptr && (int64_t)B * C * HW >= (1 << 22);
-    if (minw_host::launch_pdl_stream(!stream, kernels[lgl > 5][vec][q.bits - 1], grid, dim3(256), 0, s, x, B, C, (int)HW, q,
+    if (minw_host::launch_pdl_stream(!stream, kern, grid, dim3(256), 0, s, x, B, C, (int)HW, q,
                                      lgl, chunks, cgs, total, planes, codes, alpha, 1.0f - alpha, y, mask,
                                      mask_atomic) != cudaSuccess)
         return MINW_ECUDA;
