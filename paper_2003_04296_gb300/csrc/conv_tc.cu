@@ -2211,21 +2211,35 @@ static minw_status make_plan(const ConvArgs &a, Plan &pl, bool encode = true) {
     // fp32 outputs of a fully connected product of bf16 operands: the tile width with the least waves x columns
     // per epilogue warp (weight update 1024 x 8192 on 152 SMs: 296 tiles of 224 columns, two full waves, instead of
     // 256 of 256: 29.4 -> 28.1 us cold; input gradient 256 x 8192: 128 tiles of 128 instead of 64 of 256).  A product
-    // that splits along K keeps its full width: the number of tiles sets the slices and with them the order of the
-    // fp32 sums (128 columns on the 256 x 8192 -> 1024 forward, 9 slices instead of 19: the step 74.2 us instead of
-    // 78.6, and levels of a~ that lie at a threshold flip)
+    // that splits along K keeps the slices of its full width, as they set the order of the fp32 sums (128 columns
+    // on the 256 x 8192 -> 1024 forward, 9 slices instead of 19: the step 74.2 us instead of 78.6, and levels of a~
+    // that lie at a threshold flip); 128 columns where the reduction's length and not the tiles bounds the slices,
+    // their sums take no more room and the CTAs leave a quarter of the SMs idle (a 192 x 2048 -> 450 step, 64 CTAs
+    // instead of 32: 33.1 us instead of 35.6; 128 x 4928 -> 616, 95 instead of 57: 39.6, 41.3; 512 x 2048 -> 512, 128
+    // instead of 64: 37.4, 37.6; 256 x 6336 -> 286, 144 instead of 96: 44.2, 39.9)
     if (a.bf16 && !p.trans && a.Ho == 1 && a.Wo == 1 && a.y_out != nullptr && !a.pool && p.BN > 128) {
         const int sms_ = minw_host::num_sms() > 0 ? minw_host::num_sms() : 148;
         const long long tm = (long long)p.nbx * p.nby * p.nbb;
-        const bool split = a.workspace != nullptr && !a.upd &&
-                           auto_ksplit((int)std::min<long long>(tm * p.ntn, 1 << 30), p.nk, sms_) > 1;
-        long long best = -1;
-        for (int bn = p.BN, first = bn; !split && (bn >= 128 || bn == first); bn -= 16) {
-            const long long t = tm * ((a.O + bn - 1) / bn);
-            const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
-            if (best < 0 || cost < best) {
-                best = cost;
-                p.BN = bn;
+        auto tiles = [&](int bn) { return tm * ((a.O + bn - 1) / bn); };
+        auto slices = [&](int bn) {
+            const long long t = tiles(bn);
+            return a.workspace != nullptr && !a.upd ? auto_ksplit((int)std::min<long long>(t, 1 << 30), p.nk, sms_) : 1;
+        };
+        const int full = slices(p.BN);
+        if (full > 1) {
+            const size_t sums = (size_t)full * slice_bytes((int)tiles(p.BN), p.BN);
+            if (slices(128) == full && tiles(128) * 128 <= tiles(p.BN) * p.BN && sums <= a.workspace_bytes &&
+                4 * full * tiles(128) <= 3 * sms_)
+                p.BN = 128;
+        } else {
+            long long best = -1;
+            for (int bn = p.BN, first = bn; bn >= 128 || bn == first; bn -= 16) {
+                const long long t = tiles(bn);
+                const long long cost = (t + sms_ - 1) / sms_ * ((bn / 16 + 1) / 2);
+                if (best < 0 || cost < best) {
+                    best = cost;
+                    p.BN = bn;
+                }
             }
         }
         p.ntn = (a.O + p.BN - 1) / p.BN;

@@ -201,17 +201,17 @@ def _sliced_sum(A, slices):
     return t
 
 
-def test_forward_slices(dev, M):
+@pytest.mark.parametrize("B,K,O_", [(256, 8192, 1024), (64, 8192, 450)])     # bounded by the tiles, by K
+def test_forward_slices(dev, M, B, K, O_):
     """The K slices of the step's forward product are those of its full-width
-    tiles (256 x 256 outputs a column of tiles, one slice per SM and tile), so
-    that a~ keeps the order of its fp32 sums.  W^ = 1 and whole inputs below
+    tiles (128 rows x 256 outputs, one slice per SM and tile, each of four
+    blocks of 64 or more), so that a~ keeps the order of its fp32 sums.  W^ = 1 and whole inputs below
     2^24 a slice: every slice is exact and only the additions between slices
     round, which another number of slices would show."""
-    B, K, O_ = 256, 8192, 1024
     r = np.random.default_rng(3)
     A = np.where(r.random((B, K)) < 0.5, 16384.0, 1.0 + 2.0 * r.integers(0, 64, (B, K))).astype(np.float32)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    slices = sms // ((B // 128) * (O_ // 256))
+    slices = min(sms // (-(-B // 128) * -(-O_ // 256)), K // 64 // 4)
     want = _sliced_sum(A, slices)
     assert (want != _sliced_sum(A, slices // 2)).any()
     W = torch.full((O_, K), 0.5, device=dev)
