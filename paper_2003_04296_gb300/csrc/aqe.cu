@@ -496,15 +496,20 @@ static minw_status launch_quantize(const float *x, int B, int C, int64_t HW, con
                                    cudaStream_t s) {
     const bool vec = HW % 4 == 0 && minw_host::aligned16(x) && (!y || minw_host::aligned16(y));
     // pixels per block: 32 (lanes 8 x 4 pixels) for more than 64 channels, 64 and 128 below; scalar: 32, or as
-    // many as an image of up to 16 has; four to sixteen channels in one to four groups
-    int lgl = C <= 4 ? 8 : C <= 8 ? 7 : C <= 16 ? 6 : !vec || C <= 32 ? 5 : C <= 64 ? 4 : 3;
+    // many as an image of up to 16 has; up to 16 channels in one to four groups where the blocks of one warp a group
+    // are more than two per SM, for 9 to 16 channels four (1024 pixels of 3 channels in 38 images 1.8 us, 2.0 in one
+    // group; 57 images 2.5 and 2.0; 256 of 16 channels in 228 images 2.3 and 2.7; 304 images 2.6 and 2.0)
+    const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 152;
+    int lgl = !vec || C <= 32 ? 5 : C <= 64 ? 4 : 3;
+    const int px32 = vec ? 128 : 32;
+    const int64_t blocks32 = B * ((HW + px32 - 1) / px32);
+    if (C <= 8 ? blocks32 > 2 * sms : C <= 16 && blocks32 >= 4 * sms) lgl = C <= 4 ? 8 : C <= 8 ? 7 : 6;
     if (!vec && HW <= 16)
         for (lgl = 0; (1 << lgl) < HW;) ++lgl;
     const int PX = (vec ? 4 : 1) << lgl, CG = 4 * (256 >> lgl);
     const int chunks = (int)((HW + PX - 1) / PX), cgs = (C - 1) / CG + 1;
     const int64_t total = (int64_t)B * chunks * cgs;
     // persistent: four blocks per SM, each with its next item's loads in flight behind the current one
-    const int sms = minw_host::num_sms() > 0 ? minw_host::num_sms() : 152;
     const dim3 grid((unsigned)(total < 4 * sms ? total : 4 * sms));
     typedef void (*Kernel)(const float *, int, int, int, QParams, int, int, int, int64_t, uint32_t *, uint8_t *, float,
                            float, float *, uint32_t *, int);

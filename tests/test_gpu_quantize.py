@@ -51,8 +51,11 @@ def _at_offset(x, off):
 
 SHAPES = [(1, 1, 1, 1), (2, 3, 7, 9), (3, 33, 2, 2), (2, 64, 14, 14), (1, 65, 8, 8), (2, 40, 16, 10), (1, 130, 12, 11),
           (2, 160, 6, 6), (1, 512, 14, 14), (2, 96, 33, 4),
-          # up to 16 channels in one to four groups: whole and ragged runs of 1024, 512 and 256 pixels (scalar: a quarter)
+          # up to 16 channels, few blocks of one warp a group
           (2, 4, 32, 32), (3, 3, 33, 32), (2, 7, 13, 9), (1, 8, 50, 40), (1, 12, 40, 28), (2, 16, 29, 21), (1, 1, 47, 45),
+          # and many, in one to four groups: whole and ragged runs of 1024, 512 and 256 pixels (scalar: a quarter)
+          (40, 4, 32, 32), (3, 3, 65, 63), (1, 7, 99, 101), (1, 8, 201, 200), (1, 12, 280, 281), (2, 16, 141, 141),
+          (2, 1, 161, 160), (77, 5, 16, 32), (610, 9, 4, 6), (310, 2, 5, 5),
           # images of up to 16 pixels with as few lanes, many channels
           (4, 100, 1, 1), (3, 1030, 1, 1), (2, 70, 3, 3), (33, 40, 1, 2), (1, 5, 3, 5), (2, 600, 1, 11)]
 
@@ -82,7 +85,8 @@ def test_planes_mask_forward(M, shape, bits, off):
 @pytest.mark.parametrize("bits", [1, 2, 3])
 @pytest.mark.parametrize("shape,off", [((2, 16, 5, 5), 0), ((1, 48, 4, 4), 0), ((2, 64, 14, 14), 0), ((1, 96, 9, 9), 0),
                                        ((2, 160, 8, 8), 1), ((1, 512, 7, 7), 0), ((3, 32, 12, 11), 1),
-                                       ((1, 16, 64, 44), 0), ((2, 16, 20, 20), 1), ((3, 16, 3, 3), 0), ((3, 32, 1, 1), 0),
+                                       ((1, 16, 64, 44), 0), ((2, 16, 20, 20), 1), ((1, 16, 280, 281), 0), ((2, 16, 141, 141), 0),
+                                       ((3, 16, 3, 3), 0), ((3, 32, 1, 1), 0),
                                        ((2, 1056, 1, 1), 0), ((2, 64, 1, 5), 0)])
 def test_codes(M, shape, bits, off):
     B, C, H, W = shape
